@@ -26,6 +26,13 @@ template <typename T> __host__ __device__ __forceinline__ cx<T> csub(cx<T> a, cx
 template <typename T> __host__ __device__ __forceinline__ cx<T> cmul(cx<T> a, cx<T> b) {
   return mkc<T>(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
 }
+// The same product with, in FP32, its fused operations spelled out: left to the compiler, which of
+// the two products is fused differs from kernel to kernel, and the 2D cycle's levels give the same
+// bits in the per-level kernels and in the one-cluster tail.
+template <typename T> __host__ __device__ __forceinline__ cx<T> cmul1(cx<T> a, cx<T> b) {
+  if constexpr (sizeof(T) == 4) return mkc<T>(fma(a.x, b.x, -(a.y * b.y)), fma(a.x, b.y, a.y * b.x));
+  else return cmul<T>(a, b);
+}
 // a * b + c
 template <typename T> __host__ __device__ __forceinline__ cx<T> cfma(cx<T> a, cx<T> b, cx<T> c) {
   return mkc<T>(fma(a.x, b.x, fma(-a.y, b.y, c.x)), fma(a.x, b.y, fma(a.y, b.x, c.y)));
@@ -226,6 +233,12 @@ struct helm_ctx {
   cudaStream_t alloc_stream = nullptr;  // stream of the stream-ordered allocations of helm_create
   int tail_first = 1 << 30;          // first level run by the single-block tail kernel
   FdmCoarse fdm;                     // separable coarsest solve (constant phi there), or off
+  // one-cluster tail (mg_cluster.cu): operator level and its matrix; the arguments for each level it
+  // can begin at, and the dynamic shared memory each needs (0: it cannot)
+  int ctail_op = -1;
+  void* ctail_dense = nullptr;
+  void* ctail_dev = nullptr;
+  std::vector<size_t> ctail_smem;
   int* field_bad = nullptr;          // set by helm_create when a device k field has a non-finite entry
 };
 
@@ -383,9 +396,16 @@ void krylov_free(helm_ctx* c, cudaStream_t st);
 // next grid's blocks would then sit resident at their wait while this kernel runs, and the
 // resources they hold cost more than the launch latency they hide (measured: every workload
 // slower, the 3D FP32 path by a third).  A kernel launched without the attribute passes the wait
-// at once.
+// at once.  The exceptions are the kernel before the one-cluster tail of a 2D cycle and that tail
+// itself (mg_cluster.cu): few blocks wait, or wait briefly.
 __device__ __forceinline__ void pdl_entry() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
+// Lets the next kernel's blocks be scheduled now (it still waits, in its pdl_entry, for this one's
+// completion and memory).
+__device__ __forceinline__ void pdl_trigger() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
 // process-wide switch read by launch_pdl (set per call chain by the entry points)

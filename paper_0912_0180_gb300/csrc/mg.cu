@@ -522,10 +522,10 @@ __global__ void k_jacobi9(OpView<T> op, const cx<T>* __restrict__ u, const cx<T>
   (void)l;
   cx<T> di = op.dinv[p];  // omega / D
   if (!u) {
-    un[p] = cmul<T>(f[p], di);
+    un[p] = cmul1<T>(f[p], di);
     return;
   }
-  cx<T> g = cmul<T>(csub<T>(f[p], off9<T>(op, u, i, j, p)), di);
+  cx<T> g = cmul1<T>(csub<T>(f[p], off9<T>(op, u, i, j, p)), di);
   cx<T> u0 = u[p];
   const T om1 = T(1) - omega;
   un[p] = mkc<T>(fma(om1, u0.x, g.x), fma(om1, u0.y, g.y));
@@ -1191,9 +1191,9 @@ static bool fused_applies(const helm_ctx* c, int l) {
   const helm_precond& pcf = c->pc;
   if (pcf.flags & HELM_PF_UNFUSED) return false;
   if (pcf.smoother == HELM_SM_ILU) return false;  // ILU(0) runs as its own kernels
+  if (l >= c->tail_first) return true;
   if (c->lv[l].stg64) return false;  // 9-point Galerkin levels run the per-component kernels
   if (c->lv[l].any_offset0()) return false;  // the fused tiles assume coarse c = fine 2c + 1
-  if (l >= c->tail_first) return true;
   return c->lv[l].dim == 2 && pcf.nu1 == 1 && pcf.nu2 == 1 && l < (int)c->lv.size() - 1;
 }
 
@@ -1205,7 +1205,7 @@ static void vcycle_level(helm_ctx* c, int l, const cx<T>* f, void* out, bool out
   const LevelHost& L = c->lv[l];
   int nl = (int)c->lv.size();
   if (fused_applies<T>(c, l)) {
-    if (l >= c->tail_first) {  // this level and all coarser ones in one block
+    if (l >= c->tail_first) {  // this level and all coarser ones in one launch
       tail_vcycle<T>(c, l, f, out, out_f64, skip, st);
       return;
     }

