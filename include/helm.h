@@ -215,10 +215,9 @@ typedef struct helm_ctx helm_ctx;
  * HELM_SM_ILU: the ILU(0) factors of every level above the coarsest are computed here (FP64,
  * stored in mg_dtype; the level's own stencil pattern, unknowns in natural order).  It takes 1D
  * and 2D grids whose finest level has at most 7,264 (complex64) or 3,632 (complex128) rows along
- * y (a ring of 4 values per row in one block's 227 KB of shared memory), else HELM_ERR_ARG; each
- * smoothing step runs its two triangular solves as one single-block launch over the wavefronts
- * i + 2j (their n0 + 2 n1 - 2 steps are sequential), so the V-cycle is far slower than with the
- * point smoothers. */
+ * y, else HELM_ERR_ARG.  A smoothing step's two triangular solves are one launch of one thread-block
+ * cluster, strips of 32 rows pipelined over its blocks; their n0 + 2 n1 (9-point levels) or n0 + n1
+ * (5-point) steps are sequential, so the V-cycle is slower than with the point smoothers. */
 helm_status helm_create(const helm_grid* grid, const helm_kspec* k, const helm_precond* pc,
                         void* stream, helm_ctx** out);
 

@@ -10,23 +10,33 @@
 //
 // Both the factorisation and the two triangular solves are recurrences over the rows: the row of
 // (i, j) needs rows (i-1, j-1), (i, j-1), (i+1, j-1) and (i-1, j) first (the solve with U the
-// mirror image).  Along the wavefronts t = i + 2j those rows lie on t-3, t-2, t-1 and t-1, so
-// every point of one wavefront is independent of the others: one block walks the wavefronts, a
-// thread per row (one point of each row lies on a wavefront), with a barrier between wavefronts.
-// The values of the last three wavefronts stay in a shared-memory ring indexed by row, so a point
-// reads its neighbours from shared memory.  The factors are computed once, in FP64, at create and
-// stored in the multigrid precision; a level's 9 factor entries of point p sit at [9p + s], slot
-// s = 3 (dj + 1) + (di + 1) of the neighbour (i + di, j + dj): L at the lower slots 0..3, U at 5..8,
-// and at slot 4 the reciprocal of U's pivot (both the elimination and the solve multiply by it).
+// mirror image).  The factors are computed once, in FP64, at create by one block that walks the
+// wavefronts t = i + 2j with a barrier between them, and then packed for the solve.
+//
+// The solve runs in one cluster.  A warp takes a strip of 32 rows, a lane per row, and walks the
+// columns skewed: at step t lane l is at column i = t - K l (K = 2 for the 9-point box, whose row
+// above must be one column ahead, 1 for the cross), so every neighbour in the row above is what the
+// lane above computed one to three steps ago -- a shuffle, no barrier and no shared memory.  The
+// strips form a pipeline: a strip's last row goes value by value to the block of the strip below, by
+// asynchronous stores into its shared memory that count on an mbarrier per 8 steps (no fence stalls
+// the sender), and a strip runs 72 (box) or 40 (cross) steps behind the one above.  L's strips run
+// down, U's run up in the same launch, U's entries multiplied by the pivot's reciprocal at create.
+// What bounds it: the chain of n0 + K n1 (and the pipeline's lag) dependent steps per solve, a step
+// being one shuffle and two complex multiply-adds in FP32, and in FP64 the strip's 8 to 20 DFMAs at 2
+// lanes a clock of its SM.  The factors and the right-hand side are stored in the order the lanes
+// read them ([strip][step][entry][lane]) and fetched 16 to 24 steps ahead (cp.async), since nothing
+// else runs on the SM to hide a load.  One block walking the wavefronts with a barrier each cost 1.1
+// us a wavefront in FP32; a V(0,1) cycle of MP3's operators on 640^2 unknowns went from 8.40 to 0.99
+// ms (0.36 ms of it the finest level's two solves: about 0.11 us a step).
 #include <algorithm>
 #include <type_traits>
+#include <vector>
 
-#include "helm_internal.cuh"
+#include "stencil.cuh"
 
 namespace helm {
 
-constexpr int ILU_THREADS = 1024;        // the solve: a thread per row, up to 1024
-constexpr int ILU_FACTOR_THREADS = 512;  // the factorisation (more registers a thread)
+constexpr int ILU_FACTOR_THREADS = 512;  // the factorisation
 
 // whether (i + di, j + dj) is in row (i, j)'s pattern: inside the grid and the 3 x 3 box (the
 // elimination also produces offsets of 2, fill outside every pattern), on the cross unless box
@@ -38,9 +48,10 @@ __device__ __forceinline__ bool ilu_in_pattern(int n0, int n1, bool box, int i, 
 }
 
 // The factors of one level, FP64.  stg: the Galerkin weights [9][ntot] (box pattern), else the
-// Shortley-Weller rows of op.  f64 / f32: where the factors go (either may be null).
+// Shortley-Weller rows of op.  f64: the 9 entries of point p at [9p + s], slot s = 3 (dj + 1) + (di + 1)
+// of the neighbour (i + di, j + dj): L at the lower slots 0..3, U at 5..8, the pivot's reciprocal at 4.
 __global__ void __launch_bounds__(ILU_FACTOR_THREADS) k_ilu_factor(OpView<double> op, const double2* __restrict__ stg,
-                                                            double2* __restrict__ f64, float2* __restrict__ f32) {
+                                                            double2* __restrict__ f64) {
   const int n0 = op.n[0], n1 = op.n[1];
   const long ntot = (long)n0 * n1;
   const bool box = stg != nullptr;
@@ -92,71 +103,306 @@ __global__ void __launch_bounds__(ILU_FACTOR_THREADS) k_ilu_factor(OpView<double
       }
       a[4] = crecip<double>(a[4]);
 #pragma unroll
-      for (int s = 0; s < 9; ++s) {
-        f64[9 * p + s] = a[s];
-        if (f32) f32[9 * p + s] = cconv<float, double>(a[s]);
-      }
+      for (int s = 0; s < 9; ++s) f64[9 * p + s] = a[s];
     }
     __syncthreads();
   }
 }
 
-// One ILU(0) step's solves: y = L^{-1} in (y may be in itself), then z = U^{-1} y and u += z
-// (u = z when zero: the step from u = 0, whose residual is f).  ring: [4][n1] values of the last
-// wavefronts, dynamic shared memory.
-template <typename T>
-__global__ void __launch_bounds__(ILU_THREADS) k_ilu_solve(int n0, int n1, const cx<T>* __restrict__ fac,
-                                                           const cx<T>* in, cx<T>* y, cx<T>* __restrict__ u,
-                                                           int zero, const int* skip) {
+// ---- the solve's layout -----------------------------------------------------------------------
+constexpr int ILU_CH = 8;       // steps per chunk (fetches and hand-overs)
+constexpr int ILU_MAX_WARPS = 8;
+constexpr int ILU_MAX_BLOCKS = 16;
+template <bool BOX> struct IluShape {
+  static constexpr int K = BOX ? 2 : 1;   // columns a lane lies behind the lane above
+  static constexpr int NL = BOX ? 4 : 2;  // L's entries a point
+  static constexpr int NU = BOX ? 5 : 3;  // U's, and the pivot's reciprocal first
+};
+__host__ __device__ inline int ilu_steps(int n0, bool box) {  // a strip's steps, whole chunks
+  return (n0 + 31 * (box ? 2 : 1) + ILU_CH - 1) / ILU_CH * ILU_CH;
+}
+// place of point (i, j) in a skewed vector (entry e of `per` entries a point)
+__host__ __device__ inline long ilu_at(int i, int j, int steps, int k, int per, int e) {
+  const int l = j & 31;
+  return (((long)(j >> 5) * steps + i + k * l) * per + e) * 32 + l;
+}
+
+// Packs the natural factors for the solve: lo = L's entries, up = 1 / u_pp and U's entries times it.
+template <typename T, bool BOX>
+__global__ void k_ilu_pack(const double2* __restrict__ f, int n0, int n1, int steps, cx<T>* __restrict__ lo,
+                           cx<T>* __restrict__ up) {
+  using S = IluShape<BOX>;
+  const long p = blockIdx.x * (long)blockDim.x + threadIdx.x;
+  if (p >= (long)n0 * n1) return;
+  const int i = (int)(p % n0), j = (int)(p / n0);
+  const double2* a = f + 9 * p;
+  const int sl[4] = {BOX ? 0 : 1, BOX ? 1 : 3, 2, 3}, su[4] = {5, BOX ? 6 : 7, 7, 8};
+#pragma unroll
+  for (int e = 0; e < S::NL; ++e) lo[ilu_at(i, j, steps, S::K, S::NL, e)] = cconv<T, double>(a[sl[e]]);
+  up[ilu_at(i, j, steps, S::K, S::NU, 0)] = cconv<T, double>(a[4]);
+#pragma unroll
+  for (int e = 1; e < S::NU; ++e)
+    up[ilu_at(i, j, steps, S::K, S::NU, e)] = cconv<T, double>(cmul<double>(a[4], a[su[e - 1]]));
+}
+
+// v = f - M u (or f, from the zero guess) in the skewed order of the solve.
+template <typename T, int DIM, bool BOX>
+__global__ void k_ilu_resid(OpView<T> op, const cx<T>* __restrict__ u, const cx<T>* __restrict__ f, int steps,
+                            cx<T>* __restrict__ v, const int* skip) {
   pdl_entry();
   if (skip && *skip) return;
-  extern __shared__ __align__(16) unsigned char ilu_ring[];
-  cx<T>* ring = reinterpret_cast<cx<T>*>(ilu_ring);
-  const int waves = n0 + 2 * (n1 - 1);
-  for (int t = 0; t < waves; ++t) {
-    for (int j = threadIdx.x; j < n1; j += blockDim.x) {
-      const int i = t - 2 * j;
-      if (i < 0 || i >= n0) continue;
-      const long p = i + (long)n0 * j;
-      const cx<T>* w = fac + 9 * p;
-      cx<T> v = in[p];
-      if (j > 0) {
-        if (i > 0) v = csub<T>(v, cmul<T>(w[0], ring[((t - 3) & 3) * n1 + j - 1]));
-        v = csub<T>(v, cmul<T>(w[1], ring[((t - 2) & 3) * n1 + j - 1]));
-        if (i < n0 - 1) v = csub<T>(v, cmul<T>(w[2], ring[((t - 1) & 3) * n1 + j - 1]));
+  const int i = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y * blockDim.y + threadIdx.y;
+  if (i >= op.n[0] || j >= op.n[1]) return;
+  const long p = i + (long)op.n[0] * j;
+  cx<T> r = f[p];
+  if (u) {
+    if constexpr (BOX) {
+      cx<T> acc = mkc<T>(T(0), T(0));
+#pragma unroll
+      for (int s = 0; s < 9; ++s) {
+        const int ii = i + s % 3 - 1, jj = j + s / 3 - 1;
+        if (s == 4 || ii < 0 || ii >= op.n[0] || jj < 0 || jj >= op.n[1]) continue;
+        acc = cfma<T>(op.stg[(long)s * op.ntot + p], u[ii + (long)jj * op.n[0]], acc);
       }
-      if (i > 0) v = csub<T>(v, cmul<T>(w[3], ring[((t - 1) & 3) * n1 + j]));
-      ring[(t & 3) * n1 + j] = v;
-      y[p] = v;
+      r = csub<T>(r, cfma<T>(op.stg[4 * op.ntot + p], u[p], acc));
+    } else {
+      r = csub<T>(r, op_row<T, T, DIM>(op, u, i, j, 0, p));
     }
-    __syncthreads();
   }
-  for (int t = waves - 1; t >= 0; --t) {
-    for (int j = threadIdx.x; j < n1; j += blockDim.x) {
-      const int i = t - 2 * j;
-      if (i < 0 || i >= n0) continue;
-      const long p = i + (long)n0 * j;
-      const cx<T>* w = fac + 9 * p;
-      cx<T> v = y[p];
-      if (i < n0 - 1) v = csub<T>(v, cmul<T>(w[5], ring[((t + 1) & 3) * n1 + j]));
-      if (j < n1 - 1) {
-        if (i > 0) v = csub<T>(v, cmul<T>(w[6], ring[((t + 1) & 3) * n1 + j + 1]));
-        v = csub<T>(v, cmul<T>(w[7], ring[((t + 2) & 3) * n1 + j + 1]));
-        if (i < n0 - 1) v = csub<T>(v, cmul<T>(w[8], ring[((t + 3) & 3) * n1 + j + 1]));
-      }
-      v = cmul<T>(v, w[4]);  // w[4]: 1 / the pivot
-      ring[(t & 3) * n1 + j] = v;
-      u[p] = zero ? v : cadd<T>(u[p], v);
-    }
-    __syncthreads();
-  }
+  v[ilu_at(i, j, steps, IluShape<BOX>::K, 1, 0)] = r;
 }
 
-static int ilu_threads(int n1) { return std::min(ILU_THREADS, (n1 + 31) / 32 * 32); }
+// u += z (u = z from the zero guess), z skewed; wide: u also as complex128.
+template <typename T, bool BOX>
+__global__ void k_ilu_add(int n0, int n1, int steps, const cx<T>* __restrict__ z, cx<T>* __restrict__ u, int zero,
+                          double2* __restrict__ wide, const int* skip) {
+  pdl_entry();
+  if (skip && *skip) return;
+  const int i = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y * blockDim.y + threadIdx.y;
+  if (i >= n0 || j >= n1) return;
+  const long p = i + (long)n0 * j;
+  const cx<T> d = z[ilu_at(i, j, steps, IluShape<BOX>::K, 1, 0)];
+  const cx<T> r = zero ? d : cadd<T>(u[p], d);
+  u[p] = r;
+  if (wide) wide[p] = cconv<double, T>(r);
+}
+
+template <typename T> struct IluArgs {
+  int n0, n1, steps;
+  int s0, s1;    // strips of this launch, one after another over its blocks' warps
+  int passes;    // bit 0: L, bit 1: U
+  int depth;     // chunks of the fetch ring
+  int rows;      // whether the strips hand their edge row over in shared memory
+  const cx<T>*lo, *up;
+  cx<T>* v;      // right-hand side, y and z in turn
+};
+
+// ---- the hand-over ---------------------------------------------------------------------------
+__device__ __forceinline__ unsigned ilu_smem(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ unsigned ilu_map(unsigned a, unsigned rank) {
+  unsigned r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ void ilu_send(unsigned to, unsigned bar, float2 v) {
+  const unsigned long long b = ((unsigned long long)__float_as_uint(v.y) << 32) | __float_as_uint(v.x);
+  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.b64 [%0], %1, [%2];" ::"r"(to), "l"(b), "r"(bar)
+               : "memory");
+}
+__device__ __forceinline__ void ilu_send(unsigned to, unsigned bar, double2 v) {
+  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v2.b64 [%0], {%1, %2}, [%3];" ::"r"(to),
+               "l"(__double_as_longlong(v.x)), "l"(__double_as_longlong(v.y)), "r"(bar)
+               : "memory");
+}
+__device__ __forceinline__ void ilu_expect(unsigned bar, unsigned bytes) {
+  asm volatile("{\n .reg .b64 t;\n mbarrier.arrive.expect_tx.shared::cta.b64 t, [%0], %1;\n}" ::"r"(bar), "r"(bytes) : "memory");
+}
+// waits for the barrier's first phase, for about a second at most; false when that runs out
+__device__ __forceinline__ bool ilu_wait(unsigned bar) {
+  const long long t0 = clock64();
+  for (int tries = 0; tries < (1 << 24); ++tries) {
+    unsigned ok;
+    asm volatile(
+        "{\n .reg .pred p;\n mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
+        : "=r"(ok)
+        : "r"(bar), "r"(0u)
+        : "memory");
+    if (ok) return true;
+    if (clock64() - t0 > (1LL << 31)) break;
+  }
+  return false;
+}
+__device__ __forceinline__ void ilu_fetch(float2* dst, const float2* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(ilu_smem(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void ilu_fetch(double2* dst, const double2* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(ilu_smem(dst)), "l"(src) : "memory");
+}
+template <int N> __device__ __forceinline__ void ilu_landed() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+
+// valid columns of the edge row among a chunk's steps [m CH, m CH + CH): the edge lane is `lag` columns
+// behind the step
+__device__ __forceinline__ int ilu_sent(int m, int lag, int n0) {
+  const int lo = max(m * ILU_CH - lag, 0), hi = min(m * ILU_CH + ILU_CH - lag, n0);
+  return max(hi - lo, 0);
+}
 
 template <typename T>
-static size_t ilu_smem(int n1) {
-  return sizeof(cx<T>) * 4 * (size_t)n1;
+__device__ __forceinline__ cx<T> ilu_shfl(cx<T> v, int lane) {
+  return mkc<T>(__shfl_sync(0xffffffffu, v.x, lane), __shfl_sync(0xffffffffu, v.y, lane));
+}
+
+// One strip's solve with L (UP = false: chunks and rows ascending) or U (UP = true: both descending).
+// ring: this warp's fetch ring; row, bars: the edge row it receives and the barriers of its chunks;
+// to_row, to_bar: the same in the receiving strip (0: nobody); edge: where the edge row comes from (0
+// nowhere, 1 the row in shared memory, 2 the other strip's values in v).
+template <typename T, bool BOX, bool UP, int DEPTH>
+__device__ __forceinline__ void ilu_strip(const IluArgs<T>& g, int strip, cx<T>* ring, const cx<T>* row, unsigned bars,
+                                          unsigned to_row, unsigned to_bar, int edge) {
+  using S = IluShape<BOX>;
+  constexpr int K = S::K, NE = UP ? S::NU : S::NL, SL = NE + 1, CH = ILU_CH;
+  // lane 0 (31) takes the edge row, lane 31 (0) gives it; new value per step: one column ahead (box)
+  constexpr int TAKE = UP ? 31 : 0, GIVE = UP ? 0 : 31, LAG = UP ? 0 : 31 * K, AHEAD = BOX ? 1 : 0;
+  const int lane = threadIdx.x & 31;
+  const int n0 = g.n0, steps = g.steps, nc = steps / CH;
+  const bool has_row = strip * 32 + lane < g.n1;
+  const cx<T> zero = mkc<T>(T(0), T(0));
+  cx<T>* const v = g.v + (long)strip * steps * 32 + lane;
+  const cx<T>* const fac = (UP ? g.up : g.lo) + (long)strip * steps * NE * 32 + lane;
+  const cx<T>* const other = g.v + (long)(UP ? strip + 1 : strip - 1) * steps * 32 + GIVE;
+  bool failed = false;
+  int armed = 0;  // chunks of the edge row waited for
+  auto chunk = [&](int c) { return UP ? nc - 1 - c : c; };  // c-th chunk in this direction
+  auto fetch = [&](int c) {
+    if (c < nc) {
+      cx<T>* const to = ring + (c % DEPTH) * CH * SL * 32 + lane;
+      const long t0 = (long)chunk(c) * CH;
+#pragma unroll
+      for (int k = 0; k < CH; ++k) {
+#pragma unroll
+        for (int e = 0; e < NE; ++e) ilu_fetch(to + (k * SL + e) * 32, fac + ((t0 + k) * NE + e) * 32);
+        ilu_fetch(to + (k * SL + NE) * 32, v + (t0 + k) * 32);
+      }
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  // column that the take lane's new value has at step t; its chunk is the giving lane's
+  auto col_new = [&](int t) { return UP ? t - 31 * K - AHEAD : t + AHEAD; };
+  auto ready = [&](int c) {  // the edge values of this direction's chunk c, and the column before
+    if (edge != 1) return;
+    // giving lane's chunk of the last column needed, in this direction's count: UP gives column t at
+    // its step t, else column t - 31 K
+    const int need = min(c + (BOX ? 8 : 4), nc - 1);
+    while (armed <= need) {
+      const int m = chunk(armed), n = ilu_sent(m, LAG, n0);
+      if (n) {
+        const unsigned b = bars + m * 8;
+        if (lane == 0) ilu_expect(b, n * (unsigned)sizeof(cx<T>));
+        __syncwarp();
+        if (!failed) failed = !ilu_wait(b);
+      }
+      ++armed;
+    }
+    failed = __any_sync(0xffffffffu, failed);
+  };
+  auto edge_at = [&](int col) -> cx<T> {
+    if (edge == 0 || col < 0 || col >= n0) return zero;
+    return edge == 1 ? row[col] : __ldcg(other + (long)(col + LAG) * 32);
+  };
+#pragma unroll
+  for (int c = 0; c < DEPTH - 1; ++c) fetch(c);
+  ready(0);
+  // neighbours in the row above (below): a and b one and two columns behind the new value c (box)
+  cx<T> a = zero, b = zero, prev = zero;
+  if (BOX && lane == TAKE) b = edge_at(col_new(UP ? steps : -1));
+  for (int c = 0; c < nc; ++c) {
+    fetch(c + DEPTH - 1);
+    ready(c);
+    const int m = chunk(c);
+    // lane k holds the take lane's new value of the chunk's k-th step
+    const cx<T> en = lane < CH ? edge_at(col_new(UP ? m * CH + CH - 1 - lane : m * CH + lane)) : zero;
+    ilu_landed<DEPTH - 1>();
+    const cx<T>* const at = ring + (c % DEPTH) * CH * SL * 32 + lane;
+#pragma unroll
+    for (int k = 0; k < CH; ++k) {
+      const int kk = UP ? CH - 1 - k : k, t = m * CH + kk, i = t - K * lane;
+      const cx<T>* const q = at + kk * SL * 32;
+      const cx<T> x = q[NE * 32];
+      // the lane above's (below's) last value
+      cx<T> nw = UP ? mkc<T>(__shfl_down_sync(0xffffffffu, prev.x, 1), __shfl_down_sync(0xffffffffu, prev.y, 1))
+                    : mkc<T>(__shfl_up_sync(0xffffffffu, prev.x, 1), __shfl_up_sync(0xffffffffu, prev.y, 1));
+      const cx<T> ek = ilu_shfl<T>(en, k);
+      if (lane == TAKE) nw = ek;
+      cx<T> r;
+      if (UP) {
+        r = cmul<T>(q[0], x);
+        if (BOX) r = cfms<T>(q[4 * 32], a, cfms<T>(q[3 * 32], b, r));  // (i+1, j+1), (i, j+1)
+        r = cfms<T>(q[32], prev, r);                                   // (i+1, j)
+        r = cfms<T>(q[2 * 32], nw, r);                                 // (i-1, j+1); cross (i, j+1)
+      } else {
+        r = x;
+        if (BOX) r = cfms<T>(q[32], b, cfms<T>(q[0], a, r));           // (i-1, j-1), (i, j-1)
+        r = cfms<T>(q[(BOX ? 3 : 1) * 32], prev, r);                   // (i-1, j)
+        r = cfms<T>(q[(BOX ? 2 : 0) * 32], nw, r);                     // (i+1, j-1); cross (i, j-1)
+      }
+      if (failed) r = mkc<T>(T(NAN), T(NAN));  // the wait ran out: the solve ends with a NaN status
+      const bool in = has_row && i >= 0 && i < n0;
+      if (!in) r = zero;  // a point outside the grid is zero for the neighbours
+      else v[(long)t * 32] = r;
+      if (lane == GIVE && to_row && in) ilu_send(to_row + (unsigned)(i * sizeof(cx<T>)), to_bar + (t / CH) * 8, r);
+      a = b;
+      b = nw;
+      prev = r;
+    }
+  }
+  ilu_landed<0>();
+}
+
+template <typename T, bool BOX, int DEPTH>
+__global__ void k_ilu_solve(const IluArgs<T> g, const int* skip) {
+  pdl_entry();
+  if (skip && *skip) return;
+  using S = IluShape<BOX>;
+  extern __shared__ __align__(16) unsigned char ilu_sm[];
+  constexpr int RING = DEPTH * ILU_CH * (S::NU + 1) * 32;
+  const int wpc = blockDim.x >> 5, w = threadIdx.x >> 5, lane = threadIdx.x & 31, nc = g.steps / ILU_CH;
+  cx<T>* const ring = reinterpret_cast<cx<T>*>(ilu_sm) + w * RING;
+  cx<T>* const rows0 = reinterpret_cast<cx<T>*>(ilu_sm) + wpc * RING;
+  const int row_n = g.rows ? g.n0 : 0;
+  cx<T>* const row = rows0 + w * row_n;
+  const unsigned bars0 = ilu_smem(rows0 + wpc * row_n), rowb0 = ilu_smem(rows0);
+  const int strip = g.s0 + (int)blockIdx.x * wpc + w;
+  if (g.rows) {
+    for (int m = lane; m < 2 * nc; m += 32)  // L's hand-overs, then U's
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bars0 + (2 * w * nc + m) * 8) : "memory");
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+  }
+  if (strip >= g.s1) return;  // nothing is sent to it
+  auto row_of = [&](int st) {  // the edge row and barriers of strip st (0: not in this launch)
+    const int q = st - g.s0, blk = q / wpc, ww = q % wpc;
+    struct P { unsigned row, bar; } r{0u, 0u};
+    if (g.rows && st >= g.s0 && st < g.s1) {
+      r.row = ilu_map(rowb0 + (unsigned)(ww * row_n * sizeof(cx<T>)), blk);
+      r.bar = ilu_map(bars0 + (unsigned)(2 * ww * nc * 8), blk);
+    }
+    return r;
+  };
+  const unsigned bars = bars0 + 2 * w * nc * 8;
+  const int strips = (g.n1 + 31) / 32;
+  if (g.passes & 1) {
+    const auto to = row_of(strip + 1);
+    const int edge = strip == 0 ? 0 : strip > g.s0 ? 1 : 2;
+    ilu_strip<T, BOX, false, DEPTH>(g, strip, ring, row, bars, to.row, to.bar, edge);
+    __threadfence();  // the values of this pass are fetched asynchronously in the next
+    __syncwarp();
+  }
+  if (g.passes & 2) {
+    const auto to = row_of(strip - 1);
+    const int edge = strip == strips - 1 ? 0 : strip < g.s1 - 1 ? 1 : 2;
+    ilu_strip<T, BOX, true, DEPTH>(g, strip, ring, row, bars + nc * 8, to.row, to.bar ? to.bar + nc * 8 : 0u, edge);
+  }
 }
 
 helm_status ilu_check(int dim, const int n[3], bool f32) {
@@ -164,37 +410,146 @@ helm_status ilu_check(int dim, const int n[3], bool f32) {
     set_error("ILU(0) smoothing runs on 1D and 2D levels");
     return HELM_ERR_ARG;
   }
-  const size_t smem = f32 ? ilu_smem<float>(n[1]) : ilu_smem<double>(n[1]);
-  if (smem > ILU_SMEM_MAX) {
-    set_error("ILU(0) smoothing keeps 4 values per row in shared memory: at most " +
-              std::to_string(ILU_SMEM_MAX / (4 * (f32 ? 8 : 16))) + " rows in this precision");
+  const int most = (int)(ILU_ROW_BYTES / (4 * (f32 ? sizeof(float2) : sizeof(double2))));
+  if (n[1] > most) {
+    set_error("ILU(0) smoothing takes at most " + std::to_string(most) + " rows in this precision");
     return HELM_ERR_ARG;
   }
   return HELM_OK;
 }
 
-helm_status ilu_build(helm_ctx* c, LevelHost& L, bool f32, cudaStream_t st) {
+namespace {
+
+constexpr size_t ILU_SMEM_MAX = 224 * 1024;
+
+// The launches of one level: warps per block, blocks per cluster, ring depth, shared memory.
+struct IluPlan {
+  int wpc, blocks, depth, rows;
+  size_t smem;
+};
+// The fewest warps a block (a strip has its SM's loads and, in FP64, its FP64 pipe to itself) that put
+// all strips into one cluster; where the edge rows do not fit, fewer strips a launch; a row too long
+// for shared memory is handed over in memory, one strip a launch.
+IluPlan ilu_plan(int n0, int n1, bool box, size_t esz) {
+  const int strips = (n1 + 31) / 32, nc = ilu_steps(n0, box) / ILU_CH;
+  auto bytes = [&](int wpc, int depth, int rows) {
+    return wpc * (esz * depth * ILU_CH * ((box ? 5 : 3) + 1) * 32 + (rows ? esz * n0 + 16 * (size_t)nc : 0));
+  };
+  IluPlan p{1, 1, 3, 0, 0};
+  if (strips > 1) {
+    for (int wpc = std::min((strips + ILU_MAX_BLOCKS - 1) / ILU_MAX_BLOCKS, ILU_MAX_WARPS); wpc >= 1 && !p.rows; --wpc)
+      for (int depth = 3; depth >= 2 && !p.rows; --depth)
+        if (bytes(wpc, depth, 1) <= ILU_SMEM_MAX) p = IluPlan{wpc, 1, depth, 1, 0};
+    if (p.rows)
+      while (p.blocks < ILU_MAX_BLOCKS && p.blocks * p.wpc < strips) p.blocks *= 2;
+  }
+  p.smem = bytes(p.wpc, p.depth, p.rows);
+  return p;
+}
+
+template <typename T, bool BOX>
+cudaError_t ilu_attrs() {
+  cudaError_t e = cudaSuccess;
+  auto one = [&](auto kern) {
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ILU_SMEM_MAX);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  };
+  one(k_ilu_solve<T, BOX, 2>);
+  one(k_ilu_solve<T, BOX, 3>);
+  return e;
+}
+
+template <typename T, bool BOX>
+void ilu_launch(const IluPlan& p, const IluArgs<T>& g, const int* skip, cudaStream_t st) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(p.blocks);
+  cfg.blockDim = dim3(32 * p.wpc);
+  cfg.dynamicSmemBytes = p.smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at[2];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = p.blocks;
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = g_use_pdl ? 2 : 1;
+  if (p.depth == 3) cudaLaunchKernelEx(&cfg, k_ilu_solve<T, BOX, 3>, g, skip);
+  else cudaLaunchKernelEx(&cfg, k_ilu_solve<T, BOX, 2>, g, skip);
+}
+
+template <typename T, bool BOX>
+helm_status ilu_pack(helm_ctx* c, LevelHost& L, const double2* fac, cudaStream_t st) {
+  using S = IluShape<BOX>;
+  const int steps = ilu_steps(L.n[0], BOX), strips = (L.n[1] + 31) / 32;
+  const size_t pts = (size_t)strips * steps * 32;
   helm_status rc;
-  if ((rc = ctx_alloc(c, (void**)&L.ilu64, sizeof(double2) * 9 * L.ntot)) != HELM_OK) return rc;
-  if (f32 && (rc = ctx_alloc(c, (void**)&L.ilu32, sizeof(float2) * 9 * L.ntot)) != HELM_OK) return rc;
-  k_ilu_factor<<<1, std::min(ILU_FACTOR_THREADS, ilu_threads(L.n[1])), 0, st>>>(L.view<double>(), L.stg64, L.ilu64, f32 ? L.ilu32 : nullptr);
+  if ((rc = ctx_alloc(c, &L.ilu_lo, sizeof(cx<T>) * S::NL * pts)) != HELM_OK) return rc;
+  if ((rc = ctx_alloc(c, &L.ilu_up, sizeof(cx<T>) * S::NU * pts)) != HELM_OK) return rc;
+  if ((rc = ctx_alloc(c, &L.ilu_v, sizeof(cx<T>) * pts)) != HELM_OK) return rc;
+  // the places outside the grid stay zero
+  HELM_CUDA(cudaMemsetAsync(L.ilu_lo, 0, sizeof(cx<T>) * S::NL * pts, st));
+  HELM_CUDA(cudaMemsetAsync(L.ilu_up, 0, sizeof(cx<T>) * S::NU * pts, st));
+  HELM_CUDA(cudaMemsetAsync(L.ilu_v, 0, sizeof(cx<T>) * pts, st));
+  k_ilu_pack<T, BOX><<<(int)((L.ntot + 255) / 256), 256, 0, st>>>(fac, L.n[0], L.n[1], steps, (cx<T>*)L.ilu_lo,
+                                                                (cx<T>*)L.ilu_up);
   HELM_CUDA(cudaGetLastError());
-  // the solve's ring may exceed the default 48 KB: raise the block's limit here, outside any
-  // stream capture
-  if (f32) HELM_CUDA(cudaFuncSetAttribute(k_ilu_solve<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ILU_SMEM_MAX));
-  else HELM_CUDA(cudaFuncSetAttribute(k_ilu_solve<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ILU_SMEM_MAX));
-  return HELM_OK;
+  // (attributes are set here, outside any stream capture)
+  return cuda_err(ilu_attrs<T, BOX>());
+}
+
+template <typename T, bool BOX>
+void ilu_smooth_t(const LevelHost& L, const cx<T>* f, cx<T>* u, bool zero, double2* wide, const int* skip, cudaStream_t st) {
+  const int n0 = L.n[0], n1 = L.n[1], steps = ilu_steps(n0, BOX), strips = (n1 + 31) / 32;
+  cx<T>* const v = (cx<T>*)L.ilu_v;
+  const dim3 b(32, 8), gr((n0 + 31) / 32, (n1 + 7) / 8);
+  const cx<T>* u0 = zero ? nullptr : u;
+  if (L.dim == 1) launch_pdl(k_ilu_resid<T, 1, BOX>, gr, b, 0, st, L.view<T>(), u0, f, steps, v, skip);
+  else launch_pdl(k_ilu_resid<T, 2, BOX>, gr, b, 0, st, L.view<T>(), u0, f, steps, v, skip);
+  const IluPlan p = ilu_plan(n0, n1, BOX, sizeof(cx<T>));
+  const int per = p.wpc * p.blocks;
+  IluArgs<T> g{n0, n1, steps, 0, strips, 3, p.depth, p.rows, (const cx<T>*)L.ilu_lo, (const cx<T>*)L.ilu_up, v};
+  if (strips <= per) {
+    ilu_launch<T, BOX>(p, g, skip, st);
+  } else {  // groups of strips: L down, then U up
+    const int groups = (strips + per - 1) / per;
+    for (int q = 0; q < 2 * groups; ++q) {
+      const int grp = q < groups ? q : 2 * groups - 1 - q;
+      g.s0 = grp * per;
+      g.s1 = std::min(g.s0 + per, strips);
+      g.passes = q < groups ? 1 : 2;
+      ilu_launch<T, BOX>(p, g, skip, st);
+    }
+  }
+  launch_pdl(k_ilu_add<T, BOX>, gr, b, 0, st, n0, n1, steps, (const cx<T>*)v, u, zero ? 1 : 0, wide, skip);
+}
+
+}  // namespace
+
+helm_status ilu_build(helm_ctx* c, LevelHost& L, bool f32, cudaStream_t st) {
+  void* fac = nullptr;  // the natural factors, FP64, until they are packed
+  std::vector<DevBlock> tmp(1);
+  helm_status rc = dev_alloc(&fac, sizeof(double2) * 9 * L.ntot, st, &tmp[0]);
+  if (rc != HELM_OK) return rc;
+  k_ilu_factor<<<1, std::min(ILU_FACTOR_THREADS, (L.n[1] + 31) / 32 * 32), 0, st>>>(L.view<double>(), L.stg64,
+                                                                                  (double2*)fac);
+  rc = cuda_err(cudaGetLastError());
+  const bool box = L.stg64 != nullptr;
+  if (rc == HELM_OK) {
+    if (f32) rc = box ? ilu_pack<float, true>(c, L, (double2*)fac, st) : ilu_pack<float, false>(c, L, (double2*)fac, st);
+    else rc = box ? ilu_pack<double, true>(c, L, (double2*)fac, st) : ilu_pack<double, false>(c, L, (double2*)fac, st);
+  }
+  dev_free_all(tmp, st);
+  return rc;
 }
 
 template <typename T>
-void ilu_solve(const LevelHost& L, const cx<T>* in, cx<T>* y, cx<T>* u, bool zero, const int* skip, cudaStream_t st) {
-  const cx<T>* fac = std::is_same<T, double>::value ? (const cx<T>*)(const void*)L.ilu64 : (const cx<T>*)(const void*)L.ilu32;
-  const int n1 = L.n[1];
-  launch_pdl(k_ilu_solve<T>, dim3(1), dim3(ilu_threads(n1)), ilu_smem<T>(n1), st, L.n[0], n1, fac, in, y, u,
-             zero ? 1 : 0, skip);
+void ilu_smooth(const LevelHost& L, const cx<T>* f, cx<T>* u, bool zero, double2* wide, const int* skip, cudaStream_t st) {
+  if (L.stg64) ilu_smooth_t<T, true>(L, f, u, zero, wide, skip, st);
+  else ilu_smooth_t<T, false>(L, f, u, zero, wide, skip, st);
 }
 
-template void ilu_solve<float>(const LevelHost&, const float2*, float2*, float2*, bool, const int*, cudaStream_t);
-template void ilu_solve<double>(const LevelHost&, const double2*, double2*, double2*, bool, const int*, cudaStream_t);
+template void ilu_smooth<float>(const LevelHost&, const float2*, float2*, bool, double2*, const int*, cudaStream_t);
+template void ilu_smooth<double>(const LevelHost&, const double2*, double2*, bool, double2*, const int*, cudaStream_t);
 
 }  // namespace helm

@@ -1167,18 +1167,7 @@ static void smooth(helm_ctx* c, const LevelHost& L, cx<T>* b[2], int* cur, const
       op.jacobi(z0 ? nullptr : b[*cur], f, b[1 - *cur], (T)c->pc.omega, skip, st, w);
       *cur = 1 - *cur;
     } else if (c->pc.smoother == HELM_SM_ILU) {
-      // u += (L U)^{-1} (f - M u), the residual in the spare buffer; from u = 0 the residual is f
-      cx<T>* u = b[*cur];
-      cx<T>* r = b[1 - *cur];
-      if (z0) {
-        ilu_solve<T>(L, f, r, u, true, skip, st);
-      } else {
-        op.apply(u, f, r, skip, st);
-        ilu_solve<T>(L, r, r, u, false, skip, st);
-      }
-      if constexpr (sizeof(cx<T>) == 8) {
-        if (w) widen_c64(c, (const float2*)u, w, L.ntot, skip, st);
-      }
+      ilu_smooth<T>(L, f, b[*cur], z0, w, skip, st);
     } else {
       op.rbgs(b[*cur], f, 0, z0 ? 1 : 0, skip, st);
       op.rbgs(b[*cur], f, 1, 0, skip, st, w);
@@ -1314,7 +1303,7 @@ static helm_status level_op_t(helm_ctx* c, int op, int lvl, void* a, const void*
     case HELM_OP_SMOOTH:
     case HELM_OP_SMOOTH0: {
       if (!A || !B || count < 0) return HELM_ERR_ARG;
-      if (c->pc.smoother == HELM_SM_ILU && !L.ilu64) {
+      if (c->pc.smoother == HELM_SM_ILU && !L.ilu_lo) {
         set_error("the coarsest level is solved directly and has no ILU(0) factors");
         return HELM_ERR_ARG;
       }

@@ -64,7 +64,7 @@ extern "C" size_t helm_estimate_bytes(const helm_grid* g, const helm_precond* pc
   if (pcon) {
     long m[3] = {n[0], n[1], n[2]};
     long Nl = N;
-    int levels = 0;
+    int levels = 0, tail = 0;
     long last = N;
     for (;;) {
       ++levels;
@@ -72,8 +72,10 @@ extern "C" size_t helm_estimate_bytes(const helm_grid* g, const helm_precond* pc
       bytes += (size_t)Nl * (8 + 4 + 2 * esz + (levels == 1 ? 1 : 3) * esz);
       if (levels > 1 && (pc->flags & HELM_PF_GALERKIN))  // the stencil, FP64 and the V-cycle precision
         bytes += (size_t)Nl * (g->dim == 3 ? 27 : 9) * (16 + (esz == 8 ? 8 : 0)) + (size_t)Nl * 8;
-      if (pc->smoother == HELM_SM_ILU)  // ILU(0) factors, FP64 and the V-cycle precision
-        bytes += (size_t)Nl * 9 * (16 + (esz == 8 ? 8 : 0));
+      if (pc->smoother == HELM_SM_ILU)  // ILU(0) factors, FP64 (transient) and skewed with the solves' vector
+        bytes += (size_t)Nl * 9 * 16 + (size_t)((m[1] + 31) / 32) * 32 * (size_t)(m[0] + 70) * 10 * esz;
+      if (g->dim == 2 && pc->nu1 == 1 && pc->nu2 == 1 && Nl <= (esz == 8 ? 600 : 150) && tail++ == 0)
+        bytes += (size_t)(Nl + 1) * Nl * esz + 64 * 1024;  // the one-cluster tail's dense operator
       last = Nl;
       bool all_small = true;
       long min_n = 1L << 40;

@@ -43,3 +43,31 @@ def test_cluster_tail_vcycle(shape, sm, galerkin, mg):
     z = zs[0].cpu().numpy()
     assert np.linalg.norm(z - ref) <= tol * np.linalg.norm(ref)
     assert np.max(np.abs(z - ref)) <= tol * np.max(np.abs(ref))
+
+
+@pytest.mark.parametrize("shape,mg", [((5, 3), "c128"), ((9, 40), "c64"), ((33, 65), "c128"), ((640, 70), "c64"), ((70, 600), "c64"),
+                                      ((70, 3200), "c128"), ((70, 4200), "c64"), ((30000, 70), "c64")])
+@pytest.mark.parametrize("galerkin", [False, True])
+def test_ilu_strips(shape, mg, galerkin):
+    """The ILU(0) step's triangular solves in strips of 32 rows handed from block to block: one strip,
+    a last strip of few rows, several warps a block, more strips than one cluster holds, rows too long
+    for shared memory; on the finest level (5-point) and, Galerkin, the next one (9-point)."""
+    import paper_0912_0180_gb300._lib as L
+    from paper_0912_0180_gb300.helm import Helm
+    p = hi.make_problem(2, (shape[0] + 2, shape[1] + 2), 0, extent=((shape[0] + 1) / 32, (shape[1] + 1) / 32), k0=6.0,
+                        phi_kind="bump", rhs="zero", bump_centre=(0.4, 0.6))
+    pc = hi.Precond(kind=hi.PC_CSG_UNIFORM, theta_beta=0.4, smoother=hi.SM_ILU, galerkin=galerkin, nu1=0, nu2=1, coarse_max=2)
+    o = Oracle(p, pc)
+    h = Helm(p, pc, mg_dtype=mg)
+    dt = torch.complex128 if mg == "c128" else torch.complex64
+    tol = 1e-10 if mg == "c128" else 5e-5
+    lvl = 1 if galerkin and o.nlev > 2 else 0
+    n = o.level_size(1, lvl)
+    a, b = hi.random_vector(n, 5).astype(np.complex64), hi.random_vector(n, 6).astype(np.complex64)
+    for op, start in ((L.HELM_OP_SMOOTH, a), (L.HELM_OP_SMOOTH0, 0 * a)):
+        u = torch.from_numpy(start).cuda().to(dt)
+        h.level_op(op, lvl, u, torch.from_numpy(b).cuda().to(dt), None, count=1)
+        ref = o.smooth(lvl, start.astype(np.complex128), b.astype(np.complex128), 1)
+        d = u.cpu().numpy() - ref
+        assert np.linalg.norm(d) <= tol * np.linalg.norm(ref) and np.max(np.abs(d)) <= tol * np.max(np.abs(ref))
+    h.close()
