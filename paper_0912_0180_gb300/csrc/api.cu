@@ -326,9 +326,7 @@ helm_status helm_vcycle(helm_ctx* c, const helm_precond* pc, helm_dtype dtype, c
   }
   if (f32) {
     float2* in = (float2*)c->scratch + c->n;  // not the first half: the unfused cycle's output goes there
-    helm_status s = mg_input_from_c128(c, (const double2*)r, in, st);
-    if (s != HELM_OK) return s;
-    return mg_vcycle<float>(c, in, z, z64, nullptr, st);
+    return mg_vcycle_from_c128(c, (const double2*)r, in, z, z64, st);
   }
   if (!z64) { set_error("helm_vcycle: an FP64 hierarchy gives complex128 output"); return HELM_ERR_ARG; }
   return mg_vcycle<double>(c, (const double2*)r, z, false, nullptr, st);

@@ -287,6 +287,9 @@ helm_status build_hierarchy(helm_ctx* c, cudaStream_t st);
 // kernel that writes it -- the precision boundary into the FP64 Krylov vectors)
 template <typename T>
 helm_status mg_vcycle(helm_ctx* c, const cx<T>* f0, void* u0, bool u0_f64, const int* skip, cudaStream_t st);
+// the V-cycle of an FP32 hierarchy with a complex128 right-hand side: narrowed by the first kernel
+// where that is a fused one of the finest level, else by a conversion into `buf` (N complex64)
+helm_status mg_vcycle_from_c128(helm_ctx* c, const double2* r, void* buf, void* z, bool z64, cudaStream_t st);
 helm_status mg_level_op(helm_ctx* c, int op, int lvl, void* a, const void* b, void* out, int count,
                         cudaStream_t st);
 // y = H x (FP64 arithmetic); x of type TX; optional fused partial inner products handled in krylov.cu
@@ -369,10 +372,10 @@ template <typename T> int tail_first_level(const helm_ctx* c);
 template <typename T>
 helm_status tail_vcycle(helm_ctx* c, int first, const cx<T>* f, void* out, bool out_f64, const int* skip,
                         cudaStream_t st);
-template <typename T>
-void fused_down2d(const helm_ctx* c, int l, const cx<T>* f, cx<T>* u_out, cx<T>* fc, const int* skip, cudaStream_t st);
-template <typename T>
-void fused_up2d(const helm_ctx* c, int l, const cx<T>* u_in, const cx<T>* ec, const cx<T>* f, void* out,
+template <typename T, typename TI>
+void fused_down2d(const helm_ctx* c, int l, const cx<TI>* f, cx<T>* u_out, cx<T>* fc, const int* skip, cudaStream_t st);
+template <typename T, typename TI>
+void fused_up2d(const helm_ctx* c, int l, const cx<T>* u_in, const cx<T>* ec, const cx<TI>* f, void* out,
                 bool out_f64, const int* skip, cudaStream_t st);
 
 // krylov.cu

@@ -10,6 +10,7 @@
 #include <type_traits>
 #include <vector>
 
+#include "mg_cluster.cuh"
 #include "stencil.cuh"
 
 namespace helm {
@@ -1199,9 +1200,9 @@ static void vcycle_level(helm_ctx* c, int l, const cx<T>* f, void* out, bool out
       return;
     }
     const LevelHost& C = c->lv[l + 1];
-    fused_down2d<T>(c, l, f, (cx<T>*)L.w, (cx<T>*)C.f, skip, st);
+    fused_down2d<T, T>(c, l, f, (cx<T>*)L.w, (cx<T>*)C.f, skip, st);
     vcycle_level<T>(c, l + 1, (const cx<T>*)C.f, C.u, false, skip, st);
-    fused_up2d<T>(c, l, (const cx<T>*)L.w, (const cx<T>*)C.u, f, out, out_f64, skip, st);
+    fused_up2d<T, T>(c, l, (const cx<T>*)L.w, (const cx<T>*)C.u, f, out, out_f64, skip, st);
     return;
   }
   if (out_f64 && !std::is_same<T, double>::value) {
@@ -1278,6 +1279,20 @@ helm_status mg_input_from_c128(helm_ctx* c, const double2* in, void* out, cudaSt
   HELM_CUDA(cudaGetLastError());
   return HELM_OK;
 }
+
+helm_status mg_vcycle_from_c128(helm_ctx* c, const double2* r, void* buf, void* z, bool z64, cudaStream_t st) {
+  if (fused_applies<float>(c, 0) && (c->tail_first > 0 || ctail_applies(c))) {
+    if (c->tail_first == 0) return ctail_vcycle<float, double>(c, 0, r, z, z64, nullptr, st);
+    const LevelHost &L = c->lv[0], &C = c->lv[1];
+    fused_down2d<float, double>(c, 0, r, (float2*)L.w, (float2*)C.f, nullptr, st);
+    vcycle_level<float>(c, 1, (const float2*)C.f, C.u, false, nullptr, st);
+    fused_up2d<float, double>(c, 0, (const float2*)L.w, (const float2*)C.u, r, z, z64, nullptr, st);
+    HELM_CUDA(cudaGetLastError());
+    return HELM_OK;
+  }
+  helm_status s = mg_input_from_c128(c, r, buf, st);
+  return s == HELM_OK ? mg_vcycle<float>(c, (const float2*)buf, z, z64, nullptr, st) : s;
+}
 template helm_status mg_vcycle<float>(helm_ctx*, const float2*, void*, bool, const int*, cudaStream_t);
 template helm_status mg_vcycle<double>(helm_ctx*, const double2*, void*, bool, const int*, cudaStream_t);
 
@@ -1346,7 +1361,9 @@ static helm_status level_op_t(helm_ctx* c, int op, int lvl, void* a, const void*
     case HELM_OP_DOWN:
       if (lvl >= nl - 1 || L.dim != 2 || c->pc.nu1 != 1 || L.stg64 || L.any_offset0() || !A || !B || !O)
         return HELM_ERR_ARG;
-      fused_down2d<T>(c, lvl, B, A, O, nullptr, st);
+      fused_down2d<T, T>(c, lvl, B, A, O, nullptr, st);
+      // (FP32 damped Jacobi: the fused kernel leaves the iterate to the up kernel)
+      if (std::is_same<T, float>::value && c->pc.smoother != HELM_SM_RBGS) o.jacobi(nullptr, B, A, (T)c->pc.omega, nullptr, st);
       break;
     default: return HELM_ERR_ARG;
   }

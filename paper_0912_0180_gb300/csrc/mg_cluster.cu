@@ -130,8 +130,9 @@ __device__ __forceinline__ void ct_copy(double2* dst, const double2* src) {
 }
 
 // The levels a.first .. coarsest of one instance's cycle, by one cluster.
-template <typename T, bool RB, typename TO>
-__device__ __forceinline__ void ctail_body(const CTailArgs<T>* __restrict__ ga, const cx<T>* __restrict__ f_in,
+// TI: the type of f_in (complex128 when the whole FP32 cycle of a complex128 vector runs here).
+template <typename T, bool RB, typename TO, typename TI>
+__device__ __forceinline__ void ctail_body(const CTailArgs<T>* __restrict__ ga, const cx<TI>* __restrict__ f_in,
                                            cx<TO>* __restrict__ out, const int* skip) {
   extern __shared__ __align__(16) unsigned char ct_smem[];
   // the arguments in shared memory: as kernel parameters, every level's first use of its operator
@@ -235,7 +236,7 @@ __device__ __forceinline__ void ctail_body(const CTailArgs<T>* __restrict__ ga, 
           red[q] = !((x + j) & 1);
           if (e < ne && j >= 0 && j < s.n1) {
             if (k == 0) {
-              v[q] = f_in[x + s.n0 * j];
+              v[q] = cconv<T, TI>(f_in[x + s.n0 * j]);
             } else {
               const int o = ct_owner(j, s.n1, m1, sh);
               v[q] = remote(a.c[k] + (j - ct_first(s.n1, o, sh)) * s.n0 + x, o);
@@ -315,7 +316,7 @@ __device__ __forceinline__ void ctail_body(const CTailArgs<T>* __restrict__ ga, 
   if (last == 0) asm volatile("cp.async.wait_all;" ::: "memory");
   for (int e = tid; e < nop; e += CT) {
     if (last == 0) {
-      fl[e] = f_in[e];
+      fl[e] = cconv<T, TI>(f_in[e]);
     } else {
       int x, y;
       ct_div(e, l0, a.magic[last], x, y);
@@ -483,10 +484,10 @@ __device__ __forceinline__ void ctail_body(const CTailArgs<T>* __restrict__ ga, 
   }
 }
 
-template <typename T, bool RB, typename TO>
-__global__ void __launch_bounds__(CT, 1) k_ctail(const CTailArgs<T>* __restrict__ a, const cx<T>* __restrict__ f_in,
+template <typename T, bool RB, typename TO, typename TI>
+__global__ void __launch_bounds__(CT, 1) k_ctail(const CTailArgs<T>* __restrict__ a, const cx<TI>* __restrict__ f_in,
                                                  cx<TO>* __restrict__ out, const int* skip) {
-  ctail_body<T, RB, TO>(a, f_in, out, skip);
+  ctail_body<T, RB, TO, TI>(a, f_in, out, skip);
 }
 
 // The tails of a group's instances in one launch: virtual block w of the work list is cluster w.
@@ -500,7 +501,7 @@ __global__ void __launch_bounds__(CT, 1) kg_ctail(const GCTail<T>* __restrict__ 
   const int w = (int)(blockIdx.x / nc);
   if (w >= L.first[L.nd]) return;  // the whole cluster
   const GCTail<T>& g = A[L.map[w]];
-  ctail_body<T, RB, TO>(g.a, g.f, (cx<TO>*)g.out, g.skip);
+  ctail_body<T, RB, TO, T>(g.a, g.f, (cx<TO>*)g.out, g.skip);
 }
 
 template <typename K>
@@ -515,13 +516,17 @@ cudaError_t ct_prepare_all() {
   auto one = [&](auto kern) {
     if (e == cudaSuccess) e = ct_prepare(kern);
   };
-  one(k_ctail<T, false, T>);
-  one(k_ctail<T, true, T>);
+  one(k_ctail<T, false, T, T>);
+  one(k_ctail<T, true, T, T>);
   one(kg_ctail<T, false, T>);
   one(kg_ctail<T, true, T>);
   if (!std::is_same<T, double>::value) {
-    one(k_ctail<T, false, double>);
-    one(k_ctail<T, true, double>);
+    one(k_ctail<T, false, double, T>);
+    one(k_ctail<T, true, double, T>);
+    one(k_ctail<T, false, T, double>);
+    one(k_ctail<T, true, T, double>);
+    one(k_ctail<T, false, double, double>);
+    one(k_ctail<T, true, double, double>);
     one(kg_ctail<T, false, double>);
     one(kg_ctail<T, true, double>);
   }
@@ -554,8 +559,8 @@ int ct_blocks() {
     cfg.attrs = at;
     cfg.numAttrs = 1;
     int fit32 = 0, fit64 = 0;
-    if (cudaOccupancyMaxActiveClusters(&fit32, k_ctail<float, true, double>, &cfg) == cudaSuccess &&
-        cudaOccupancyMaxActiveClusters(&fit64, k_ctail<double, true, double>, &cfg) == cudaSuccess && fit32 > 0 &&
+    if (cudaOccupancyMaxActiveClusters(&fit32, k_ctail<float, true, double, double>, &cfg) == cudaSuccess &&
+        cudaOccupancyMaxActiveClusters(&fit64, k_ctail<double, true, double, double>, &cfg) == cudaSuccess && fit32 > 0 &&
         fit64 > 0) {
       known[dev] = nc;
       return nc;
@@ -824,8 +829,8 @@ template <typename T> size_t ctail_args(const helm_ctx* c, int first, const CTai
   return first < (int)c->ctail_smem.size() ? c->ctail_smem[first] : 0;
 }
 
-template <typename T>
-helm_status ctail_vcycle(const helm_ctx* c, int first, const cx<T>* f, void* out, bool out_f64, const int* skip,
+template <typename T, typename TI>
+helm_status ctail_vcycle(const helm_ctx* c, int first, const cx<TI>* f, void* out, bool out_f64, const int* skip,
                          cudaStream_t st) {
   const CTailArgs<T>* a;
   const size_t smem = ctail_args<T>(c, first, &a);
@@ -836,11 +841,11 @@ helm_status ctail_vcycle(const helm_ctx* c, int first, const cx<T>* f, void* out
   const bool rb = c->pc.smoother == HELM_SM_RBGS;
   const int nc = ct_blocks();
   if (out_f64) {
-    if (rb) launch_cluster(k_ctail<T, true, double>, nc, nc, smem, st, a, f, (double2*)out, skip);
-    else launch_cluster(k_ctail<T, false, double>, nc, nc, smem, st, a, f, (double2*)out, skip);
+    if (rb) launch_cluster(k_ctail<T, true, double, TI>, nc, nc, smem, st, a, f, (double2*)out, skip);
+    else launch_cluster(k_ctail<T, false, double, TI>, nc, nc, smem, st, a, f, (double2*)out, skip);
   } else {
-    if (rb) launch_cluster(k_ctail<T, true, T>, nc, nc, smem, st, a, f, (cx<T>*)out, skip);
-    else launch_cluster(k_ctail<T, false, T>, nc, nc, smem, st, a, f, (cx<T>*)out, skip);
+    if (rb) launch_cluster(k_ctail<T, true, T, TI>, nc, nc, smem, st, a, f, (cx<T>*)out, skip);
+    else launch_cluster(k_ctail<T, false, T, TI>, nc, nc, smem, st, a, f, (cx<T>*)out, skip);
   }
   HELM_CUDA(cudaGetLastError());
   return HELM_OK;
@@ -863,8 +868,9 @@ template helm_status ctail_build<float>(helm_ctx*, const double2*, cudaStream_t)
 template helm_status ctail_build<double>(helm_ctx*, const double2*, cudaStream_t);
 template size_t ctail_args<float>(const helm_ctx*, int, const CTailArgs<float>**);
 template size_t ctail_args<double>(const helm_ctx*, int, const CTailArgs<double>**);
-template helm_status ctail_vcycle<float>(const helm_ctx*, int, const float2*, void*, bool, const int*, cudaStream_t);
-template helm_status ctail_vcycle<double>(const helm_ctx*, int, const double2*, void*, bool, const int*, cudaStream_t);
+template helm_status ctail_vcycle<float, double>(const helm_ctx*, int, const double2*, void*, bool, const int*, cudaStream_t);
+template helm_status ctail_vcycle<float, float>(const helm_ctx*, int, const float2*, void*, bool, const int*, cudaStream_t);
+template helm_status ctail_vcycle<double, double>(const helm_ctx*, int, const double2*, void*, bool, const int*, cudaStream_t);
 template void ctail_group<float>(const GCTail<float>*, const GroupList*, int, int, bool, bool, size_t, cudaStream_t);
 template void ctail_group<double>(const GCTail<double>*, const GroupList*, int, int, bool, bool, size_t, cudaStream_t);
 

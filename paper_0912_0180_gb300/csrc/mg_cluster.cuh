@@ -40,8 +40,8 @@ int ctail_first_level(const helm_ctx* c, long points);
 template <typename T> helm_status ctail_build(helm_ctx* c, const double2* inv, cudaStream_t st);
 // the device arguments of a tail from level `first`, and its dynamic shared memory (0: does not fit)
 template <typename T> size_t ctail_args(const helm_ctx* c, int first, const CTailArgs<T>** a);
-template <typename T>
-helm_status ctail_vcycle(const helm_ctx* c, int first, const cx<T>* f, void* out, bool out_f64, const int* skip,
+template <typename T, typename TI>
+helm_status ctail_vcycle(const helm_ctx* c, int first, const cx<TI>* f, void* out, bool out_f64, const int* skip,
                          cudaStream_t st);
 template <typename T>
 void ctail_group(const GCTail<T>* args, const GroupList* LT, int li, int instances, bool rb, bool out_f64, size_t smem,

@@ -63,8 +63,18 @@ __device__ __forceinline__ bool colour_item(int k, int W, int gi0, int gj0, int 
   return x < W;
 }
 
-template <typename T, bool RBGS, int CX, int CY, int NT>
-__device__ __forceinline__ void down2d_body(int bx_, int by_, const OpView<T>& op, int nc0, int nc1, const cx<T>* __restrict__ f, cx<T>* __restrict__ u_out,
+// Whether the smoothed iterate of the zero guess goes through memory between the two halves of a level.
+// In FP32 damped Jacobi the up kernel forms it again, u = (omega / D) f, from the f and omega / D that it
+// reads anyway: 16 bytes a point less, one product more (2304^2 cycle with the narrowing below 158 ->
+// 141 us, 640^2 33.8 -> 29.4 us).
+// In FP64 the product is dearer than the bytes (2 FP64 lanes a clock), and red-black sweeps would need
+// their neighbours.
+template <typename T, bool RBGS> constexpr bool keeps_u() { return RBGS || sizeof(T) == 8; }
+
+// TI: element type of f -- complex128 on the finest level of an FP32 cycle called with a complex128
+// vector, narrowed as it is read (no conversion pass).
+template <typename T, bool RBGS, int CX, int CY, int NT, typename TI>
+__device__ __forceinline__ void down2d_body(int bx_, int by_, const OpView<T>& op, int nc0, int nc1, const cx<TI>* __restrict__ f, cx<T>* __restrict__ u_out,
          cx<T>* __restrict__ fc, T omega) {
   constexpr int HF = RBGS ? 2 : 1;
   constexpr int RX = 2 * CX + 1, RY = 2 * CY + 1;  // residual region
@@ -90,7 +100,7 @@ __device__ __forceinline__ void down2d_body(int bx_, int by_, const OpView<T>& o
       dv[it] = mkc<T>(T(0), T(0));
       if (e < FX * FY && i >= 0 && i < n0 && j >= 0 && j < n1) {
         int p = i + n0 * j;
-        fv[it] = f[p];
+        fv[it] = cconv<T, TI>(f[p]);
         dv[it] = op.dinv[p];
       }
     }
@@ -123,7 +133,7 @@ __device__ __forceinline__ void down2d_body(int bx_, int by_, const OpView<T>& o
   }
   // write the smoothed iterate of the points this tile owns (the last tile also owns the
   // fine point past the last coarse node when n is odd)
-  {
+  if constexpr (keeps_u<T, RBGS>()) {
     const int oi1 = (I0 + CX >= nc0) ? n0 : 2 * (I0 + CX);
     const int oj1 = (J0 + CY >= nc1) ? n1 : 2 * (J0 + CY);
     const int wx = oi1 - 2 * I0, wy = oj1 - 2 * J0;
@@ -182,20 +192,20 @@ __device__ __forceinline__ void down2d_body(int bx_, int by_, const OpView<T>& o
     fc[I + nc0 * J] = cscale<T>(T(0.0625), acc);
   }
 }
-template <typename T, bool RBGS, int CX, int CY, int NT>
+template <typename T, bool RBGS, int CX, int CY, int NT, typename TI>
 __global__ void __launch_bounds__(NT)
-k_down2d(OpView<T> op, int nc0, int nc1, const cx<T>* __restrict__ f, cx<T>* __restrict__ u_out,
+k_down2d(OpView<T> op, int nc0, int nc1, const cx<TI>* __restrict__ f, cx<T>* __restrict__ u_out,
          cx<T>* __restrict__ fc, T omega, const int* skip, int early) {
   if (early) pdl_trigger();
   pdl_entry();
   if (skip && *skip) return;
-  down2d_body<T, RBGS, CX, CY, NT>(blockIdx.x, blockIdx.y, op, nc0, nc1, f, u_out, fc, omega);
+  down2d_body<T, RBGS, CX, CY, NT, TI>(blockIdx.x, blockIdx.y, op, nc0, nc1, f, u_out, fc, omega);
 }
 
 // ---- up: prolongation + correction + post-smoothing (2D, nu2 = 1), out of place --------------
-template <typename T, bool RBGS, typename TO, int FX, int FY, int NT>
+template <typename T, bool RBGS, typename TO, int FX, int FY, int NT, typename TI>
 __device__ __forceinline__ void up2d_body(int bx_, int by_, const OpView<T>& op, int nc0, int nc1, const cx<T>* __restrict__ u_in, const cx<T>* __restrict__ ec,
-       const cx<T>* __restrict__ f, cx<TO>* __restrict__ u_out, T omega) {
+       const cx<TI>* __restrict__ f, cx<TO>* __restrict__ u_out, T omega) {
   constexpr int HU = RBGS ? 2 : 1;                 // halo of the corrected iterate
   constexpr int UX = FX + 2 * HU, UY = FY + 2 * HU;
   constexpr int CXN = UX / 2 + 3, CYN = UY / 2 + 3;  // coarse values covering the region
@@ -225,13 +235,20 @@ __device__ __forceinline__ void up2d_body(int bx_, int by_, const OpView<T>& op,
     y = 2 * (k / HX) + (c >> 1);
   };
   constexpr int NU = (UX * UY + NT - 1) / NT;
-  cx<T> uold[NU];
+  cx<T> uold[NU], dold[keeps_u<T, RBGS>() ? 1 : NU];
+  (void)dold;
 #pragma unroll
   for (int it = 0; it < NU; ++it) {
     int e = tid + it * NT, x, y;
     item(e, x, y);
     int i = ux0 + x, j = uy0 + y;
-    uold[it] = (e < UX * UY && i >= 0 && i < n0 && j >= 0 && j < n1) ? u_in[i + n0 * j] : mkc<T>(T(0), T(0));
+    const bool in = e < UX * UY && i >= 0 && i < n0 && j >= 0 && j < n1;
+    if constexpr (keeps_u<T, RBGS>()) {
+      uold[it] = in ? u_in[i + n0 * j] : mkc<T>(T(0), T(0));
+    } else {
+      uold[it] = in ? cconv<T, TI>(f[i + n0 * j]) : mkc<T>(T(0), T(0));
+      dold[it] = in ? op.dinv[i + n0 * j] : mkc<T>(T(0), T(0));
+    }
   }
 #pragma unroll
   for (int it = 0; it < NU; ++it) {
@@ -261,7 +278,8 @@ __device__ __forceinline__ void up2d_body(int bx_, int by_, const OpView<T>& op,
         w = ((i & 1) ? T(1) : T(0.5)) * ((j & 1) ? T(1) : T(0.5));
       }
       // the weight is a power of two, so w acc is exact and one FMA gives u + w acc as before
-      const cx<T> uo = uold[it];
+      cx<T> uo = uold[it];
+      if constexpr (!keeps_u<T, RBGS>()) uo = cmul1<T>(uo, dold[it]);
       v = mkc<T>(fma(w, acc.x, uo.x), fma(w, acc.y, uo.y));
     }
     su[y][x] = v;
@@ -275,7 +293,7 @@ __device__ __forceinline__ void up2d_body(int bx_, int by_, const OpView<T>& op,
       int p = i + n0 * j;
       int sx = x + HU, sy = y + HU;
       cx<T> acc = off2d<T>(op, i, j, su[sy][sx - 1], su[sy][sx + 1], su[sy - 1][sx], su[sy + 1][sx]);
-      cx<T> g = cmul1<T>(csub<T>(f[p], acc), op.dinv[p]);  // dinv holds omega / D
+      cx<T> g = cmul1<T>(csub<T>(cconv<T, TI>(f[p]), acc), op.dinv[p]);  // dinv holds omega / D
       cx<T> uc = su[sy][sx];
       const T om1 = T(1) - omega;
       u_out[p] = cconv<TO, T>(mkc<T>(fma(om1, uc.x, g.x), fma(om1, uc.y, g.y)));
@@ -295,7 +313,7 @@ __device__ __forceinline__ void up2d_body(int bx_, int by_, const OpView<T>& op,
       if (c == 0 && i >= 0 && i < n0 && j >= 0 && j < n1) {
         int p = i + n0 * j;
         cx<T> acc = off2d<T>(op, i, j, su[sy][sx - 1], su[sy][sx + 1], su[sy - 1][sx], su[sy + 1][sx]);
-        v = cmul1<T>(csub<T>(f[p], acc), op.dinv[p]);
+        v = cmul1<T>(csub<T>(cconv<T, TI>(f[p]), acc), op.dinv[p]);
       }
       sred[y][x] = v;
     }
@@ -312,19 +330,19 @@ __device__ __forceinline__ void up2d_body(int bx_, int by_, const OpView<T>& op,
       cx<T> v = sred[sy][sx];
       if (c == 1) {
         cx<T> acc = off2d<T>(op, i, j, sred[sy][sx - 1], sred[sy][sx + 1], sred[sy - 1][sx], sred[sy + 1][sx]);
-        v = cmul1<T>(csub<T>(f[p], acc), op.dinv[p]);
+        v = cmul1<T>(csub<T>(cconv<T, TI>(f[p]), acc), op.dinv[p]);
       }
       u_out[p] = cconv<TO, T>(v);
     }
   }
 }
-template <typename T, bool RBGS, typename TO, int FX, int FY, int NT>
+template <typename T, bool RBGS, typename TO, int FX, int FY, int NT, typename TI>
 __global__ void __launch_bounds__(NT)
 k_up2d(OpView<T> op, int nc0, int nc1, const cx<T>* __restrict__ u_in, const cx<T>* __restrict__ ec,
-       const cx<T>* __restrict__ f, cx<TO>* __restrict__ u_out, T omega, const int* skip) {
+       const cx<TI>* __restrict__ f, cx<TO>* __restrict__ u_out, T omega, const int* skip) {
   pdl_entry();
   if (skip && *skip) return;
-  up2d_body<T, RBGS, TO, FX, FY, NT>(blockIdx.x, blockIdx.y, op, nc0, nc1, u_in, ec, f, u_out, omega);
+  up2d_body<T, RBGS, TO, FX, FY, NT, TI>(blockIdx.x, blockIdx.y, op, nc0, nc1, u_in, ec, f, u_out, omega);
 }
 
 // ---- tail: the coarsest levels in one block ------------------------------------------------
@@ -659,7 +677,7 @@ static size_t tail_args(const helm_ctx* c, int first, TailArgs<T>& a) {
 template <typename T>
 helm_status tail_vcycle(helm_ctx* c, int first, const cx<T>* f, void* out, bool out_f64, const int* skip,
                         cudaStream_t st) {
-  if (ctail_applies(c)) return ctail_vcycle<T>(c, first, f, out, out_f64, skip, st);
+  if (ctail_applies(c)) return ctail_vcycle<T, T>(c, first, f, out, out_f64, skip, st);
   TailArgs<T> a;
   const size_t smem = tail_args<T>(c, first, a);
   if (out_f64) return tail_launch<T, double>(a, c->grid.dim, smem, f, (double2*)out, skip, st);
@@ -672,22 +690,22 @@ static bool big_tiles(const helm_ctx* c, long blocks) {
   return blocks >= 2L * sms;
 }
 
-template <typename T, bool RB, int CX, int CY, int NT>
-static void down_launch(const LevelHost& F, const LevelHost& C, const cx<T>* f, cx<T>* u_out, cx<T>* fc, T om,
+template <typename T, bool RB, int CX, int CY, int NT, typename TI>
+static void down_launch(const LevelHost& F, const LevelHost& C, const cx<TI>* f, cx<T>* u_out, cx<T>* fc, T om,
                         const int* skip, cudaStream_t st, int early) {
   dim3 g((C.n[0] + CX - 1) / CX, (C.n[1] + CY - 1) / CY);
-  launch_pdl(k_down2d<T, RB, CX, CY, NT>, dim3(g), dim3(NT), 0, st, F.view<T>(), C.n[0], C.n[1], f, u_out, fc, om, skip,
+  launch_pdl(k_down2d<T, RB, CX, CY, NT, TI>, dim3(g), dim3(NT), 0, st, F.view<T>(), C.n[0], C.n[1], f, u_out, fc, om, skip,
              early);
 }
 
-template <typename T, bool RB>
-static void down_tile(int tile, const LevelHost& F, const LevelHost& C, const cx<T>* f, cx<T>* u_out, cx<T>* fc, T om,
+template <typename T, bool RB, typename TI = T>
+static void down_tile(int tile, const LevelHost& F, const LevelHost& C, const cx<TI>* f, cx<T>* u_out, cx<T>* fc, T om,
                       const int* skip, cudaStream_t st, int early = 0) {
-  if (tile == TILE_BIG) down_launch<T, RB, DN_CX, DN_CY, FUSED_THREADS>(F, C, f, u_out, fc, om, skip, st, early);
-  else if (tile == TILE_TINY) down_launch<T, RB, DN_TCX, DN_TCY, FUSED_TINY_THREADS>(F, C, f, u_out, fc, om, skip, st, early);
-  else if (tile == TILE_SQUARE) down_launch<T, RB, DN_QCX, DN_QCY, FUSED_SMALL_THREADS>(F, C, f, u_out, fc, om, skip, st, early);
-  else if (tile == TILE_WIDE) down_launch<T, RB, DN_WCX, DN_WCY, FUSED_THREADS>(F, C, f, u_out, fc, om, skip, st, early);
-  else down_launch<T, RB, DN_SCX, DN_SCY, FUSED_SMALL_THREADS>(F, C, f, u_out, fc, om, skip, st, early);
+  if (tile == TILE_BIG) down_launch<T, RB, DN_CX, DN_CY, FUSED_THREADS, TI>(F, C, f, u_out, fc, om, skip, st, early);
+  else if (tile == TILE_TINY) down_launch<T, RB, DN_TCX, DN_TCY, FUSED_TINY_THREADS, TI>(F, C, f, u_out, fc, om, skip, st, early);
+  else if (tile == TILE_SQUARE) down_launch<T, RB, DN_QCX, DN_QCY, FUSED_SMALL_THREADS, TI>(F, C, f, u_out, fc, om, skip, st, early);
+  else if (tile == TILE_WIDE) down_launch<T, RB, DN_WCX, DN_WCY, FUSED_THREADS, TI>(F, C, f, u_out, fc, om, skip, st, early);
+  else down_launch<T, RB, DN_SCX, DN_SCY, FUSED_SMALL_THREADS, TI>(F, C, f, u_out, fc, om, skip, st, early);
 }
 
 // The tile a level's fused kernels use (the autotuner's choice, else the block-count rule) and its
@@ -714,8 +732,8 @@ static int up_tile_of(const helm_ctx* c, int l, int* tx, int* ty) {
   return tile;
 }
 
-template <typename T>
-void fused_down2d(const helm_ctx* c, int l, const cx<T>* f, cx<T>* u_out, cx<T>* fc, const int* skip, cudaStream_t st) {
+template <typename T, typename TI>
+void fused_down2d(const helm_ctx* c, int l, const cx<TI>* f, cx<T>* u_out, cx<T>* fc, const int* skip, cudaStream_t st) {
   const LevelHost& F = c->lv[l];
   const LevelHost& C = c->lv[l + 1];
   long nb = (long)((C.n[0] + DN_CX - 1) / DN_CX) * ((C.n[1] + DN_CY - 1) / DN_CY);
@@ -724,46 +742,46 @@ void fused_down2d(const helm_ctx* c, int l, const cx<T>* f, cx<T>* u_out, cx<T>*
   // before the one-cluster tail (16 blocks, which read their constants before they wait) the launch
   // of the next kernel is triggered at once
   const int early = l + 1 == c->tail_first && ctail_applies(c);
-  if (c->pc.smoother == HELM_SM_RBGS) down_tile<T, true>(tile, F, C, f, u_out, fc, om, skip, st, early);
-  else down_tile<T, false>(tile, F, C, f, u_out, fc, om, skip, st, early);
+  if (c->pc.smoother == HELM_SM_RBGS) down_tile<T, true, TI>(tile, F, C, f, u_out, fc, om, skip, st, early);
+  else down_tile<T, false, TI>(tile, F, C, f, u_out, fc, om, skip, st, early);
 }
 
-template <typename T, bool RB, typename TO, int FX, int FY, int NT>
-static void up_launch(const LevelHost& F, const LevelHost& C, const cx<T>* u_in, const cx<T>* ec, const cx<T>* f,
+template <typename T, bool RB, typename TO, int FX, int FY, int NT, typename TI>
+static void up_launch(const LevelHost& F, const LevelHost& C, const cx<T>* u_in, const cx<T>* ec, const cx<TI>* f,
                       TO* out, T om, const int* skip, cudaStream_t st) {
   dim3 g((F.n[0] + FX - 1) / FX, (F.n[1] + FY - 1) / FY);
-  launch_pdl(k_up2d<T, RB, TO, FX, FY, NT>, dim3(g), dim3(NT), 0, st, F.view<T>(), C.n[0], C.n[1], u_in, ec, f,
+  launch_pdl(k_up2d<T, RB, TO, FX, FY, NT, TI>, dim3(g), dim3(NT), 0, st, F.view<T>(), C.n[0], C.n[1], u_in, ec, f,
              (cx<TO>*)out, om, skip);
 }
 
-template <typename T, bool RB, typename TO>
+template <typename T, bool RB, typename TO, typename TI = T>
 static void up_tile(int tile, const LevelHost& F, const LevelHost& C, const cx<T>* u_in, const cx<T>* ec,
-                    const cx<T>* f, TO* o, T om, const int* skip, cudaStream_t st) {
-  if (tile == TILE_BIG) up_launch<T, RB, TO, UP_FX, UP_FY, FUSED_THREADS>(F, C, u_in, ec, f, o, om, skip, st);
-  else if (tile == TILE_TINY) up_launch<T, RB, TO, UP_TFX, UP_TFY, FUSED_TINY_THREADS>(F, C, u_in, ec, f, o, om, skip, st);
-  else if (tile == TILE_SQUARE) up_launch<T, RB, TO, UP_QFX, UP_QFY, FUSED_SMALL_THREADS>(F, C, u_in, ec, f, o, om, skip, st);
-  else if (tile == TILE_WIDE) up_launch<T, RB, TO, UP_WFX, UP_WFY, FUSED_THREADS>(F, C, u_in, ec, f, o, om, skip, st);
-  else up_launch<T, RB, TO, UP_SFX, UP_SFY, FUSED_SMALL_THREADS>(F, C, u_in, ec, f, o, om, skip, st);
+                    const cx<TI>* f, TO* o, T om, const int* skip, cudaStream_t st) {
+  if (tile == TILE_BIG) up_launch<T, RB, TO, UP_FX, UP_FY, FUSED_THREADS, TI>(F, C, u_in, ec, f, o, om, skip, st);
+  else if (tile == TILE_TINY) up_launch<T, RB, TO, UP_TFX, UP_TFY, FUSED_TINY_THREADS, TI>(F, C, u_in, ec, f, o, om, skip, st);
+  else if (tile == TILE_SQUARE) up_launch<T, RB, TO, UP_QFX, UP_QFY, FUSED_SMALL_THREADS, TI>(F, C, u_in, ec, f, o, om, skip, st);
+  else if (tile == TILE_WIDE) up_launch<T, RB, TO, UP_WFX, UP_WFY, FUSED_THREADS, TI>(F, C, u_in, ec, f, o, om, skip, st);
+  else up_launch<T, RB, TO, UP_SFX, UP_SFY, FUSED_SMALL_THREADS, TI>(F, C, u_in, ec, f, o, om, skip, st);
 }
 
-template <typename T, typename TO>
+template <typename T, typename TO, typename TI>
 static void up_dispatch(const helm_ctx* c, const LevelHost& F, const LevelHost& C, const cx<T>* u_in, const cx<T>* ec,
-                        const cx<T>* f, void* out, const int* skip, cudaStream_t st) {
+                        const cx<TI>* f, void* out, const int* skip, cudaStream_t st) {
   long nb = (long)((F.n[0] + UP_FX - 1) / UP_FX) * ((F.n[1] + UP_FY - 1) / UP_FY);
   int tile = F.tile_up >= 0 ? F.tile_up : (big_tiles(c, nb) ? TILE_BIG : TILE_SMALL);
   T om = (T)c->pc.omega;
   TO* o = (TO*)out;
-  if (c->pc.smoother == HELM_SM_RBGS) up_tile<T, true, TO>(tile, F, C, u_in, ec, f, o, om, skip, st);
-  else up_tile<T, false, TO>(tile, F, C, u_in, ec, f, o, om, skip, st);
+  if (c->pc.smoother == HELM_SM_RBGS) up_tile<T, true, TO, TI>(tile, F, C, u_in, ec, f, o, om, skip, st);
+  else up_tile<T, false, TO, TI>(tile, F, C, u_in, ec, f, o, om, skip, st);
 }
 
-template <typename T>
-void fused_up2d(const helm_ctx* c, int l, const cx<T>* u_in, const cx<T>* ec, const cx<T>* f, void* out,
+template <typename T, typename TI>
+void fused_up2d(const helm_ctx* c, int l, const cx<T>* u_in, const cx<T>* ec, const cx<TI>* f, void* out,
                 bool out_f64, const int* skip, cudaStream_t st) {
   const LevelHost& F = c->lv[l];
   const LevelHost& C = c->lv[l + 1];
-  if (out_f64) up_dispatch<T, double>(c, F, C, u_in, ec, f, out, skip, st);
-  else up_dispatch<T, T>(c, F, C, u_in, ec, f, out, skip, st);
+  if (out_f64) up_dispatch<T, double, TI>(c, F, C, u_in, ec, f, out, skip, st);
+  else up_dispatch<T, T, TI>(c, F, C, u_in, ec, f, out, skip, st);
 }
 
 // ---- grouped V-cycle: one launch per level for many instances --------------------------------
@@ -809,7 +827,7 @@ __global__ void __launch_bounds__(NT) kg_down2d(const GDown<T>* __restrict__ A, 
   group_visit(LT[li], [&](int d, int vb) {
     const GDown<T>& g = A[d];
     if (g.skip && *g.skip) return;
-    down2d_body<T, RBGS, CX, CY, NT>(vb % g.tiles_x, vb / g.tiles_x, g.op, g.nc0, g.nc1, g.f, g.u_out, g.fc,
+    down2d_body<T, RBGS, CX, CY, NT, T>(vb % g.tiles_x, vb / g.tiles_x, g.op, g.nc0, g.nc1, g.f, g.u_out, g.fc,
                                      g.omega);
   });
 }
@@ -820,7 +838,7 @@ __global__ void __launch_bounds__(NT) kg_up2d(const GUp<T>* __restrict__ A, cons
   group_visit(LT[li], [&](int d, int vb) {
     const GUp<T>& g = A[d];
     if (g.skip && *g.skip) return;
-    up2d_body<T, RBGS, TO, FX, FY, NT>(vb % g.tiles_x, vb / g.tiles_x, g.op, g.nc0, g.nc1, g.u_in, g.ec, g.f,
+    up2d_body<T, RBGS, TO, FX, FY, NT, T>(vb % g.tiles_x, vb / g.tiles_x, g.op, g.nc0, g.nc1, g.u_in, g.ec, g.f,
                                        (cx<TO>*)g.u_out, g.omega);
   });
 }
@@ -1277,9 +1295,11 @@ template int tail_first_level<float>(const helm_ctx*);
 template int tail_first_level<double>(const helm_ctx*);
 template helm_status tail_vcycle<float>(helm_ctx*, int, const float2*, void*, bool, const int*, cudaStream_t);
 template helm_status tail_vcycle<double>(helm_ctx*, int, const double2*, void*, bool, const int*, cudaStream_t);
-template void fused_down2d<float>(const helm_ctx*, int, const float2*, float2*, float2*, const int*, cudaStream_t);
-template void fused_down2d<double>(const helm_ctx*, int, const double2*, double2*, double2*, const int*, cudaStream_t);
-template void fused_up2d<float>(const helm_ctx*, int, const float2*, const float2*, const float2*, void*, bool, const int*, cudaStream_t);
-template void fused_up2d<double>(const helm_ctx*, int, const double2*, const double2*, const double2*, void*, bool, const int*, cudaStream_t);
+template void fused_down2d<float, float>(const helm_ctx*, int, const float2*, float2*, float2*, const int*, cudaStream_t);
+template void fused_down2d<float, double>(const helm_ctx*, int, const double2*, float2*, float2*, const int*, cudaStream_t);
+template void fused_down2d<double, double>(const helm_ctx*, int, const double2*, double2*, double2*, const int*, cudaStream_t);
+template void fused_up2d<float, float>(const helm_ctx*, int, const float2*, const float2*, const float2*, void*, bool, const int*, cudaStream_t);
+template void fused_up2d<float, double>(const helm_ctx*, int, const float2*, const float2*, const double2*, void*, bool, const int*, cudaStream_t);
+template void fused_up2d<double, double>(const helm_ctx*, int, const double2*, const double2*, const double2*, void*, bool, const int*, cudaStream_t);
 
 }  // namespace helm
