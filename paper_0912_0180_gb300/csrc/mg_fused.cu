@@ -27,6 +27,7 @@
 #include <tuple>
 #include <type_traits>
 
+#include "march2d.cuh"
 #include "mg_cluster.cuh"
 #include "stencil.cuh"
 
@@ -45,8 +46,9 @@ constexpr int FUSED_THREADS = 256, FUSED_SMALL_THREADS = 128, FUSED_TINY_THREADS
 // between the small and the large tile's (for an even spread over the SMs)
 // and a wide tile of 256 threads (16 x 12 coarse / 32 x 24 fine), whose halo is the smallest (the
 // recomputed sweep and residual cost most in FP64, where the fine levels are bound by the FP64 pipe)
-enum { TILE_SMALL = 0, TILE_BIG = 1, TILE_TINY = 2, TILE_SQUARE = 3, TILE_WIDE = 4 };
-constexpr int NUM_TILES = 5;
+// and, for damped Jacobi, the row-walking kernels of march2d.cuh in two lengths
+enum { TILE_SMALL = 0, TILE_BIG = 1, TILE_TINY = 2, TILE_SQUARE = 3, TILE_WIDE = 4, TILE_LONG = 5, TILE_SHORT = 6 };
+constexpr int NUM_TILES = 7;
 constexpr int DN_WCX = 16, DN_WCY = 12, UP_WFX = 32, UP_WFY = 24;
 
 // ---- down: smooth from zero + residual + restriction (2D, nu1 = 1) ---------------------------
@@ -343,6 +345,25 @@ k_up2d(OpView<T> op, int nc0, int nc1, const cx<T>* __restrict__ u_in, const cx<
   pdl_entry();
   if (skip && *skip) return;
   up2d_body<T, RBGS, TO, FX, FY, NT, TI>(blockIdx.x, blockIdx.y, op, nc0, nc1, u_in, ec, f, u_out, omega);
+}
+
+// ---- the row-walking kernels (damped Jacobi) ---------------------------------------------------
+template <typename T, typename TI, int CR>
+__global__ void __launch_bounds__(MARCH_THREADS)
+k_march_down(OpView<T> op, int nc0, int nc1, const cx<TI>* __restrict__ f, cx<T>* __restrict__ u_out,
+             cx<T>* __restrict__ fc, T omega, int vec, const int* skip, int early) {
+  if (early) pdl_trigger();
+  pdl_entry();
+  if (skip && *skip) return;
+  march_down<T, TI, CR, keeps_u<T, false>()>(blockIdx.x, blockIdx.y, op, nc0, nc1, f, u_out, fc, omega, vec != 0);
+}
+template <typename T, typename TO, typename TI, int CR>
+__global__ void __launch_bounds__(MARCH_THREADS)
+k_march_up(OpView<T> op, int nc0, int nc1, const cx<T>* __restrict__ u_in, const cx<T>* __restrict__ ec,
+           const cx<TI>* __restrict__ f, cx<TO>* __restrict__ u_out, T omega, int vec, const int* skip) {
+  pdl_entry();
+  if (skip && *skip) return;
+  march_up<T, TO, TI, CR, keeps_u<T, false>()>(blockIdx.x, blockIdx.y, op, nc0, nc1, u_in, ec, f, u_out, omega, vec != 0);
 }
 
 // ---- tail: the coarsest levels in one block ------------------------------------------------
@@ -698,9 +719,35 @@ static void down_launch(const LevelHost& F, const LevelHost& C, const cx<TI>* f,
              early);
 }
 
+// whether pairs of columns of complex64 are 16-byte aligned in every array a level's kernel reads or
+// writes by pairs
+template <typename T>
+static int march_vec(const LevelHost& F, const void* f, const void* b) {
+  if (sizeof(T) != 4) return 0;
+  return F.n[0] % 2 == 0 && ((((uintptr_t)f | (uintptr_t)b | (uintptr_t)F.dinv32) & 15) == 0);
+}
+template <typename T, int CR, typename TI>
+static void march_down_launch(const LevelHost& F, const LevelHost& C, const cx<TI>* f, cx<T>* u_out, cx<T>* fc, T om,
+                              const int* skip, cudaStream_t st, int early) {
+  dim3 g(march_strips((F.n[0] + 1) / 2), (C.n[1] + CR - 1) / CR);
+  launch_pdl(k_march_down<T, TI, CR>, g, dim3(MARCH_THREADS), 0, st, F.view<T>(), C.n[0], C.n[1], f, u_out, fc, om,
+             march_vec<T>(F, f, u_out), skip, early);
+}
+template <typename T, typename TO, int CR, typename TI>
+static void march_up_launch(const LevelHost& F, const LevelHost& C, const cx<T>* u_in, const cx<T>* ec, const cx<TI>* f,
+                            TO* out, T om, const int* skip, cudaStream_t st) {
+  dim3 g(march_strips((F.n[0] + 1) / 2), (F.n[1] + 2 * CR - 1) / (2 * CR));
+  launch_pdl(k_march_up<T, TO, TI, CR>, g, dim3(MARCH_THREADS), 0, st, F.view<T>(), C.n[0], C.n[1], u_in, ec, f,
+             (cx<TO>*)out, om, march_vec<T>(F, f, out), skip);
+}
+
 template <typename T, bool RB, typename TI = T>
 static void down_tile(int tile, const LevelHost& F, const LevelHost& C, const cx<TI>* f, cx<T>* u_out, cx<T>* fc, T om,
                       const int* skip, cudaStream_t st, int early = 0) {
+  if constexpr (!RB) {
+    if (tile == TILE_LONG) return march_down_launch<T, MARCH_LONG, TI>(F, C, f, u_out, fc, om, skip, st, early);
+    if (tile == TILE_SHORT) return march_down_launch<T, MARCH_SHORT, TI>(F, C, f, u_out, fc, om, skip, st, early);
+  }
   if (tile == TILE_BIG) down_launch<T, RB, DN_CX, DN_CY, FUSED_THREADS, TI>(F, C, f, u_out, fc, om, skip, st, early);
   else if (tile == TILE_TINY) down_launch<T, RB, DN_TCX, DN_TCY, FUSED_TINY_THREADS, TI>(F, C, f, u_out, fc, om, skip, st, early);
   else if (tile == TILE_SQUARE) down_launch<T, RB, DN_QCX, DN_QCY, FUSED_SMALL_THREADS, TI>(F, C, f, u_out, fc, om, skip, st, early);
@@ -708,27 +755,43 @@ static void down_tile(int tile, const LevelHost& F, const LevelHost& C, const cx
   else down_launch<T, RB, DN_SCX, DN_SCY, FUSED_SMALL_THREADS, TI>(F, C, f, u_out, fc, om, skip, st, early);
 }
 
-// The tile a level's fused kernels use (the autotuner's choice, else the block-count rule) and its
-// coarse (down) or fine (up) extent.
-static int down_tile_of(const helm_ctx* c, int l, int* tx, int* ty) {
+// The tile a level's fused kernels use (the autotuner's choice, else the block-count rule) and the
+// launch's blocks.
+static int down_tile_of(const helm_ctx* c, int l, int* bx, int* by) {
   const LevelHost& F = c->lv[l];
   const LevelHost& C = c->lv[l + 1];
   long nb = (long)((C.n[0] + DN_CX - 1) / DN_CX) * ((C.n[1] + DN_CY - 1) / DN_CY);
   int tile = F.tile_down >= 0 ? F.tile_down : (big_tiles(c, nb) ? TILE_BIG : TILE_SMALL);
-  *tx = tile == TILE_BIG ? DN_CX : tile == TILE_TINY ? DN_TCX : tile == TILE_SQUARE ? DN_QCX
+  if (tile == TILE_LONG || tile == TILE_SHORT) {
+    const int cr = tile == TILE_LONG ? MARCH_LONG : MARCH_SHORT;
+    *bx = march_strips((F.n[0] + 1) / 2);
+    *by = (C.n[1] + cr - 1) / cr;
+    return tile;
+  }
+  const int tx = tile == TILE_BIG ? DN_CX : tile == TILE_TINY ? DN_TCX : tile == TILE_SQUARE ? DN_QCX
       : tile == TILE_WIDE ? DN_WCX : DN_SCX;
-  *ty = tile == TILE_BIG ? DN_CY : tile == TILE_TINY ? DN_TCY : tile == TILE_SQUARE ? DN_QCY
+  const int ty = tile == TILE_BIG ? DN_CY : tile == TILE_TINY ? DN_TCY : tile == TILE_SQUARE ? DN_QCY
       : tile == TILE_WIDE ? DN_WCY : DN_SCY;
+  *bx = (C.n[0] + tx - 1) / tx;
+  *by = (C.n[1] + ty - 1) / ty;
   return tile;
 }
-static int up_tile_of(const helm_ctx* c, int l, int* tx, int* ty) {
+static int up_tile_of(const helm_ctx* c, int l, int* bx, int* by) {
   const LevelHost& F = c->lv[l];
   long nb = (long)((F.n[0] + UP_FX - 1) / UP_FX) * ((F.n[1] + UP_FY - 1) / UP_FY);
   int tile = F.tile_up >= 0 ? F.tile_up : (big_tiles(c, nb) ? TILE_BIG : TILE_SMALL);
-  *tx = tile == TILE_BIG ? UP_FX : tile == TILE_TINY ? UP_TFX : tile == TILE_SQUARE ? UP_QFX
+  if (tile == TILE_LONG || tile == TILE_SHORT) {
+    const int fr = 2 * (tile == TILE_LONG ? MARCH_LONG : MARCH_SHORT);
+    *bx = march_strips((F.n[0] + 1) / 2);
+    *by = (F.n[1] + fr - 1) / fr;
+    return tile;
+  }
+  const int tx = tile == TILE_BIG ? UP_FX : tile == TILE_TINY ? UP_TFX : tile == TILE_SQUARE ? UP_QFX
       : tile == TILE_WIDE ? UP_WFX : UP_SFX;
-  *ty = tile == TILE_BIG ? UP_FY : tile == TILE_TINY ? UP_TFY : tile == TILE_SQUARE ? UP_QFY
+  const int ty = tile == TILE_BIG ? UP_FY : tile == TILE_TINY ? UP_TFY : tile == TILE_SQUARE ? UP_QFY
       : tile == TILE_WIDE ? UP_WFY : UP_SFY;
+  *bx = (F.n[0] + tx - 1) / tx;
+  *by = (F.n[1] + ty - 1) / ty;
   return tile;
 }
 
@@ -757,6 +820,10 @@ static void up_launch(const LevelHost& F, const LevelHost& C, const cx<T>* u_in,
 template <typename T, bool RB, typename TO, typename TI = T>
 static void up_tile(int tile, const LevelHost& F, const LevelHost& C, const cx<T>* u_in, const cx<T>* ec,
                     const cx<TI>* f, TO* o, T om, const int* skip, cudaStream_t st) {
+  if constexpr (!RB) {
+    if (tile == TILE_LONG) return march_up_launch<T, TO, MARCH_LONG, TI>(F, C, u_in, ec, f, o, om, skip, st);
+    if (tile == TILE_SHORT) return march_up_launch<T, TO, MARCH_SHORT, TI>(F, C, u_in, ec, f, o, om, skip, st);
+  }
   if (tile == TILE_BIG) up_launch<T, RB, TO, UP_FX, UP_FY, FUSED_THREADS, TI>(F, C, u_in, ec, f, o, om, skip, st);
   else if (tile == TILE_TINY) up_launch<T, RB, TO, UP_TFX, UP_TFY, FUSED_TINY_THREADS, TI>(F, C, u_in, ec, f, o, om, skip, st);
   else if (tile == TILE_SQUARE) up_launch<T, RB, TO, UP_QFX, UP_QFY, FUSED_SMALL_THREADS, TI>(F, C, u_in, ec, f, o, om, skip, st);
@@ -800,7 +867,7 @@ template <typename T> struct GDown {
   cx<T>* fc;
   T omega;
   const int* skip;
-  int tiles_x;
+  int tiles_x, vec;
 };
 template <typename T> struct GUp {
   OpView<T> op;
@@ -811,7 +878,7 @@ template <typename T> struct GUp {
   void* u_out;  // cx<T>, or complex128 on the finest level
   T omega;
   const int* skip;
-  int tiles_x;
+  int tiles_x, vec;
 };
 template <typename T> struct GCoarse {
   const cx<T>* ainv;
@@ -840,6 +907,29 @@ __global__ void __launch_bounds__(NT) kg_up2d(const GUp<T>* __restrict__ A, cons
     if (g.skip && *g.skip) return;
     up2d_body<T, RBGS, TO, FX, FY, NT, T>(vb % g.tiles_x, vb / g.tiles_x, g.op, g.nc0, g.nc1, g.u_in, g.ec, g.f,
                                        (cx<TO>*)g.u_out, g.omega);
+  });
+}
+
+template <typename T, int CR>
+__global__ void __launch_bounds__(MARCH_THREADS) kg_march_down(const GDown<T>* __restrict__ A,
+                                                               const GroupList* __restrict__ LT, int li) {
+  pdl_entry();
+  group_visit(LT[li], [&](int d, int vb) {
+    const GDown<T>& g = A[d];
+    if (g.skip && *g.skip) return;
+    march_down<T, T, CR, keeps_u<T, false>()>(vb % g.tiles_x, vb / g.tiles_x, g.op, g.nc0, g.nc1, g.f, g.u_out, g.fc,
+                                              g.omega, g.vec != 0);
+  });
+}
+template <typename T, typename TO, int CR>
+__global__ void __launch_bounds__(MARCH_THREADS) kg_march_up(const GUp<T>* __restrict__ A,
+                                                             const GroupList* __restrict__ LT, int li) {
+  pdl_entry();
+  group_visit(LT[li], [&](int d, int vb) {
+    const GUp<T>& g = A[d];
+    if (g.skip && *g.skip) return;
+    march_up<T, TO, T, CR, keeps_u<T, false>()>(vb % g.tiles_x, vb / g.tiles_x, g.op, g.nc0, g.nc1, g.u_in, g.ec, g.f,
+                                                (cx<TO>*)g.u_out, g.omega, g.vec != 0);
   });
 }
 
@@ -923,20 +1013,21 @@ helm_status group_vcycle_build(helm_ctx* const* cs, int ni, const void* const* i
         const LevelHost& F = c->lv[l];
         const LevelHost& C = c->lv[l + 1];
         const cx<T>* f = l == 0 ? (const cx<T>*)in[i] : (const cx<T>*)F.f;
-        int tx, ty;
-        if (down_tile_of(c, l, &tx, &ty) == tile) {
+        int bx, by;
+        if (down_tile_of(c, l, &bx, &by) == tile) {
           GDown<T> d{F.view<T>(), C.n[0], C.n[1], f, (cx<T>*)F.w, (cx<T>*)C.f, (T)c->pc.omega, skip[i],
-                     (C.n[0] + tx - 1) / tx};
+                     bx, march_vec<T>(F, f, F.w)};
           dv.push_back(d);
           di.push_back(i);
-          dn.push_back(d.tiles_x * ((C.n[1] + ty - 1) / ty));
+          dn.push_back(bx * by);
         }
-        if (up_tile_of(c, l, &tx, &ty) == tile) {
+        if (up_tile_of(c, l, &bx, &by) == tile) {
           GUp<T> u{F.view<T>(), C.n[0], C.n[1], (const cx<T>*)F.w, (const cx<T>*)C.u, f,
-                   l == 0 ? (void*)out[i] : F.u, (T)c->pc.omega, skip[i], (F.n[0] + tx - 1) / tx};
+                   l == 0 ? (void*)out[i] : F.u, (T)c->pc.omega, skip[i], bx,
+                   march_vec<T>(F, f, l == 0 ? (const void*)out[i] : F.u)};
           uv.push_back(u);
           ui.push_back(i);
-          un.push_back(u.tiles_x * ((F.n[1] + ty - 1) / ty));
+          un.push_back(bx * by);
         }
       }
       GroupVcycle::Launch ld, lu;
@@ -1021,6 +1112,12 @@ helm_status group_vcycle_finalize(GroupVcycle* P, const GroupLists* lists) {
 template <typename T, bool RB>
 static void group_down_launch(const GroupVcycle::Launch& L, const GroupList* LT, cudaStream_t st) {
   const GDown<T>* a = (const GDown<T>*)L.args;
+  if constexpr (!RB) {
+    if (L.tile == TILE_LONG)
+      return launch_pdl(kg_march_down<T, MARCH_LONG>, dim3(L.grid), dim3(MARCH_THREADS), 0, st, a, LT, L.li);
+    if (L.tile == TILE_SHORT)
+      return launch_pdl(kg_march_down<T, MARCH_SHORT>, dim3(L.grid), dim3(MARCH_THREADS), 0, st, a, LT, L.li);
+  }
   if (L.tile == TILE_BIG)
     launch_pdl(kg_down2d<T, RB, DN_CX, DN_CY, FUSED_THREADS>, dim3(L.grid), dim3(FUSED_THREADS), 0, st, a, LT, L.li);
   else if (L.tile == TILE_TINY)
@@ -1039,6 +1136,12 @@ static void group_down_launch(const GroupVcycle::Launch& L, const GroupList* LT,
 template <typename T, bool RB, typename TO>
 static void group_up_launch(const GroupVcycle::Launch& L, const GroupList* LT, cudaStream_t st) {
   const GUp<T>* a = (const GUp<T>*)L.args;
+  if constexpr (!RB) {
+    if (L.tile == TILE_LONG)
+      return launch_pdl(kg_march_up<T, TO, MARCH_LONG>, dim3(L.grid), dim3(MARCH_THREADS), 0, st, a, LT, L.li);
+    if (L.tile == TILE_SHORT)
+      return launch_pdl(kg_march_up<T, TO, MARCH_SHORT>, dim3(L.grid), dim3(MARCH_THREADS), 0, st, a, LT, L.li);
+  }
   if (L.tile == TILE_BIG)
     launch_pdl(kg_up2d<T, RB, TO, UP_FX, UP_FY, FUSED_THREADS>, dim3(L.grid), dim3(FUSED_THREADS), 0, st, a, LT, L.li);
   else if (L.tile == TILE_TINY)
@@ -1196,7 +1299,7 @@ static helm_status autotune_t(helm_ctx* c, cudaStream_t st) {
     for (int l = 0; l < nl - 1; ++l) {
       if (c->lv[l].stg64) continue;  // Galerkin levels do not run the fused kernels
       auto it = g_tune.find(std::make_tuple((int)sizeof(T), (int)RB, c->lv[l].n[0], c->lv[l].n[1]));
-      auto valid = [](int t) { return t >= 0 && t < NUM_TILES; };
+      auto valid = [](int t) { return t >= 0 && t < (RB ? TILE_LONG : NUM_TILES); };
       if (it != g_tune.end() && valid(it->second.first) && valid(it->second.second)) {
         c->lv[l].tile_down = it->second.first;
         c->lv[l].tile_up = it->second.second;
@@ -1242,7 +1345,8 @@ static helm_status autotune_t(helm_ctx* c, cudaStream_t st) {
     const LevelHost& C = c->lv[l + 1];
     int best_d = TILE_BIG, best_u = TILE_BIG;
     float td = 1e30f, tu = 1e30f;
-    for (int tile : {TILE_BIG, TILE_SMALL, TILE_TINY, TILE_SQUARE, TILE_WIDE}) {
+    for (int tile : {TILE_BIG, TILE_SMALL, TILE_TINY, TILE_SQUARE, TILE_WIDE, TILE_LONG, TILE_SHORT}) {
+      if (RB && (tile == TILE_LONG || tile == TILE_SHORT)) continue;
       float a = time_variant([&] { down_tile<T, RB>(tile, F, C, f, u, fc, om, nullptr, st); }, st, e0, e1);
       float b = time_variant([&] { up_tile<T, RB, T>(tile, F, C, u, fc, f, (T*)o, om, nullptr, st); }, st, e0, e1);
       if (a < td) { td = a; best_d = tile; }

@@ -71,3 +71,55 @@ def test_ilu_strips(shape, mg, galerkin):
         d = u.cpu().numpy() - ref
         assert np.linalg.norm(d) <= tol * np.linalg.norm(ref) and np.max(np.abs(d)) <= tol * np.max(np.abs(ref))
     h.close()
+
+
+@pytest.mark.parametrize("mg", ["c64", "c128"])
+@pytest.mark.parametrize("tile", [5, 6])
+@pytest.mark.parametrize("shape", [(62, 47), (122, 33), (121, 64), (242, 35), (243, 70), (300, 131)])
+def test_row_walking_kernels(shape, tile, mg, tmp_path):
+    """The row-walking kernels of damped-Jacobi levels (forced through the tuner's cache file) where their
+    split can go wrong: one strip and several, odd sizes, blocks cut short at either end; the V-cycle
+    against the oracle's, complex64 and (narrowed on the way in) complex128 right-hand sides alike."""
+    import os
+    import subprocess
+    import sys
+    n = [s - 2 for s in shape]
+    b = 4 if mg == "c64" else 8
+    lines, m = [], list(n)
+    while min(m) >= 3 and max(m) > 8:
+        lines.append(f"tile {b} 0 {m[0]} {m[1]} {tile} {tile}")
+        m = [v // 2 for v in m]
+    lines.append(f"depth {b} 4 2 {n[0]} {n[1]} 1 {len(lines) + 1} 1")  # the tail begins below the finest level
+    path = tmp_path / "tune"
+    path.write_text("\n".join(lines) + "\n")
+    code = f"""
+import numpy as np, torch, helm_inputs as hi
+from oracle import Oracle
+from paper_0912_0180_gb300.helm import Helm
+p = hi.make_problem(2, {shape!r}, 0, k0=30.0, phi_kind="bump", rhs="zero", bump_centre=(0.3, 0.6))
+pc = hi.Precond(kind=hi.PC_CSG_UNIFORM, theta_beta=0.3, smoother=hi.SM_JACOBI, omega=0.5)
+r = hi.random_vector(p.n, 41)
+ref = Oracle(p, pc).vcycle(r)
+h = Helm(p, pc, mg_dtype={mg!r})
+z = h.vcycle(torch.from_numpy(r).cuda()).cpu().numpy()
+tol = 1e-10 if {mg!r} == "c128" else 5e-5
+assert np.linalg.norm(z - ref) <= tol * np.linalg.norm(ref), np.linalg.norm(z - ref) / np.linalg.norm(ref)
+assert np.max(np.abs(z - ref)) <= tol * np.max(np.abs(ref))
+import paper_0912_0180_gb300._lib as L
+o = Oracle(p, pc)
+dt = torch.complex64 if {mg!r} == "c64" else torch.complex128
+f = hi.random_vector(p.n, 42).astype(np.complex64)
+u = torch.zeros(p.n, dtype=dt, device="cuda")
+fc = torch.zeros(o.level_size(1, 1), dtype=dt, device="cuda")
+h.level_op(L.HELM_OP_DOWN, 0, u, torch.from_numpy(f).cuda().to(dt), fc)
+f = f.astype(np.complex128)
+u_ref = o.smooth(0, np.zeros(p.n), f, 1)
+fc_ref = o.restrict(0, f - o.apply(u_ref, 1, 0))
+for got, want, t in ((u, u_ref, tol), (fc, fc_ref, 10 * tol)):
+    d = got.cpu().numpy() - want
+    assert np.linalg.norm(d) <= t * np.linalg.norm(want) and np.max(np.abs(d)) <= t * np.max(np.abs(want))
+"""
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    out = subprocess.run([sys.executable, "-c", code], cwd=root, env=dict(os.environ, HELM_TUNE_CACHE=str(path)),
+                         capture_output=True, text=True)
+    assert out.returncode == 0, out.stderr[-2000:]
