@@ -14,6 +14,7 @@
 // which is already Hessenberg), eigenvectors by back substitution on the triangular factor, V^{-1}
 // by Gauss-Jordan with partial pivoting.  The decomposition is used only if it reproduces T_a
 // (||T V - V Lambda|| and ||V V^{-1} - I|| below 1e-11 relative); otherwise the dense inverse is built.
+#include <algorithm>
 #include <cmath>
 #include <complex>
 #include <vector>
@@ -218,6 +219,74 @@ __global__ void k_fdm_axis(const cx<T>* __restrict__ in, cx<T>* __restrict__ out
   out[p] = acc;
 }
 
+// The same transforms in three launches instead of six (FP32, 3D, planes of at most FDM_PLANE points):
+// both in-plane transforms of a plane in one block, the plane in shared memory; the z transform, the
+// scaling and the z transform back of 16 columns in one block.  A launch of the six cost its latency (4
+// to 7 us for 20^3 points); in FP64 one SM's two lanes would need longer for a plane than the launches.
+// Every sum is k_fdm_axis's.
+constexpr int FDM_PLANE = 1024, FDM_COLS = 16;
+template <typename T>
+__global__ void __launch_bounds__(FDM_PLANE) k_fdm_plane(const cx<T>* __restrict__ in, cx<T>* __restrict__ out,
+                                                         const cx<T>* __restrict__ A, const cx<T>* __restrict__ B, int n0,
+                                                         int n1, int y_first, const int* skip) {
+  extern __shared__ __align__(16) unsigned char fdm_sm[];
+  cx<T>* const a = reinterpret_cast<cx<T>*>(fdm_sm);  // the x matrix, the y matrix, the plane and its transform
+  cx<T>* const b = a + n0 * n0;
+  cx<T>* const s = b + n1 * n1;
+  cx<T>* const w = s + n0 * n1;
+  for (int q = threadIdx.x; q < n0 * n0; q += blockDim.x) a[q] = A[q];
+  for (int q = threadIdx.x; q < n1 * n1; q += blockDim.x) b[q] = B[q];
+  pdl_entry();
+  if (skip && *skip) return;
+  const int np = n0 * n1, p = threadIdx.x, i = p % n0, j = p / n0;
+  const long base = (long)blockIdx.x * np;
+  if (p < np) s[p] = in[base + p];
+  __syncthreads();
+  for (int pass = 0; pass < 2; ++pass) {
+    const bool y = (pass == 0) == (y_first != 0);
+    const cx<T>* src = pass ? w : s;
+    cx<T> acc = mkc<T>(T(0), T(0));
+    if (p < np) {
+      if (y) {
+#pragma unroll 4
+        for (int m = 0; m < n1; ++m) acc = cfma<T>(b[j * n1 + m], src[i + m * n0], acc);
+      } else {
+#pragma unroll 4
+        for (int m = 0; m < n0; ++m) acc = cfma<T>(a[i * n0 + m], src[j * n0 + m], acc);
+      }
+      if (pass) out[base + p] = acc;
+      else w[p] = acc;
+    }
+    __syncthreads();
+  }
+}
+template <typename T>
+__global__ void k_fdm_cols(const cx<T>* __restrict__ in, cx<T>* __restrict__ out, const cx<T>* __restrict__ Vi,
+                           const cx<T>* __restrict__ V, const cx<T>* __restrict__ dsc, int np, int n2, const int* skip) {
+  extern __shared__ __align__(16) unsigned char fdm_sm[];
+  cx<T>* const s = reinterpret_cast<cx<T>*>(fdm_sm);  // [n2][FDM_COLS]
+  cx<T>* const w = s + n2 * FDM_COLS;
+  pdl_entry();
+  if (skip && *skip) return;
+  const int c = threadIdx.x, p = blockIdx.x * FDM_COLS + c;
+  for (int l = threadIdx.y; l < n2; l += blockDim.y)
+    if (p < np) s[l * FDM_COLS + c] = in[p + (long)l * np];
+  __syncthreads();
+  for (int l = threadIdx.y; l < n2; l += blockDim.y) {
+    cx<T> acc = mkc<T>(T(0), T(0));
+#pragma unroll 4
+    for (int m = 0; m < n2; ++m) acc = cfma<T>(Vi[l * n2 + m], s[m * FDM_COLS + c], acc);
+    if (p < np) w[l * FDM_COLS + c] = cmul<T>(acc, dsc[p + (long)l * np]);
+  }
+  __syncthreads();
+  for (int l = threadIdx.y; l < n2; l += blockDim.y) {
+    cx<T> acc = mkc<T>(T(0), T(0));
+#pragma unroll 4
+    for (int m = 0; m < n2; ++m) acc = cfma<T>(V[l * n2 + m], w[m * FDM_COLS + c], acc);
+    if (p < np) out[p + (long)l * np] = acc;
+  }
+}
+
 // z = M^{-1} f on the coarsest level: forward transforms (V_a^{-1}) along every axis, the scaling,
 // and the transforms back (V_a), ping-ponging through two scratch vectors.
 template <typename T>
@@ -227,6 +296,21 @@ void fdm_apply(const helm_ctx* c, const cx<T>* f, cx<T>* z, const int* skip, cud
   const long ntot = (long)F.n[0] * F.n[1] * F.n[2];
   const int thr = 256, blocks = (int)((ntot + thr - 1) / thr);
   cx<T>* s[2] = {(cx<T>*)F.scr, (cx<T>*)F.scr + ntot};
+  if constexpr (sizeof(T) == 4) {
+    const int n0 = F.n[0], n1 = F.n[1], n2 = F.n[2], np = n0 * n1;
+    const size_t plane = sizeof(cx<T>) * ((size_t)n0 * n0 + (size_t)n1 * n1 + 2 * (size_t)np);
+    const size_t cols = sizeof(cx<T>) * 2 * (size_t)n2 * FDM_COLS;
+    if (d == 3 && np <= FDM_PLANE && plane <= 48 * 1024 && cols <= 48 * 1024) {
+      const int pt = (np + 31) / 32 * 32;
+      launch_pdl(k_fdm_plane<T>, dim3(n2), dim3(pt), plane, st, f, s[0], (const cx<T>*)F.Vi[0], (const cx<T>*)F.Vi[1], n0,
+                 n1, 0, skip);
+      launch_pdl(k_fdm_cols<T>, dim3((np + FDM_COLS - 1) / FDM_COLS), dim3(FDM_COLS, std::min(n2, 32)), cols, st,
+                 (const cx<T>*)s[0], s[1], (const cx<T>*)F.Vi[2], (const cx<T>*)F.V[2], (const cx<T>*)F.dinv, np, n2, skip);
+      launch_pdl(k_fdm_plane<T>, dim3(n2), dim3(pt), plane, st, (const cx<T>*)s[1], z, (const cx<T>*)F.V[0],
+                 (const cx<T>*)F.V[1], n0, n1, 1, skip);
+      return;
+    }
+  }
   const cx<T>* src = f;
   int k = 0;
   for (int a = 0; a < d; ++a) {  // forward

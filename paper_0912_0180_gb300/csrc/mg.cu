@@ -156,12 +156,15 @@ __global__ void k_rbgs(OpView<T> op, cx<T>* __restrict__ u, const cx<T>* __restr
 // end lane's x neighbour, V(p + 2)) is issued before plane p is computed: they read the other
 // colour or read-only data, which this half-sweep never writes.  IDX: the offset type (int when
 // N < 2^31).
-template <typename T, bool RESID, bool WIDE, int W, typename IDX>
+template <typename T, bool RESID, typename TW, int W, typename IDX>
 __global__ void __launch_bounds__(128) k_rbgs3z(OpView<T> op, cx<T>* __restrict__ u, const cx<T>* __restrict__ f,
                                                 cx<T>* __restrict__ r, int colour, int lz,
-                                                double2* __restrict__ wide, const int* skip) {
+                                                void* __restrict__ wide_, const int* skip) {
   pdl_entry();
   if (skip && *skip) return;
+  constexpr bool WIDE = !std::is_void<TW>::value;
+  using TO = typename std::conditional<WIDE, TW, T>::type;
+  cx<TO>* __restrict__ const wide = (cx<TO>*)wide_;
   constexpr int SEGS = 32 / W;  // rows per warp
   const int n0 = op.n[0], n1 = op.n[1], n2 = op.n[2];
   const int h = (n0 + 1) >> 1;
@@ -255,13 +258,13 @@ __global__ void __launch_bounds__(128) k_rbgs3z(OpView<T> op, cx<T>* __restrict_
         r[pc] = mkc<T>(-off.x, -off.y);
       } else {
         const cx<T> v = cmul<T>(csub<T>(f0, off), d0);
-        u[pc] = v;
-        if (WIDE) wide[rowoff + 2 * t + C + o] = cconv<double, T>(v);
+        if (WIDE) wide[rowoff + 2 * t + C + o] = cconv<TO, T>(v);
+        else u[pc] = v;
       }
     }
     if (ho) {
       if (RESID) r[po] = zero;
-      else if (WIDE) wide[rowoff + 2 * t + 1 - C + o] = cconv<double, T>(v0);
+      else if (WIDE) wide[rowoff + 2 * t + 1 - C + o] = cconv<TO, T>(v0);
     }
     vm = v0;
     v0 = vp;
@@ -301,12 +304,15 @@ __device__ __forceinline__ void st_x2(float2* p, float2 a, float2 b) {
 // 16-byte access is aligned when the arrays are.  The per-point arithmetic is k_rbgs3z's, operation
 // for operation.  A row is a segment of W lanes (4, 8 or 16); the rows of a warp are blockDim.y
 // apart (even), so the colour's column is uniform over the warp.
-template <bool RESID, bool WIDE, int W, typename IDX>
+template <bool RESID, typename TW, int W, typename IDX>
 __global__ void __launch_bounds__(128) k_rbgs3z2(OpView<float> op, float2* __restrict__ u,
                                                  const float2* __restrict__ f, float2* __restrict__ r,
-                                                 int colour, int lz, double2* __restrict__ wide,
+                                                 int colour, int lz, void* __restrict__ wide_,
                                                  const int* skip) {
   using T = float;
+  constexpr bool WIDE = !std::is_void<TW>::value;
+  using TO = typename std::conditional<WIDE, TW, T>::type;
+  cx<TO>* __restrict__ const wide = (cx<TO>*)wide_;
   pdl_entry();
   if (skip && *skip) return;
   constexpr int SEGS = 32 / W;  // rows per warp
@@ -418,13 +424,14 @@ __global__ void __launch_bounds__(128) k_rbgs3z2(OpView<float> op, float2* __res
         st_x2(r + (C ? ce : co) + o, zero, zero);  // the other colour's points
       } else {
         const float2 va = cmul<T>(csub<T>(f0.a, oa), d0.a), vb = cmul<T>(csub<T>(f0.b, ob), d0.b);
-        st_x2(u + pc, va, vb);
         if (WIDE) {
-          double2* w = wide + rowoff + x0 + o;
-          w[C] = cconv<double, T>(va);
-          w[1 - C] = cconv<double, T>(v0.a);
-          w[2 + C] = cconv<double, T>(vb);
-          w[3 - C] = cconv<double, T>(v0.b);
+          cx<TO>* w = wide + rowoff + x0 + o;
+          w[C] = cconv<TO, T>(va);
+          w[1 - C] = cconv<TO, T>(v0.a);
+          w[2 + C] = cconv<TO, T>(vb);
+          w[3 - C] = cconv<TO, T>(v0.b);
+        } else {
+          st_x2(u + pc, va, vb);
         }
       }
     }
@@ -762,12 +769,132 @@ __global__ void __launch_bounds__(128) k_restrict3z(Dims d, const cx<T>* __restr
   }
 }
 
+// Residual after the zero-guess red-black sweep and its full weighting in one pass (x-split levels,
+// coarsening offset 1): the residual is zero on black points and -offdiag(u) on red ones, so a coarse
+// value needs the black points around it only, and the residual itself never goes to memory.  A lane
+// owns the fine pair (2t, 2t + 1) -- coarse column t -- of the fine rows 2J .. 2J + 2 and walks the
+// planes; V(k, p) is the black value of its pair in row 2J - 1 + k, plane p.  Per point the arithmetic
+// is that of the RESID sweep and of k_restrict, so the result is bitwise theirs (the products' fused
+// forms spelled out as the compiler chose them there).  30 coarse columns a
+// warp (the outer lanes are the halo).  With u_c it also runs the red half of the coarse level's sweep
+// from the zero guess, whose f it has just made.
+template <typename IDX>
+__global__ void __launch_bounds__(128) k_resrest3z(OpView<float> op, Dims d, const float2* __restrict__ u,
+                                                   float2* __restrict__ fc, int lz, const float2* __restrict__ dinv_c,
+                                                   float2* __restrict__ u_c, const int* skip) {
+  using T = float;
+  pdl_entry();
+  if (skip && *skip) return;
+  const int n0 = op.n[0], n1 = op.n[1], n2 = op.n[2], h = (n0 + 1) >> 1;
+  const int lane = threadIdx.x, t = blockIdx.x * 30 + lane - 1;
+  const int J = blockIdx.y * blockDim.y + threadIdx.y;
+  const int L0 = blockIdx.z * lz, L1 = min(L0 + lz, d.c[2]);
+  if (J >= d.c[1]) return;  // the whole warp
+  const float2 zero = make_float2(0.f, 0.f);
+  const bool has0 = t >= 0 && 2 * t < n0, has1 = t >= 0 && 2 * t + 1 < n0;
+  const float2 axm0 = has0 ? op.am[0][2 * t] : zero, axp0 = has0 ? op.ap[0][2 * t] : zero;
+  const float2 axm1 = has1 ? op.am[0][2 * t + 1] : zero, axp1 = has1 ? op.ap[0][2 * t + 1] : zero;
+  float2 aym[3], ayp[3];
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    const bool in = 2 * J + k < n1;
+    aym[k] = in ? op.am[1][2 * J + k] : zero;
+    ayp[k] = in ? op.ap[1][2 * J + k] : zero;
+  }
+  const IDX P = (IDX)n0 * n1;
+  const IDX row0 = (IDX)n0 * (2 * J - 1);
+  auto V = [&](int k, int p) -> float2 {
+    const int y = 2 * J - 1 + k;
+    if (y < 0 || y >= n1 || p < 0 || p >= n2) return zero;
+    const bool odd = !((y + p) & 1);  // the black column
+    if (!(odd ? has1 : has0)) return zero;
+    return u[row0 + (IDX)k * n0 + (IDX)p * P + (odd ? h + t : t)];
+  };
+  float2 vm[3], v0[5], vp[3], vpp[3];
+  int p = 2 * L0;
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    vm[k] = V(k + 1, p - 1);
+    vp[k] = V(k + 1, p + 1);
+  }
+#pragma unroll
+  for (int k = 0; k < 5; ++k) v0[k] = V(k, p);
+  // the row-and-column weighted residual of plane p, whose rows' red columns are pe, 1 - pe, pe
+  auto plane = [&](auto pe_) -> float2 {
+    constexpr int pe = decltype(pe_)::value;
+    // the next plane's outer rows and the one after it
+    const float2 o0 = V(0, p + 1), o4 = V(4, p + 1);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) vpp[k] = V(k + 1, p + 2);
+    float2 sum = zero;
+    if (p < n2) {
+      const float2 azm = op.am[2][p], azp = op.ap[2][p];
+      float2 rs[3];
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        const int C = (k & 1) ? 1 - pe : pe;
+        const float2 v = v0[k + 1];
+        float2 xo;
+        if (C == 0) {
+          xo.x = __shfl_up_sync(0xffffffffu, v.x, 1);
+          xo.y = __shfl_up_sync(0xffffffffu, v.y, 1);
+        } else {
+          xo.x = __shfl_down_sync(0xffffffffu, v.x, 1);
+          xo.y = __shfl_down_sync(0xffffffffu, v.y, 1);
+        }
+        float2 off = cmul1<T>(C ? axm1 : axm0, C ? v : xo);
+        off = cfma<T>(C ? axp1 : axp0, C ? xo : v, off);
+        off = cfma<T>(aym[k], v0[k], off);
+        off = cfma<T>(ayp[k], v0[k + 2], off);
+        off = cfma<T>(azm, vm[k], off);
+        off = cfma<T>(azp, vp[k], off);
+        float2 r = (C ? has1 : has0) && 2 * J + k < n1 ? make_float2(-off.x, -off.y) : zero;
+        if (C == 0) {  // columns 2t and 2t + 2
+          const float2 rn = make_float2(__shfl_down_sync(0xffffffffu, r.x, 1), __shfl_down_sync(0xffffffffu, r.y, 1));
+          rs[k] = cadd<T>(r, rn);
+        } else {
+          rs[k] = make_float2(2.f * r.x, 2.f * r.y);
+        }
+      }
+      sum = make_float2(fmaf(2.f, rs[1].x, rs[0].x + rs[2].x), fmaf(2.f, rs[1].y, rs[0].y + rs[2].y));
+    }
+    v0[0] = o0;
+    v0[4] = o4;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      vm[k] = v0[k + 1];
+      v0[k + 1] = vp[k];
+      vp[k] = vpp[k];
+    }
+    ++p;
+    return sum;
+  };
+  float2 prev = plane(std::integral_constant<int, 0>());
+  const bool own = lane >= 1 && lane <= 30 && t < d.c[0];
+  const IDX cq = (IDX)(own ? xpos(t, d.ch) : 0) + (IDX)d.c[0] * J, CP = (IDX)d.c[0] * d.c[1];
+  for (int L = L0; L < L1; ++L) {
+    const bool red = own && u_c && !((t + J + L) & 1);
+    const float2 di = red ? dinv_c[cq + CP * L] : zero;
+    const float2 mid = plane(std::integral_constant<int, 1>()), last = plane(std::integral_constant<int, 0>());
+    const float2 acc = make_float2(fmaf(2.f, mid.x, prev.x + last.x), fmaf(2.f, mid.y, prev.y + last.y));
+    if (own) {
+      const float2 v = cscale<T>(0.015625f, acc);
+      fc[cq + CP * L] = v;
+      // the coarse level's zero-guess red half-sweep
+      if (red) u_c[cq + CP * L] = cmul1<T>(di, v);
+    }
+    prev = last;
+  }
+}
+
 // Trilinear prolongation onto an x-split fine level: thread (t, j) owns the fine pair (2t, 2t + 1)
 // of row j and walks fine planes [l0, l1).  The pair reads coarse columns a = t - o and a + 1, the
 // row coarse rows jA (and jB); the coarse values of the two coarse planes a fine plane can need
 // stay in registers.  Every fine point sums its coarse values in k_prolong's order (lower plane,
 // row, column first) and scales once.
-template <typename T, typename IDX>
+// BLACK: only the black points, before a red-black sweep (whose red half overwrites the red points from
+// the black ones): half the bytes and sums.
+template <typename T, typename IDX, bool BLACK>
 __global__ void __launch_bounds__(128) k_prolong3z(Dims d, const cx<T>* __restrict__ ec, cx<T>* __restrict__ u,
                                                    int overwrite, int lz, const int* skip) {
   pdl_entry();
@@ -825,6 +952,12 @@ __global__ void __launch_bounds__(128) k_prolong3z(Dims d, const cx<T>* __restri
   };
   const IDX P = (IDX)d.f[0] * d.f[1];
   const IDX ce = (IDX)d.f[0] * j + t, co = (IDX)d.f[0] * j + d.fh + t;
+  // BLACK: the black value of plane l (a thread's planes are a chain: read two planes ahead)
+  auto black = [&](int l) -> cx<T> {
+    const bool odd = !((j + l) & 1);
+    return !BLACK || overwrite || l >= l1 || (odd && !has1) ? zero : u[(odd ? co : ce) + (IDX)l * P];
+  };
+  cx<T> ub = black(l0), ub1 = black(l0 + 1);
   int rz = l0 - d.o[2];
   int Lc = rz >> 1;  // floor
   Cp A = load_plane(Lc), B = load_plane(Lc + 1);
@@ -837,6 +970,19 @@ __global__ void __launch_bounds__(128) k_prolong3z(Dims d, const cx<T>* __restri
     const bool zon = !(rz & 1);  // on coarse plane Lc; otherwise between Lc and Lc + 1
     const T wz = zon ? T(1) : T(0.5);
     const IDX oe = ce + (IDX)l * P, oo = co + (IDX)l * P;
+    if (BLACK) {
+      const bool odd = !((j + l) & 1);  // the black column of the pair
+      const cx<T> uo = ub;
+      ub = ub1;
+      ub1 = black(l + 2);
+      if (odd && !has1) continue;
+      const cx<T> sb = odd ? point(A, B, !zon, true) : point(A, B, !zon, false);
+      const T w = (odd ? wxo : wxe) * wy * wz;
+      const IDX o = odd ? oo : oe;
+      if (overwrite) u[o] = cscale<T>(w, sb);
+      else u[o] = mkc<T>(fma(w, sb.x, uo.x), fma(w, sb.y, uo.y));
+      continue;
+    }
     const cx<T> se = point(A, B, !zon, false);
     const T we = wxe * wy * wz;
     if (overwrite) u[oe] = cscale<T>(we, se);
@@ -927,7 +1073,7 @@ static void xs_convert(const LevelHost& L, const cx<TI>* a, cx<TO>* b, bool to_x
 
 template <typename T>
 static void vcycle_unfused(helm_ctx* c, int l, const cx<T>* f, cx<T>* out, const int* skip, cudaStream_t st,
-                           double2* wide = nullptr);
+                           double2* wide = nullptr, float2* nat = nullptr, bool red_done = false);
 
 // a Galerkin level: 9-point in 2D, 27-point in 3D
 template <typename T> static bool is9(const LevelHost& L) { return L.stg64 != nullptr; }
@@ -941,38 +1087,45 @@ static int plane_chunk(long warps, int nz) {
   return lz;
 }
 
+// where the last sweep of a cycle writes the whole iterate in natural order instead of its own points
+// in storage order: complex128 (f64) or, on x-split levels, complex64
+struct NatOut {
+  void* p = nullptr;
+  bool f64 = true;
+  NatOut() = default;
+  NatOut(double2* w) : p(w) {}
+  explicit NatOut(float2* w) : p(w), f64(false) {}
+};
+
 // the z-marching sweep: row segments of 32 or 16 pairs (whichever idles fewer lanes), 4 warps a
 // block
-template <typename T, bool RESID, bool WIDE, int W, typename IDX>
-static void launch_rbgs3z_g(const LevelHost& L, cx<T>* u, const cx<T>* f, cx<T>* r, int colour, double2* wide,
-                            const int* skip, cudaStream_t st);
-template <typename T, bool RESID, int W, typename IDX>
-static void launch_rbgs3z_w(const LevelHost& L, cx<T>* u, const cx<T>* f, cx<T>* r, int colour, double2* wide,
-                            const int* skip, cudaStream_t st) {
-  if (wide) {
-    launch_rbgs3z_g<T, RESID, true, W, IDX>(L, u, f, r, colour, wide, skip, st);
-    return;
-  }
-  launch_rbgs3z_g<T, RESID, false, W, IDX>(L, u, f, r, colour, wide, skip, st);
-}
-template <typename T, bool RESID, bool WIDE, int W, typename IDX>
-static void launch_rbgs3z_g(const LevelHost& L, cx<T>* u, const cx<T>* f, cx<T>* r, int colour, double2* wide,
+template <typename T, bool RESID, typename TW, int W, typename IDX>
+static void launch_rbgs3z_g(const LevelHost& L, cx<T>* u, const cx<T>* f, cx<T>* r, int colour, void* wide,
                             const int* skip, cudaStream_t st) {
   const int h = (L.n[0] + 1) / 2;
   const int rows_per_block = 4 * (32 / W);
   const long gx = (h + W - 1) / W, gy = (L.n[1] + rows_per_block - 1) / rows_per_block;
   const int lz = plane_chunk(gx * gy * 4, L.n[2]);
   dim3 g((unsigned)gx, (unsigned)gy, (unsigned)((L.n[2] + lz - 1) / lz));
-  launch_pdl(k_rbgs3z<T, RESID, WIDE, W, IDX>, g, dim3(32, 4), 0, st, L.view<T>(), u, f, r, colour, lz, wide, skip);
+  launch_pdl(k_rbgs3z<T, RESID, TW, W, IDX>, g, dim3(32, 4), 0, st, L.view<T>(), u, f, r, colour, lz, wide, skip);
+}
+template <typename T, bool RESID, int W, typename IDX>
+static void launch_rbgs3z_w(const LevelHost& L, cx<T>* u, const cx<T>* f, cx<T>* r, int colour, NatOut wide,
+                            const int* skip, cudaStream_t st) {
+  if constexpr (!RESID) {
+    if (wide.p && wide.f64) return launch_rbgs3z_g<T, RESID, double, W, IDX>(L, u, f, r, colour, wide.p, skip, st);
+    if (wide.p) return launch_rbgs3z_g<T, RESID, float, W, IDX>(L, u, f, r, colour, wide.p, skip, st);
+  }
+  launch_rbgs3z_g<T, RESID, void, W, IDX>(L, u, f, r, colour, nullptr, skip, st);
 }
 // k_rbgs3z2: W lanes (two pairs each) per row segment, whichever of 16, 8, 4 idles the fewest
 // lanes; blockDim.y = 4 or 2 rows, whichever idles fewer; planes per thread: the fewest that still
 // fit the grid in one wave of resident blocks (a thread's planes run one after another, so the
 // kernel lasts about one chain of planes)
-template <bool RESID, bool WIDE, int W, typename IDX>
-static void launch_rbgs3z2_g(const LevelHost& L, float2* u, const float2* f, float2* r, int colour, double2* wide,
+template <bool RESID, typename TW, int W, typename IDX>
+static void launch_rbgs3z2_g(const LevelHost& L, float2* u, const float2* f, float2* r, int colour, void* wide,
                              const int* skip, cudaStream_t st) {
-  auto kern = k_rbgs3z2<RESID, WIDE, W, IDX>;
+  auto kern = k_rbgs3z2<RESID, TW, W, IDX>;
   const int h = L.n[0] / 2;
   const int segs = 32 / W;
   const int by4 = (L.n[1] + 4 * segs - 1) / (4 * segs) * 4 * segs, by2 = (L.n[1] + 2 * segs - 1) / (2 * segs) * 2 * segs;
@@ -993,13 +1146,16 @@ static void launch_rbgs3z2_g(const LevelHost& L, float2* u, const float2* f, flo
   launch_pdl(kern, g, dim3(32, by), 0, st, L.view<float>(), u, f, r, colour, lz, wide, skip);
 }
 template <bool RESID, int W, typename IDX>
-static void launch_rbgs3z2_w(const LevelHost& L, float2* u, const float2* f, float2* r, int colour, double2* wide,
+static void launch_rbgs3z2_w(const LevelHost& L, float2* u, const float2* f, float2* r, int colour, NatOut wide,
                              const int* skip, cudaStream_t st) {
-  if (wide) launch_rbgs3z2_g<RESID, true, W, IDX>(L, u, f, r, colour, wide, skip, st);
-  else launch_rbgs3z2_g<RESID, false, W, IDX>(L, u, f, r, colour, wide, skip, st);
+  if constexpr (!RESID) {
+    if (wide.p && wide.f64) return launch_rbgs3z2_g<RESID, double, W, IDX>(L, u, f, r, colour, wide.p, skip, st);
+    if (wide.p) return launch_rbgs3z2_g<RESID, float, W, IDX>(L, u, f, r, colour, wide.p, skip, st);
+  }
+  launch_rbgs3z2_g<RESID, void, W, IDX>(L, u, f, r, colour, nullptr, skip, st);
 }
 template <bool RESID, typename IDX>
-static void launch_rbgs3z2(const LevelHost& L, float2* u, const float2* f, float2* r, int colour, double2* wide,
+static void launch_rbgs3z2(const LevelHost& L, float2* u, const float2* f, float2* r, int colour, NatOut wide,
                            const int* skip, cudaStream_t st) {
   const int h = L.n[0] / 2;
   const int p16 = (h + 31) / 32 * 32, p8 = (h + 15) / 16 * 16, p4 = (h + 7) / 8 * 8;
@@ -1016,7 +1172,7 @@ static bool rbgs3z2_fits(const LevelHost& L, const void* u, const void* f, const
 // x-split half-sweep or zero-guess residual: two pairs a thread where the row length and the
 // arrays allow, else one
 template <typename T, bool RESID>
-static void launch_rbgs3z(const LevelHost& L, cx<T>* u, const cx<T>* f, cx<T>* r, int colour, double2* wide,
+static void launch_rbgs3z(const LevelHost& L, cx<T>* u, const cx<T>* f, cx<T>* r, int colour, NatOut wide,
                           const int* skip, cudaStream_t st) {
   if constexpr (sizeof(cx<T>) == 8) {
     if (rbgs3z2_fits(L, u, f, r)) {
@@ -1050,13 +1206,13 @@ template <typename T, int DIM> struct Launch {
       launch_pdl(k_jacobi27<T>, dim3(g), dim3(b), 0, st, L.view<T>(), u, f, un, omega, wide, skip);
     else launch_pdl(k_jacobi<T, DIM>, dim3(g), dim3(b), 0, st, L.view<T>(), u, f, un, omega, wide, skip);
   }
-  static void rbgs(const LevelHost& L, cx<T>* u, const cx<T>* f, int colour, int zero, double2* wide,
+  static void rbgs(const LevelHost& L, cx<T>* u, const cx<T>* f, int colour, int zero, NatOut wide,
                    const int* skip, cudaStream_t st) {
     int half[3] = {(L.n[0] + 1) / 2, L.n[1], L.n[2]};
     dim3 g, b; rb_cfg<DIM>(half, g, b);
     if (DIM == 3 && L.xs && !zero) launch_rbgs3z<T, false>(L, u, f, nullptr, colour, wide, skip, st);
-    else if (DIM == 3 && L.xs) launch_pdl(k_rbgs<T, DIM, true>, dim3(g), dim3(b), 0, st, L.view<T>(), u, f, colour, zero, wide, skip);
-    else launch_pdl(k_rbgs<T, DIM>, dim3(g), dim3(b), 0, st, L.view<T>(), u, f, colour, zero, wide, skip);
+    else if (DIM == 3 && L.xs) launch_pdl(k_rbgs<T, DIM, true>, dim3(g), dim3(b), 0, st, L.view<T>(), u, f, colour, zero, (double2*)nullptr, skip);
+    else launch_pdl(k_rbgs<T, DIM>, dim3(g), dim3(b), 0, st, L.view<T>(), u, f, colour, zero, (double2*)wide.p, skip);
   }
   static void resid0(const LevelHost& L, const cx<T>* u, const cx<T>* f, cx<T>* r, T omega, bool rb, const int* skip,
                      cudaStream_t st) {
@@ -1064,7 +1220,7 @@ template <typename T, int DIM> struct Launch {
     dim3 g, b;
     if (rb) {
       rb_cfg<DIM>(half, g, b);
-      if (DIM == 3 && L.xs) launch_rbgs3z<T, true>(L, const_cast<cx<T>*>(u), nullptr, r, 0, nullptr, skip, st);
+      if (DIM == 3 && L.xs) launch_rbgs3z<T, true>(L, const_cast<cx<T>*>(u), nullptr, r, 0, NatOut(), skip, st);
       else launch_pdl(k_resid0<T, DIM, true>, dim3(g), dim3(b), 0, st, L.view<T>(), u, f, r, omega, skip);
     } else {
       cfg<DIM>(L.n, g, b);
@@ -1088,21 +1244,47 @@ template <typename T, int DIM> struct Launch {
     dim3 g, b; cfg<DIM>(C.n, g, b);
     launch_pdl(k_restrict<T, DIM>, dim3(g), dim3(b), 0, st, d, r, fc, skip);
   }
-  static void prolong(const LevelHost& F, const LevelHost& C, const cx<T>* ec, cx<T>* u, int overwrite, const int* skip, cudaStream_t st) {
+  static void prolong(const LevelHost& F, const LevelHost& C, const cx<T>* ec, cx<T>* u, int overwrite, const int* skip, cudaStream_t st,
+                      bool black = false) {
     Dims d; for (int a = 0; a < 3; ++a) { d.f[a] = F.n[a]; d.c[a] = C.n[a]; d.o[a] = F.offset(a); }
     d.fh = F.xs_half(); d.ch = C.xs_half();
     if (DIM == 3 && F.xs) {  // marching along z over the fine planes, one thread per fine pair
       const long gx = (d.fh + 31) / 32, gy = (F.n[1] + 3) / 4;
       const int lz = plane_chunk(gx * gy * 4, F.n[2]);
       dim3 g((unsigned)gx, (unsigned)gy, (unsigned)((F.n[2] + lz - 1) / lz));
-      if (F.ntot < 0x7fffffffL) launch_pdl(k_prolong3z<T, int>, g, dim3(32, 4), 0, st, d, ec, u, overwrite, lz, skip);
-      else launch_pdl(k_prolong3z<T, long>, g, dim3(32, 4), 0, st, d, ec, u, overwrite, lz, skip);
+      const bool i32 = F.ntot < 0x7fffffffL;
+      if (black && i32) launch_pdl(k_prolong3z<T, int, true>, g, dim3(32, 4), 0, st, d, ec, u, overwrite, lz, skip);
+      else if (black) launch_pdl(k_prolong3z<T, long, true>, g, dim3(32, 4), 0, st, d, ec, u, overwrite, lz, skip);
+      else if (i32) launch_pdl(k_prolong3z<T, int, false>, g, dim3(32, 4), 0, st, d, ec, u, overwrite, lz, skip);
+      else launch_pdl(k_prolong3z<T, long, false>, g, dim3(32, 4), 0, st, d, ec, u, overwrite, lz, skip);
       return;
     }
     dim3 g, b; cfg<DIM>(F.n, g, b);
     launch_pdl(k_prolong<T, DIM>, dim3(g), dim3(b), 0, st, d, ec, u, overwrite, skip);
   }
 };
+
+// residual and restriction of an x-split level in one launch, where k_resrest3z takes it
+// u_c: the coarse level's iterate, to start its zero-guess sweep (nullptr: not)
+static bool resrest3z(const LevelHost& F, const LevelHost& C, const float2* u, float2* fc, float2* u_c, const int* skip,
+                      cudaStream_t st) {
+  if (!F.xs || F.dim != 3 || F.stg64) return false;
+  Dims d;
+  for (int a = 0; a < 3; ++a) {
+    d.f[a] = F.n[a];
+    d.c[a] = C.n[a];
+    d.o[a] = F.offset(a);
+    if (d.o[a] != 1) return false;
+  }
+  d.fh = F.xs_half();
+  d.ch = C.xs_half();
+  const long gx = (C.n[0] + 29) / 30, gy = (C.n[1] + 3) / 4;
+  const int lz = plane_chunk(gx * gy * 4, C.n[2]);
+  dim3 g((unsigned)gx, (unsigned)gy, (unsigned)((C.n[2] + lz - 1) / lz));
+  if (F.ntot < 0x7fffffffL) launch_pdl(k_resrest3z<int>, g, dim3(32, 4), 0, st, F.view<float>(), d, u, fc, lz, (const float2*)C.dinv32, u_c, skip);
+  else launch_pdl(k_resrest3z<long>, g, dim3(32, 4), 0, st, F.view<float>(), d, u, fc, lz, (const float2*)C.dinv32, u_c, skip);
+  return true;
+}
 
 template <typename T> struct Ops {
   const LevelHost& L;
@@ -1119,7 +1301,7 @@ template <typename T> struct Ops {
     else Launch<T, 3>::jacobi(L, u, f, un, om, wide, skip, st);
   }
   void rbgs(cx<T>* u, const cx<T>* f, int colour, int zero, const int* skip, cudaStream_t st,
-            double2* wide = nullptr) const {
+            NatOut wide = NatOut()) const {
     if (dim == 1) Launch<T, 1>::rbgs(L, u, f, colour, zero, wide, skip, st);
     else if (dim == 2) Launch<T, 2>::rbgs(L, u, f, colour, zero, wide, skip, st);
     else Launch<T, 3>::rbgs(L, u, f, colour, zero, wide, skip, st);
@@ -1138,10 +1320,11 @@ static void restrict_any(const LevelHost& F, const LevelHost& C, const cx<T>* r,
   else Launch<T, 3>::restrict_(F, C, r, fc, skip, st);
 }
 template <typename T>
-static void prolong_any(const LevelHost& F, const LevelHost& C, const cx<T>* ec, cx<T>* u, int ow, const int* skip, cudaStream_t st) {
+static void prolong_any(const LevelHost& F, const LevelHost& C, const cx<T>* ec, cx<T>* u, int ow, const int* skip, cudaStream_t st,
+                        bool black = false) {
   if (F.dim == 1) Launch<T, 1>::prolong(F, C, ec, u, ow, skip, st);
   else if (F.dim == 2) Launch<T, 2>::prolong(F, C, ec, u, ow, skip, st);
-  else Launch<T, 3>::prolong(F, C, ec, u, ow, skip, st);
+  else Launch<T, 3>::prolong(F, C, ec, u, ow, skip, st, black);
 }
 template <typename T>
 static void coarse_solve(helm_ctx* c, const cx<T>* f, cx<T>* z, const int* skip, cudaStream_t st) {
@@ -1156,10 +1339,13 @@ static void coarse_solve(helm_ctx* c, const cx<T>* f, cx<T>* z, const int* skip,
 }
 
 // Smoothing sweeps on level L; buffers b[2] with *cur the index holding u.  zero: start from u = 0.
-// wide (optional): the last sweep also writes the result widened to complex128.
+// wide (optional): the last sweep also writes the result widened to complex128; nat (x-split levels):
+// it writes the result in natural order instead; red_done: whoever made f also ran the red half of the
+// sweep from the zero guess.
 template <typename T>
 static void smooth(helm_ctx* c, const LevelHost& L, cx<T>* b[2], int* cur, const cx<T>* f, int sweeps,
-                   bool zero, const int* skip, cudaStream_t st, double2* wide = nullptr) {
+                   bool zero, const int* skip, cudaStream_t st, double2* wide = nullptr, float2* nat = nullptr,
+                   bool red_done = false) {
   Ops<T> op{L, L.dim};
   for (int k = 0; k < sweeps; ++k) {
     bool z0 = zero && k == 0;
@@ -1170,8 +1356,8 @@ static void smooth(helm_ctx* c, const LevelHost& L, cx<T>* b[2], int* cur, const
     } else if (c->pc.smoother == HELM_SM_ILU) {
       ilu_smooth<T>(L, f, b[*cur], z0, w, skip, st);
     } else {
-      op.rbgs(b[*cur], f, 0, z0 ? 1 : 0, skip, st);
-      op.rbgs(b[*cur], f, 1, 0, skip, st, w);
+      if (!(z0 && red_done)) op.rbgs(b[*cur], f, 0, z0 ? 1 : 0, skip, st);
+      op.rbgs(b[*cur], f, 1, 0, skip, st, nat && k == sweeps - 1 ? NatOut(nat) : NatOut(w));
     }
   }
 }
@@ -1215,10 +1401,11 @@ static void vcycle_level(helm_ctx* c, int l, const cx<T>* f, void* out, bool out
 }
 
 // the one-kernel-per-component V-cycle on level l (below it, fused levels may take over); with
-// `wide` the result goes there as complex128 instead of to `out` (which is then scratch)
+// `wide` the result goes there as complex128 instead of to `out` (which is then scratch), with `nat`
+// (an x-split level) there in natural order
 template <typename T>
 static void vcycle_unfused(helm_ctx* c, int l, const cx<T>* f, cx<T>* out, const int* skip, cudaStream_t st,
-                           double2* wide) {
+                           double2* wide, float2* nat, bool red_done) {
   const LevelHost& L = c->lv[l];
   int nl = (int)c->lv.size();
   if (l == nl - 1) {
@@ -1233,18 +1420,30 @@ static void vcycle_unfused(helm_ctx* c, int l, const cx<T>* f, cx<T>* out, const
   int cur = jac ? ((pc.nu1 + pc.nu2) & 1) : 0;  // so that the last Jacobi sweep writes `out`
   Ops<T> op{L, L.dim};
   cx<T>* fc = (cx<T>*)C.f;
+  bool red_next = false;  // the coarse level's red half-sweep is done
   if (pc.nu1 > 0) {
-    smooth<T>(c, L, b, &cur, f, pc.nu1, true, skip, st);
+    smooth<T>(c, L, b, &cur, f, pc.nu1, true, skip, st, nullptr, nullptr, red_done);
+    bool done = false;
+    if constexpr (std::is_same<T, float>::value) {
+      float2* uc = C.xs && l + 1 < nl - 1 ? (float2*)C.u : nullptr;
+      done = pc.nu1 == 1 && pc.smoother == HELM_SM_RBGS && resrest3z(L, C, b[cur], fc, uc, skip, st);
+      red_next = done && uc;
+    }
     // residual into the spare buffer; after a single sweep from zero without the diagonal
-    if (pc.nu1 == 1 && pc.smoother != HELM_SM_ILU) op.resid0(b[cur], f, b[1 - cur], (T)pc.omega, !jac, skip, st);
-    else op.apply(b[cur], f, b[1 - cur], skip, st);
-    restrict_any<T>(L, C, b[1 - cur], fc, skip, st);
+    if (!done) {
+      if (pc.nu1 == 1 && pc.smoother != HELM_SM_ILU) op.resid0(b[cur], f, b[1 - cur], (T)pc.omega, !jac, skip, st);
+      else op.apply(b[cur], f, b[1 - cur], skip, st);
+      restrict_any<T>(L, C, b[1 - cur], fc, skip, st);
+    }
   } else {
     restrict_any<T>(L, C, f, fc, skip, st);
   }
-  vcycle_level<T>(c, l + 1, fc, C.u, false, skip, st);
-  prolong_any<T>(L, C, (const cx<T>*)C.u, b[cur], pc.nu1 > 0 ? 0 : 1, skip, st);
-  smooth<T>(c, L, b, &cur, f, pc.nu2, false, skip, st, wide);
+  if (red_next) vcycle_unfused<T>(c, l + 1, fc, (cx<T>*)C.u, skip, st, nullptr, nullptr, true);
+  else vcycle_level<T>(c, l + 1, fc, C.u, false, skip, st);
+  prolong_any<T>(L, C, (const cx<T>*)C.u, b[cur], pc.nu1 > 0 ? 0 : 1, skip, st,
+                 pc.smoother == HELM_SM_RBGS && pc.nu2 > 0);
+  smooth<T>(c, L, b, &cur, f, pc.nu2, false, skip, st, wide, nat);
+  if (nat && pc.nu2 == 0) xs_convert<T, float>(L, b[cur], nat, false, skip, st);
   if (wide && pc.nu2 == 0) {
     if (L.xs) xs_convert<float, double>(L, (const float2*)b[cur], wide, false, skip, st);
     else widen_c64(c, (const float2*)b[cur], wide, L.ntot, skip, st);
@@ -1254,12 +1453,10 @@ static void vcycle_unfused(helm_ctx* c, int l, const cx<T>* f, cx<T>* out, const
 template <typename T>
 helm_status mg_vcycle(helm_ctx* c, const cx<T>* f0, void* u0, bool u0_f64, const int* skip, cudaStream_t st) {
   const bool wide = u0_f64 && !std::is_same<T, double>::value;
-  vcycle_level<T>(c, 0, f0, u0, wide, skip, st);
   const LevelHost& L = c->lv[0];
-  if (L.xs && !wide) {  // an x-split result in the multigrid precision: back to natural order
-    HELM_CUDA(cudaMemcpyAsync(L.w, u0, sizeof(cx<T>) * L.ntot, cudaMemcpyDeviceToDevice, st));
-    xs_convert<T, T>(L, (const cx<T>*)L.w, (cx<T>*)u0, false, skip, st);
-  }
+  // an x-split result in the multigrid precision: the last sweep writes it in natural order
+  if (L.xs && !wide) vcycle_unfused<T>(c, 0, f0, (cx<T>*)c->scratch, skip, st, nullptr, (float2*)u0);
+  else vcycle_level<T>(c, 0, f0, u0, wide, skip, st);
   HELM_CUDA(cudaGetLastError());
   return HELM_OK;
 }
@@ -1280,6 +1477,25 @@ helm_status mg_input_from_c128(helm_ctx* c, const double2* in, void* out, cudaSt
   return HELM_OK;
 }
 
+// The complex64 x-split copy of a natural complex128 vector and the zero-guess red half-sweep on it, a
+// thread per pair of columns: 130 MB at 160^3 where the two passes moved 147, and one launch.
+__global__ void k_xs_in(const double2* __restrict__ a, float2* __restrict__ f, float2* __restrict__ u,
+                        const float2* __restrict__ dinv, int n0, int n1, long rows) {
+  pdl_entry();
+  const int t = blockIdx.x * blockDim.x + threadIdx.x, h = (n0 + 1) >> 1;
+  const long r = blockIdx.y + (long)gridDim.y * blockIdx.z;
+  if (2 * t >= n0 || r >= rows) return;
+  const long row = r * n0;
+  const bool odd = ((r % n1 + r / n1) & 1) != 0, has1 = 2 * t + 1 < n0;  // odd: the red column is 2t + 1
+  const float2 v0 = cconv<float, double>(a[row + 2 * t]);
+  float2 v1 = make_float2(0.f, 0.f);
+  if (has1) v1 = cconv<float, double>(a[row + 2 * t + 1]);
+  f[row + t] = v0;
+  if (has1) f[row + h + t] = v1;
+  const long q = row + (odd ? h + t : t);
+  if (!odd || has1) u[q] = cmul1<float>(dinv[q], odd ? v1 : v0);
+}
+
 helm_status mg_vcycle_from_c128(helm_ctx* c, const double2* r, void* buf, void* z, bool z64, cudaStream_t st) {
   if (fused_applies<float>(c, 0) && (c->tail_first > 0 || ctail_applies(c))) {
     if (c->tail_first == 0) return ctail_vcycle<float, double>(c, 0, r, z, z64, nullptr, st);
@@ -1287,6 +1503,19 @@ helm_status mg_vcycle_from_c128(helm_ctx* c, const double2* r, void* buf, void* 
     fused_down2d<float, double>(c, 0, r, (float2*)L.w, (float2*)C.f, nullptr, st);
     vcycle_level<float>(c, 1, (const float2*)C.f, C.u, false, nullptr, st);
     fused_up2d<float, double>(c, 0, (const float2*)L.w, (const float2*)C.u, r, z, z64, nullptr, st);
+    HELM_CUDA(cudaGetLastError());
+    return HELM_OK;
+  }
+  const LevelHost& L0 = c->lv[0];
+  if (L0.xs && c->pc.nu1 > 0) {  // (x-split levels smooth with red-black Gauss-Seidel)
+    const long rows = L0.ntot / L0.n[0];
+    const int gy = (int)std::min<long>(rows, 65535), h = (L0.n[0] + 1) / 2;
+    const int thr = std::min(128, (h + 31) / 32 * 32);
+    dim3 g((h + thr - 1) / thr, gy, (unsigned)((rows + gy - 1) / gy));
+    float2* u = (float2*)c->scratch;
+    launch_pdl(k_xs_in, g, dim3(thr), 0, st, r, (float2*)buf, u, (const float2*)L0.dinv32, L0.n[0], L0.n[1], rows);
+    vcycle_unfused<float>(c, 0, (const float2*)buf, u, nullptr, st, z64 ? (double2*)z : nullptr,
+                          z64 ? nullptr : (float2*)z, true);
     HELM_CUDA(cudaGetLastError());
     return HELM_OK;
   }

@@ -123,3 +123,23 @@ for got, want, t in ((u, u_ref, tol), (fc, fc_ref, 10 * tol)):
     out = subprocess.run([sys.executable, "-c", code], cwd=root, env=dict(os.environ, HELM_TUNE_CACHE=str(path)),
                          capture_output=True, text=True)
     assert out.returncode == 0, out.stderr[-2000:]
+
+
+@pytest.mark.parametrize("wide", [False, True])
+@pytest.mark.parametrize("shape,levels,kind", [((35, 20, 23), 2, "const"), ((22, 31, 28), 2, "const"), ((66, 33, 31), 32, "bump"),
+                                               ((63, 64, 29), 32, "bump"), ((11, 70, 35), 32, "const")])
+def test_xsplit_cycle_3d(shape, levels, kind, wide):
+    """FP32 red-black 3D cycles: the complex128 input taken with the red half-sweep, residual and full
+    weighting in one kernel (with the coarse red half-sweep), the black-only prolongation, the separable
+    coarse solve in planes and columns, and the last sweep writing natural order in either precision; odd
+    and even sizes, more and fewer columns than a warp's 30."""
+    from paper_0912_0180_gb300.helm import Helm
+    p = hi.make_problem(3, shape, 0, k0=6.0, phi_kind=kind, rhs="zero", bump_centre=(0.3, 0.6, 0.4))
+    pc = hi.Precond(kind=hi.PC_CSG_UNIFORM, theta_beta=0.3, smoother=hi.SM_RBGS, max_levels=levels)
+    r = hi.random_vector(p.n, 51)
+    ref = Oracle(p, pc).vcycle(r)
+    h = Helm(p, pc, mg_dtype="c64")
+    z = h.vcycle(torch.from_numpy(r).cuda(), dtype=torch.complex128 if wide else torch.complex64).cpu().numpy()
+    h.close()
+    assert np.linalg.norm(z - ref) <= 5e-5 * np.linalg.norm(ref)
+    assert np.max(np.abs(z - ref)) <= 5e-5 * np.max(np.abs(ref))
