@@ -35,12 +35,32 @@ template <int DIM> static void rb_cfg(const int n[3], dim3& g, dim3& b) {
   g = dim3((n[0] + 15) / 16, (n[1] + 2 * b.y - 1) / (2 * b.y), n[2]);
 }
 
-#define POINT_INDEX(op)                                                        \
-  int i = blockIdx.x * blockDim.x + threadIdx.x;                               \
-  int j = blockIdx.y * blockDim.y + threadIdx.y;                               \
-  int l = blockIdx.z;                                                          \
-  if (i >= (op).n[0] || j >= (op).n[1]) return;                                \
+// The point of a thread in the one-thread-per-point kernels launched by cfg; false: none.  A 3D grid whose
+// rows end in a short chunk (at most TAIL_COLS columns past a multiple of 32) takes those columns of a
+// plane by other threads of the last column of blocks: lanes along y, packed.  FP64 only: its pipe (2 lanes
+// a clock) bills a warp's 32 lanes whatever they do -- a row of 129 points cost five chunks (129 x 145 x
+// 113 points: sweep 160 -> 129 us, residual 113 -> 90 us).  A point's formula depends on its indices alone.
+constexpr int TAIL_COLS = 16;
+template <typename T, int DIM>
+__device__ __forceinline__ bool point_of(const int (&n)[3], int& i, int& j, int& l) {
+  i = blockIdx.x * blockDim.x + threadIdx.x;
+  j = blockIdx.y * blockDim.y + threadIdx.y;
+  l = blockIdx.z;
+  if constexpr (DIM == 3 && sizeof(T) == 8) {
+    const int rem = n[0] & 31;
+    if (rem && rem <= TAIL_COLS && (int)blockIdx.x == n[0] >> 5) {
+      const int q = (blockIdx.y * blockDim.y + threadIdx.y) * 32 + threadIdx.x;
+      j = q / rem;
+      i = (n[0] & ~31) + q - j * rem;
+    }
+  }
+  return i < n[0] && j < n[1];
+}
+#define POINT_INDEX_T(op, T, DIM)                                              \
+  int i, j, l;                                                                 \
+  if (!point_of<T, DIM>((op).n, i, j, l)) return;                              \
   long p = i + (long)(op).n[0] * (j + (long)(op).n[1] * l);
+#define POINT_INDEX(op) POINT_INDEX_T(op, float, 2)
 
 // y = M x, or y = f - M x when f is given.  XS: x, f and y are stored x-split (h = (n0 + 1) / 2).
 template <typename T, int DIM, bool XS = false>
@@ -48,7 +68,7 @@ __global__ void k_mg_apply(OpView<T> op, const cx<T>* __restrict__ x, const cx<T
                            cx<T>* __restrict__ y, const int* skip) {
   pdl_entry();
   if (skip && *skip) return;
-  POINT_INDEX(op);
+  POINT_INDEX_T(op, T, DIM);
   if (XS) {
     const int h = (op.n[0] + 1) >> 1;
     const long row = p - i, ps = row + xs_pos(i, h);
@@ -68,7 +88,7 @@ __global__ void k_jacobi(OpView<T> op, const cx<T>* __restrict__ u, const cx<T>*
                          cx<T>* __restrict__ un, T omega, double2* __restrict__ wide, const int* skip) {
   pdl_entry();
   if (skip && *skip) return;
-  POINT_INDEX(op);
+  POINT_INDEX_T(op, T, DIM);
   cx<T> di = op.dinv[p];  // omega / D
   cx<T> v;
   if (!u) {
@@ -465,11 +485,8 @@ __global__ void k_resid0(OpView<T> op, const cx<T>* __restrict__ u, const cx<T>*
   if (skip && *skip) return;
   int t, j;
   if (RB) rb_pair_index<DIM>(t, j);
-  else {
-    t = blockIdx.x * blockDim.x + threadIdx.x;
-    j = blockIdx.y * blockDim.y + threadIdx.y;
-  }
   int l = blockIdx.z;
+  if (!RB && !point_of<T, DIM>(op.n, t, j, l)) return;
   if (j >= op.n[1]) return;
   const long row = (long)op.n[0] * (j + (long)op.n[1] * l);
   if (RB) {
@@ -717,6 +734,67 @@ __global__ void k_prolong(Dims d, const cx<T>* __restrict__ ec, cx<T>* __restric
     cx<T> uo = u[p];
     u[p] = mkc<T>(fma(w, acc.x, uo.x), fma(w, acc.y, uo.y));
   }
+}
+
+// Trilinear prolongation in natural order, a thread per pair of columns (2t, 2t + 1): no lane runs the other
+// parity's sums, and in FP64 the two points share the sums over their common coarse column (1.75 complex
+// additions a point; k_prolong's lanes paid for 4.5; 129 x 145 x 113 points: 67 -> 49 us).  FP32 adds in k_prolong's
+// order, bit for bit its result; so does BLACK, which corrects only the black points, before a red-black
+// sweep (whose red half overwrites the red ones): one column a row, the same for all its lanes.
+template <typename T, bool BLACK>
+__global__ void __launch_bounds__(128) k_prolong3p(Dims d, const cx<T>* __restrict__ ec, cx<T>* __restrict__ u,
+                                                   int overwrite, const int* skip) {
+  pdl_entry();
+  if (skip && *skip) return;
+  const int t = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y * blockDim.y + threadIdx.y, l = blockIdx.z;
+  if (2 * t >= d.f[0] || j >= d.f[1]) return;
+  const bool has1 = 2 * t + 1 < d.f[0];
+  int cj[2] = {0, 0}, cl[2] = {0, 0};
+  const int nj = interp1(j, d.c[1], d.o[1], cj), nl = interp1(l, d.c[2], d.o[2], cl);
+  auto on_coarse = [](int x, int o) { return x - o >= 0 && !((x - o) & 1); };
+  const T wyz = (on_coarse(j, d.o[1]) ? T(1) : T(0.5)) * (on_coarse(l, d.o[2]) ? T(1) : T(0.5));
+  // coarse columns a, a + 1: the column on a coarse node takes one of them, the other both
+  const int a = t - d.o[0];
+  const bool va = a >= 0 && a < d.c[0], vb = a + 1 < d.c[0];
+  const cx<T> zero = mkc<T>(T(0), T(0));
+  const long row = (long)d.f[0] * (j + (long)d.f[1] * l) + 2 * t;
+  if (BLACK) {
+    const bool odd = !((j + l) & 1);  // the black column
+    if (odd && !has1) return;
+    const bool ca = odd ? d.o[0] == 0 : true, cb = odd ? true : d.o[0] == 1;
+    cx<T> acc = zero;
+    for (int c3 = 0; c3 < nl; ++c3)
+      for (int c2 = 0; c2 < nj; ++c2) {
+        const cx<T>* e = ec + (long)d.c[0] * (cj[c2] + (long)d.c[1] * cl[c3]) + a;
+        if (ca && va) acc = cadd<T>(acc, e[0]);
+        if (cb && vb) acc = cadd<T>(acc, e[1]);
+      }
+    const T w = ca && cb ? T(0.5) * wyz : wyz;
+    cx<T>* const q = u + row + (odd ? 1 : 0);
+    *q = overwrite ? cscale<T>(w, acc) : mkc<T>(fma(w, acc.x, q->x), fma(w, acc.y, q->y));
+    return;
+  }
+  cx<T> u0 = zero, u1 = zero;
+  if (!overwrite) {
+    u0 = u[row];
+    if (has1) u1 = u[row + 1];
+  }
+  cx<T> sa = zero, sb = zero, both = zero;
+  for (int c3 = 0; c3 < nl; ++c3)
+    for (int c2 = 0; c2 < nj; ++c2) {
+      const cx<T>* e = ec + (long)d.c[0] * (cj[c2] + (long)d.c[1] * cl[c3]) + a;
+      const cx<T> ea = va ? e[0] : zero, eb = vb ? e[1] : zero;
+      const bool first = c2 == 0 && c3 == 0;
+      sa = first ? ea : cadd<T>(sa, ea);
+      sb = first ? eb : cadd<T>(sb, eb);
+      if (sizeof(T) == 4) both = cadd<T>(cadd<T>(both, ea), eb);
+    }
+  if (sizeof(T) == 8) both = cadd<T>(sa, sb);
+  // o = 1: the even column lies between a and a + 1, the odd one on a + 1; o = 0: on a, and between
+  const cx<T> s0 = d.o[0] ? both : sa, s1 = d.o[0] ? sb : both;
+  const T w0 = d.o[0] ? T(0.5) * wyz : wyz, w1 = d.o[0] ? wyz : T(0.5) * wyz;
+  u[row] = overwrite ? cscale<T>(w0, s0) : mkc<T>(fma(w0, s0.x, u0.x), fma(w0, s0.y, u0.y));
+  if (has1) u[row + 1] = overwrite ? cscale<T>(w1, s1) : mkc<T>(fma(w1, s1.x, u1.x), fma(w1, s1.y, u1.y));
 }
 
 // The 3D transfers onto / from an x-split fine level, marching along z (one thread per coarse
@@ -1025,7 +1103,7 @@ __global__ void k_coarse(const cx<T>* __restrict__ Ainv, int n, const cx<T>* __r
 template <typename TX, int DIM>
 __global__ void k_h_apply(OpView<double> op, const cx<TX>* __restrict__ x, double2* __restrict__ y) {
   pdl_entry();
-  POINT_INDEX(op);
+  POINT_INDEX_T(op, double, DIM);
   y[p] = op_row<double, TX, DIM>(op, x, i, j, l, p);
 }
 
@@ -1257,6 +1335,12 @@ template <typename T, int DIM> struct Launch {
       else if (black) launch_pdl(k_prolong3z<T, long, true>, g, dim3(32, 4), 0, st, d, ec, u, overwrite, lz, skip);
       else if (i32) launch_pdl(k_prolong3z<T, int, false>, g, dim3(32, 4), 0, st, d, ec, u, overwrite, lz, skip);
       else launch_pdl(k_prolong3z<T, long, false>, g, dim3(32, 4), 0, st, d, ec, u, overwrite, lz, skip);
+      return;
+    }
+    if (DIM == 3 && !F.xs && !C.xs) {
+      dim3 g((unsigned)(((F.n[0] + 1) / 2 + 31) / 32), (unsigned)((F.n[1] + 3) / 4), (unsigned)F.n[2]);
+      if (black) launch_pdl(k_prolong3p<T, true>, g, dim3(32, 4), 0, st, d, ec, u, overwrite, skip);
+      else launch_pdl(k_prolong3p<T, false>, g, dim3(32, 4), 0, st, d, ec, u, overwrite, skip);
       return;
     }
     dim3 g, b; cfg<DIM>(F.n, g, b);

@@ -143,3 +143,24 @@ def test_xsplit_cycle_3d(shape, levels, kind, wide):
     h.close()
     assert np.linalg.norm(z - ref) <= 5e-5 * np.linalg.norm(ref)
     assert np.max(np.abs(z - ref)) <= 5e-5 * np.max(np.abs(ref))
+
+
+@pytest.mark.parametrize("sm", [hi.SM_JACOBI, hi.SM_RBGS])
+@pytest.mark.parametrize("mg", ["c128", "c64"])
+@pytest.mark.parametrize("shape", [(35, 20, 23), (50, 21, 12), (51, 9, 30), (66, 18, 17), (82, 12, 11)])
+def test_natural_cycle_3d(shape, mg, sm):
+    """Natural-order 3D levels: rows ending in a short chunk of columns (1, 16, 17, 0 and 16 past a multiple of
+    32), whose points FP64 kernels pack along y, and the pairwise prolongation, at odd and even sizes."""
+    from paper_0912_0180_gb300.helm import Helm
+    p = hi.make_problem(3, shape, 0, k0=6.0, phi_kind="bump", rhs="zero", bump_centre=(0.3, 0.6, 0.4))
+    pc = hi.Precond(kind=hi.PC_CSL, shift=1 + 0.5j, smoother=sm)
+    r = hi.random_vector(p.n, 61)
+    o = Oracle(p, pc)
+    ref = o.vcycle(r)
+    tol = 1e-10 if mg == "c128" else 5e-5
+    h = Helm(p, pc, mg_dtype=mg)
+    z = h.vcycle(torch.from_numpy(r).cuda()).cpu().numpy()
+    assert np.linalg.norm(z - ref) <= tol * np.linalg.norm(ref) and np.max(np.abs(z - ref)) <= tol * np.max(np.abs(ref))
+    y, y_ref = h.apply(torch.from_numpy(r).cuda()).cpu().numpy(), o.apply(r)
+    assert np.linalg.norm(y - y_ref) <= 1e-12 * np.linalg.norm(y_ref)
+    h.close()
