@@ -27,7 +27,8 @@
 // read them ([strip][step][entry][lane]) and fetched 16 to 24 steps ahead (cp.async), since nothing
 // else runs on the SM to hide a load.  One block walking the wavefronts with a barrier each cost 1.1
 // us a wavefront in FP32; a V(0,1) cycle of MP3's operators on 640^2 unknowns went from 8.40 to 0.99
-// ms (0.36 ms of it the finest level's two solves: about 0.11 us a step).
+// ms, 0.96 with the factors of eight steps read into registers at once (about 0.1 us a step, 54 instructions of
+// which half wait on the one before).
 #include <algorithm>
 #include <type_traits>
 #include <vector>
@@ -204,15 +205,19 @@ __device__ __forceinline__ unsigned ilu_map(unsigned a, unsigned rank) {
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
   return r;
 }
-__device__ __forceinline__ void ilu_send(unsigned to, unsigned bar, float2 v) {
-  const unsigned long long b = ((unsigned long long)__float_as_uint(v.y) << 32) | __float_as_uint(v.x);
-  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.b64 [%0], %1, [%2];" ::"r"(to), "l"(b), "r"(bar)
-               : "memory");
+// (predicated, not branched around: a branch a step costs its resolution; no memory clobber: the next
+// steps' loads may move above it)
+__device__ __forceinline__ void ilu_send(bool on, unsigned to, unsigned bar, float2 v) {
+  asm volatile(
+      "{\n .reg .pred p;\n .reg .b64 d;\n setp.ne.u32 p, %0, 0;\n mov.b64 d, {%2, %3};\n"
+      " @p st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.b64 [%1], d, [%4];\n}" ::"r"((unsigned)on),
+      "r"(to), "f"(v.x), "f"(v.y), "r"(bar));
 }
-__device__ __forceinline__ void ilu_send(unsigned to, unsigned bar, double2 v) {
-  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v2.b64 [%0], {%1, %2}, [%3];" ::"r"(to),
-               "l"(__double_as_longlong(v.x)), "l"(__double_as_longlong(v.y)), "r"(bar)
-               : "memory");
+__device__ __forceinline__ void ilu_send(bool on, unsigned to, unsigned bar, double2 v) {
+  asm volatile(
+      "{\n .reg .pred p;\n setp.ne.u32 p, %0, 0;\n"
+      " @p st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v2.b64 [%1], {%2, %3}, [%4];\n}" ::"r"((unsigned)on),
+      "r"(to), "l"(__double_as_longlong(v.x)), "l"(__double_as_longlong(v.y)), "r"(bar));
 }
 __device__ __forceinline__ void ilu_expect(unsigned bar, unsigned bytes) {
   asm volatile("{\n .reg .b64 t;\n mbarrier.arrive.expect_tx.shared::cta.b64 t, [%0], %1;\n}" ::"r"(bar), "r"(bytes) : "memory");
@@ -270,6 +275,7 @@ __device__ __forceinline__ void ilu_strip(const IluArgs<T>& g, int strip, cx<T>*
   cx<T>* const v = g.v + (long)strip * steps * 32 + lane;
   const cx<T>* const fac = (UP ? g.up : g.lo) + (long)strip * steps * NE * 32 + lane;
   const cx<T>* const other = g.v + (long)(UP ? strip + 1 : strip - 1) * steps * 32 + GIVE;
+  const bool gives = lane == GIVE && to_row != 0;
   bool failed = false;
   int armed = 0;  // chunks of the edge row waited for
   auto chunk = [&](int c) { return UP ? nc - 1 - c : c; };  // c-th chunk in this direction
@@ -323,37 +329,47 @@ __device__ __forceinline__ void ilu_strip(const IluArgs<T>& g, int strip, cx<T>*
     const cx<T> en = lane < CH ? edge_at(col_new(UP ? m * CH + CH - 1 - lane : m * CH + lane)) : zero;
     ilu_landed<DEPTH - 1>();
     const cx<T>* const at = ring + (c % DEPTH) * CH * SL * 32 + lane;
+    // a few steps' factors and right-hand sides into registers at once: one warp has nobody to hide a
+    // shared-memory load behind
+    constexpr int BS = sizeof(T) == 4 ? 8 : 4;
 #pragma unroll
-    for (int k = 0; k < CH; ++k) {
-      const int kk = UP ? CH - 1 - k : k, t = m * CH + kk, i = t - K * lane;
-      const cx<T>* const q = at + kk * SL * 32;
-      const cx<T> x = q[NE * 32];
-      // the lane above's (below's) last value
-      cx<T> nw = UP ? mkc<T>(__shfl_down_sync(0xffffffffu, prev.x, 1), __shfl_down_sync(0xffffffffu, prev.y, 1))
-                    : mkc<T>(__shfl_up_sync(0xffffffffu, prev.x, 1), __shfl_up_sync(0xffffffffu, prev.y, 1));
-      const cx<T> ek = ilu_shfl<T>(en, k);
-      if (lane == TAKE) nw = ek;
-      cx<T> r;
-      if (UP) {
-        r = cmul<T>(q[0], x);
-        if (BOX) r = cfms<T>(q[4 * 32], a, cfms<T>(q[3 * 32], b, r));  // (i+1, j+1), (i, j+1)
-        r = cfms<T>(q[32], prev, r);                                   // (i+1, j)
-        r = cfms<T>(q[2 * 32], nw, r);                                 // (i-1, j+1); cross (i, j+1)
-      } else {
-        r = x;
-        if (BOX) r = cfms<T>(q[32], b, cfms<T>(q[0], a, r));           // (i-1, j-1), (i, j-1)
-        r = cfms<T>(q[(BOX ? 3 : 1) * 32], prev, r);                   // (i-1, j)
-        r = cfms<T>(q[(BOX ? 2 : 0) * 32], nw, r);                     // (i+1, j-1); cross (i, j-1)
+    for (int kb = 0; kb < CH; kb += BS) {
+      cx<T> q[BS][SL];
+#pragma unroll
+      for (int k = 0; k < BS; ++k)
+#pragma unroll
+        for (int e = 0; e < SL; ++e) q[k][e] = at[((UP ? CH - 1 - kb - k : kb + k) * SL + e) * 32];
+#pragma unroll
+      for (int k = 0; k < BS; ++k) {
+        const int kk = UP ? CH - 1 - kb - k : kb + k, t = m * CH + kk, i = t - K * lane;
+        const cx<T> x = q[k][NE];
+        // the lane above's (below's) last value
+        cx<T> nw = UP ? mkc<T>(__shfl_down_sync(0xffffffffu, prev.x, 1), __shfl_down_sync(0xffffffffu, prev.y, 1))
+                      : mkc<T>(__shfl_up_sync(0xffffffffu, prev.x, 1), __shfl_up_sync(0xffffffffu, prev.y, 1));
+        const cx<T> ek = ilu_shfl<T>(en, kb + k);
+        if (lane == TAKE) nw = ek;
+        cx<T> r;
+        if (UP) {
+          r = cmul<T>(q[k][0], x);
+          if (BOX) r = cfms<T>(q[k][BOX ? 4 : 0], a, cfms<T>(q[k][BOX ? 3 : 0], b, r));  // (i+1, j+1), (i, j+1)
+          r = cfms<T>(q[k][1], prev, r);                                                 // (i+1, j)
+          r = cfms<T>(q[k][2], nw, r);                                                   // (i-1, j+1); cross (i, j+1)
+        } else {
+          r = x;
+          if (BOX) r = cfms<T>(q[k][1], b, cfms<T>(q[k][0], a, r));  // (i-1, j-1), (i, j-1)
+          r = cfms<T>(q[k][BOX ? 3 : 1], prev, r);                   // (i-1, j)
+          r = cfms<T>(q[k][BOX ? 2 : 0], nw, r);                     // (i+1, j-1); cross (i, j-1)
+        }
+        const bool in = has_row && i >= 0 && i < n0;
+        if (!in) r = zero;  // a point outside the grid is zero for the neighbours
+        else v[(long)t * 32] = r;
+        ilu_send(gives && in, to_row + (unsigned)(i * (int)sizeof(cx<T>)), to_bar + m * 8, r);
+        a = b;
+        b = nw;
+        prev = r;
       }
-      if (failed) r = mkc<T>(T(NAN), T(NAN));  // the wait ran out: the solve ends with a NaN status
-      const bool in = has_row && i >= 0 && i < n0;
-      if (!in) r = zero;  // a point outside the grid is zero for the neighbours
-      else v[(long)t * 32] = r;
-      if (lane == GIVE && to_row && in) ilu_send(to_row + (unsigned)(i * sizeof(cx<T>)), to_bar + (t / CH) * 8, r);
-      a = b;
-      b = nw;
-      prev = r;
     }
+    if (failed) prev = b = mkc<T>(T(NAN), T(NAN));  // the wait ran out: the solve ends with a NaN status
   }
   ilu_landed<0>();
 }
