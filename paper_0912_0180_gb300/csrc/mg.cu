@@ -1452,7 +1452,7 @@ static bool fused_applies(const helm_ctx* c, int l) {
   if (pcf.flags & HELM_PF_UNFUSED) return false;
   if (pcf.smoother == HELM_SM_ILU) return false;  // ILU(0) runs as its own kernels
   if (l >= c->tail_first) return true;
-  if (c->lv[l].stg64) return false;  // 9-point Galerkin levels run the per-component kernels
+  if (c->lv[l].stg64 && pcf.smoother != HELM_SM_JACOBI) return false;
   if (c->lv[l].any_offset0()) return false;  // the fused tiles assume coarse c = fine 2c + 1
   return c->lv[l].dim == 2 && pcf.nu1 == 1 && pcf.nu2 == 1 && l < (int)c->lv.size() - 1;
 }

@@ -100,23 +100,9 @@ __device__ __forceinline__ Share ct_share(const CTailArgs<T>& a, int k, int r) {
   return s;
 }
 
-// Off-diagonal part of a 9-point row at (i, j): u points at its value in the padded staged rows
-// (pitch w; zero outside the grid, where the weights are not used by off9 either).
-template <typename T>
-__device__ __forceinline__ cx<T> ct_off9(const OpView<T>& op, const cx<T>* u, int w, long p) {
-  cx<T> acc = mkc<T>(T(0), T(0));
-#pragma unroll
-  for (int dj = -1; dj <= 1; ++dj)
-#pragma unroll
-    for (int di = -1; di <= 1; ++di) {
-      if (di == 0 && dj == 0) continue;
-      acc = cfma<T>(op.stg[(long)(3 * (dj + 1) + (di + 1)) * op.ntot + p], u[di + dj * w], acc);
-    }
-  return acc;
-}
 template <typename T>
 __device__ __forceinline__ cx<T> ct_off(const OpView<T>& op, const cx<T>* u, int w, int i, int j) {
-  if (op.stg) return ct_off9<T>(op, u, w, i + (long)op.n[0] * j);
+  if (op.stg) return off9_staged<T>(op, u, w, i + (long)op.n[0] * j);
   return off2d<T>(op, i, j, u[-1], u[1], u[-w], u[w]);
 }
 

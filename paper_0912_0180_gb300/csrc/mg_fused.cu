@@ -74,8 +74,10 @@ __device__ __forceinline__ bool colour_item(int k, int W, int gi0, int gj0, int 
 template <typename T, bool RBGS> constexpr bool keeps_u() { return RBGS || sizeof(T) == 8; }
 
 // TI: element type of f -- complex128 on the finest level of an FP32 cycle called with a complex128
-// vector, narrowed as it is read (no conversion pass).
-template <typename T, bool RBGS, int CX, int CY, int NT, typename TI>
+// vector, narrowed as it is read (no conversion pass).  NINE: a Galerkin level's 9-point rows (damped
+// Jacobi; they were three kernels down and two up: at 256^2 in FP64 16 -> 12 and 14 -> 11 us, the MP2 cycle
+// 100.7 -> 93.7 us).
+template <typename T, bool RBGS, int CX, int CY, int NT, typename TI, bool NINE = false>
 __device__ __forceinline__ void down2d_body(int bx_, int by_, const OpView<T>& op, int nc0, int nc1, const cx<TI>* __restrict__ f, cx<T>* __restrict__ u_out,
          cx<T>* __restrict__ fc, T omega) {
   constexpr int HF = RBGS ? 2 : 1;
@@ -155,7 +157,9 @@ __device__ __forceinline__ void down2d_body(int bx_, int by_, const OpView<T>& o
       cx<T> rv = mkc<T>(T(0), T(0));
       if (i < n0 && j < n1) {
         int sx = x + HF, sy = y + HF;
-        cx<T> acc = off2d<T>(op, i, j, su[sy][sx - 1], su[sy][sx + 1], su[sy - 1][sx], su[sy + 1][sx]);
+        cx<T> acc;
+        if constexpr (NINE) acc = off9_staged<T>(op, &su[sy][sx], FX, i + (long)n0 * j);
+        else acc = off2d<T>(op, i, j, su[sy][sx - 1], su[sy][sx + 1], su[sy - 1][sx], su[sy + 1][sx]);
         const T om1 = T(1) - omega;  // (1 - omega) f - acc in two fused multiply-adds, as k_resid0
         rv = mkc<T>(fma(om1, sf[sy][sx].x, -acc.x), fma(om1, sf[sy][sx].y, -acc.y));
       }
@@ -194,18 +198,18 @@ __device__ __forceinline__ void down2d_body(int bx_, int by_, const OpView<T>& o
     fc[I + nc0 * J] = cscale<T>(T(0.0625), acc);
   }
 }
-template <typename T, bool RBGS, int CX, int CY, int NT, typename TI>
+template <typename T, bool RBGS, int CX, int CY, int NT, typename TI, bool NINE = false>
 __global__ void __launch_bounds__(NT)
 k_down2d(OpView<T> op, int nc0, int nc1, const cx<TI>* __restrict__ f, cx<T>* __restrict__ u_out,
          cx<T>* __restrict__ fc, T omega, const int* skip, int early) {
   if (early) pdl_trigger();
   pdl_entry();
   if (skip && *skip) return;
-  down2d_body<T, RBGS, CX, CY, NT, TI>(blockIdx.x, blockIdx.y, op, nc0, nc1, f, u_out, fc, omega);
+  down2d_body<T, RBGS, CX, CY, NT, TI, NINE>(blockIdx.x, blockIdx.y, op, nc0, nc1, f, u_out, fc, omega);
 }
 
 // ---- up: prolongation + correction + post-smoothing (2D, nu2 = 1), out of place --------------
-template <typename T, bool RBGS, typename TO, int FX, int FY, int NT, typename TI>
+template <typename T, bool RBGS, typename TO, int FX, int FY, int NT, typename TI, bool NINE = false>
 __device__ __forceinline__ void up2d_body(int bx_, int by_, const OpView<T>& op, int nc0, int nc1, const cx<T>* __restrict__ u_in, const cx<T>* __restrict__ ec,
        const cx<TI>* __restrict__ f, cx<TO>* __restrict__ u_out, T omega) {
   constexpr int HU = RBGS ? 2 : 1;                 // halo of the corrected iterate
@@ -294,7 +298,9 @@ __device__ __forceinline__ void up2d_body(int bx_, int by_, const OpView<T>& op,
       if (i >= n0 || j >= n1) continue;
       int p = i + n0 * j;
       int sx = x + HU, sy = y + HU;
-      cx<T> acc = off2d<T>(op, i, j, su[sy][sx - 1], su[sy][sx + 1], su[sy - 1][sx], su[sy + 1][sx]);
+      cx<T> acc;
+      if constexpr (NINE) acc = off9_staged<T>(op, &su[sy][sx], UX, i + (long)n0 * j);
+      else acc = off2d<T>(op, i, j, su[sy][sx - 1], su[sy][sx + 1], su[sy - 1][sx], su[sy + 1][sx]);
       cx<T> g = cmul1<T>(csub<T>(cconv<T, TI>(f[p]), acc), op.dinv[p]);  // dinv holds omega / D
       cx<T> uc = su[sy][sx];
       const T om1 = T(1) - omega;
@@ -338,13 +344,13 @@ __device__ __forceinline__ void up2d_body(int bx_, int by_, const OpView<T>& op,
     }
   }
 }
-template <typename T, bool RBGS, typename TO, int FX, int FY, int NT, typename TI>
+template <typename T, bool RBGS, typename TO, int FX, int FY, int NT, typename TI, bool NINE = false>
 __global__ void __launch_bounds__(NT)
 k_up2d(OpView<T> op, int nc0, int nc1, const cx<T>* __restrict__ u_in, const cx<T>* __restrict__ ec,
        const cx<TI>* __restrict__ f, cx<TO>* __restrict__ u_out, T omega, const int* skip) {
   pdl_entry();
   if (skip && *skip) return;
-  up2d_body<T, RBGS, TO, FX, FY, NT, TI>(blockIdx.x, blockIdx.y, op, nc0, nc1, u_in, ec, f, u_out, omega);
+  up2d_body<T, RBGS, TO, FX, FY, NT, TI, NINE>(blockIdx.x, blockIdx.y, op, nc0, nc1, u_in, ec, f, u_out, omega);
 }
 
 // ---- the row-walking kernels (damped Jacobi) ---------------------------------------------------
@@ -711,11 +717,11 @@ static bool big_tiles(const helm_ctx* c, long blocks) {
   return blocks >= 2L * sms;
 }
 
-template <typename T, bool RB, int CX, int CY, int NT, typename TI>
+template <typename T, bool RB, int CX, int CY, int NT, typename TI, bool NINE = false>
 static void down_launch(const LevelHost& F, const LevelHost& C, const cx<TI>* f, cx<T>* u_out, cx<T>* fc, T om,
                         const int* skip, cudaStream_t st, int early) {
   dim3 g((C.n[0] + CX - 1) / CX, (C.n[1] + CY - 1) / CY);
-  launch_pdl(k_down2d<T, RB, CX, CY, NT, TI>, dim3(g), dim3(NT), 0, st, F.view<T>(), C.n[0], C.n[1], f, u_out, fc, om, skip,
+  launch_pdl(k_down2d<T, RB, CX, CY, NT, TI, NINE>, dim3(g), dim3(NT), 0, st, F.view<T>(), C.n[0], C.n[1], f, u_out, fc, om, skip,
              early);
 }
 
@@ -805,15 +811,22 @@ void fused_down2d(const helm_ctx* c, int l, const cx<TI>* f, cx<T>* u_out, cx<T>
   // before the one-cluster tail (16 blocks, which read their constants before they wait) the launch
   // of the next kernel is triggered at once
   const int early = l + 1 == c->tail_first && ctail_applies(c);
+  if (F.stg64) {  // a Galerkin level (never the finest): the block-count rule's tiles
+    if constexpr (std::is_same<T, TI>::value) {
+      if (big_tiles(c, nb)) down_launch<T, false, DN_CX, DN_CY, FUSED_THREADS, T, true>(F, C, f, u_out, fc, om, skip, st, early);
+      else down_launch<T, false, DN_SCX, DN_SCY, FUSED_SMALL_THREADS, T, true>(F, C, f, u_out, fc, om, skip, st, early);
+    }
+    return;
+  }
   if (c->pc.smoother == HELM_SM_RBGS) down_tile<T, true, TI>(tile, F, C, f, u_out, fc, om, skip, st, early);
   else down_tile<T, false, TI>(tile, F, C, f, u_out, fc, om, skip, st, early);
 }
 
-template <typename T, bool RB, typename TO, int FX, int FY, int NT, typename TI>
+template <typename T, bool RB, typename TO, int FX, int FY, int NT, typename TI, bool NINE = false>
 static void up_launch(const LevelHost& F, const LevelHost& C, const cx<T>* u_in, const cx<T>* ec, const cx<TI>* f,
                       TO* out, T om, const int* skip, cudaStream_t st) {
   dim3 g((F.n[0] + FX - 1) / FX, (F.n[1] + FY - 1) / FY);
-  launch_pdl(k_up2d<T, RB, TO, FX, FY, NT, TI>, dim3(g), dim3(NT), 0, st, F.view<T>(), C.n[0], C.n[1], u_in, ec, f,
+  launch_pdl(k_up2d<T, RB, TO, FX, FY, NT, TI, NINE>, dim3(g), dim3(NT), 0, st, F.view<T>(), C.n[0], C.n[1], u_in, ec, f,
              (cx<TO>*)out, om, skip);
 }
 
@@ -847,6 +860,15 @@ void fused_up2d(const helm_ctx* c, int l, const cx<T>* u_in, const cx<T>* ec, co
                 bool out_f64, const int* skip, cudaStream_t st) {
   const LevelHost& F = c->lv[l];
   const LevelHost& C = c->lv[l + 1];
+  if (F.stg64) {
+    if constexpr (std::is_same<T, TI>::value) {
+      const long nb = (long)((F.n[0] + UP_FX - 1) / UP_FX) * ((F.n[1] + UP_FY - 1) / UP_FY);
+      const T om = (T)c->pc.omega;
+      if (big_tiles(c, nb)) up_launch<T, false, T, UP_FX, UP_FY, FUSED_THREADS, T, true>(F, C, u_in, ec, f, (T*)out, om, skip, st);
+      else up_launch<T, false, T, UP_SFX, UP_SFY, FUSED_SMALL_THREADS, T, true>(F, C, u_in, ec, f, (T*)out, om, skip, st);
+    }
+    return;
+  }
   if (out_f64) up_dispatch<T, double, TI>(c, F, C, u_in, ec, f, out, skip, st);
   else up_dispatch<T, T, TI>(c, F, C, u_in, ec, f, out, skip, st);
 }

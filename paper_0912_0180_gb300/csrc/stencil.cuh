@@ -183,6 +183,21 @@ __device__ __forceinline__ cx<T> off2d(const OpView<T>& op, int i, int j, cx<T> 
   return cfma<T>(op.ap[1][j], xn, cfma<T>(op.am[1][j], xs, acc));
 }
 
+// Off-diagonal part of a 9-point (Galerkin) row at point p: u points at its value in rows of pitch w, staged
+// with zeros outside the grid.
+template <typename T>
+__device__ __forceinline__ cx<T> off9_staged(const OpView<T>& op, const cx<T>* u, int w, long p) {
+  cx<T> acc = mkc<T>(T(0), T(0));
+#pragma unroll
+  for (int dj = -1; dj <= 1; ++dj)
+#pragma unroll
+    for (int di = -1; di <= 1; ++di) {
+      if (di == 0 && dj == 0) continue;
+      acc = cfma<T>(op.stg[(long)(3 * (dj + 1) + (di + 1)) * op.ntot + p], u[di + dj * w], acc);
+    }
+  return acc;
+}
+
 // point coordinates from a linear index
 __device__ __forceinline__ void unflatten(long p, const int n[3], int& i, int& j, int& l) {
   i = (int)(p % n[0]);
