@@ -1337,14 +1337,14 @@ template <typename T, int DIM> struct Launch {
       else launch_pdl(k_prolong3z<T, long, false>, g, dim3(32, 4), 0, st, d, ec, u, overwrite, lz, skip);
       return;
     }
-    if (DIM == 3 && !F.xs && !C.xs) {
+    if constexpr (DIM == 3) {  // (the level below a natural one is natural)
       dim3 g((unsigned)(((F.n[0] + 1) / 2 + 31) / 32), (unsigned)((F.n[1] + 3) / 4), (unsigned)F.n[2]);
       if (black) launch_pdl(k_prolong3p<T, true>, g, dim3(32, 4), 0, st, d, ec, u, overwrite, skip);
       else launch_pdl(k_prolong3p<T, false>, g, dim3(32, 4), 0, st, d, ec, u, overwrite, skip);
-      return;
+    } else {
+      dim3 g, b; cfg<DIM>(F.n, g, b);
+      launch_pdl(k_prolong<T, DIM>, dim3(g), dim3(b), 0, st, d, ec, u, overwrite, skip);
     }
-    dim3 g, b; cfg<DIM>(F.n, g, b);
-    launch_pdl(k_prolong<T, DIM>, dim3(g), dim3(b), 0, st, d, ec, u, overwrite, skip);
   }
 };
 

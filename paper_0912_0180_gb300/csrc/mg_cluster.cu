@@ -382,14 +382,16 @@ __device__ __forceinline__ void ctail_body(const CTailArgs<T>* __restrict__ ga, 
     if (k == 0) pdl_trigger();  // the next kernel's blocks may come up while this one finishes
     if (k == 0) ct_arrive();  // the last read of another block's shared memory
     __syncthreads();
-    {  // corrected iterate on rows 2A - HU .. pe - 1 + HU, in place
-      const int jb = 2 * s.A - HU, ne = s.rows ? (s.pe + HU - jb) * s.n0 : 0;
+    {  // corrected iterate on rows 2A - HU .. pe - 1 + HU, in place (red-black: its black points, all that
+       // the red half-sweep reads)
+      const int jb = 2 * s.A - HU, wi = RB ? (s.n0 + 1) >> 1 : s.n0, ne = s.rows ? (s.pe + HU - jb) * wi : 0;
 #pragma unroll 2
       for (int e = tid; e < ne; e += CT) {
         int i, y;
-        ct_div(e, s.n0, a.magic[k], i, y);
+        ct_div(e, wi, RB ? a.magich[k] : a.magic[k], i, y);
         const int j = jb + y;
-        if (j < 0 || j >= s.n1) continue;
+        if (RB) i = 2 * i + ((j + 1) & 1);
+        if (i >= s.n0 || j < 0 || j >= s.n1) continue;
         const int ia = (i - 1) >> 1, ja = (j - 1) >> 1;  // odd: the coarse node; even: the one before
         const cx<T>* ra = scr + (ja - c0) * we + 1 + ia;
         cx<T> acc;
