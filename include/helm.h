@@ -146,13 +146,16 @@ typedef struct {
  * same arithmetic as the default fused kernels; for testing the fusion); HELM_PF_NO_PDL
  * launches the solve-path kernels without programmatic dependent launch (same kernels);
  * HELM_PF_NO_AUTOTUNE skips the autotuner of helm_create, which times the large, small, square, wide
- * and one-warp tiles of the fused 2D kernels on every fused level and then whole V-cycles for every
- * admissible depth of the one-block tail kernel, keeps the fastest, and caches the choices for the
- * process (tiles by precision, smoother and level shape; depth by precision, smoother and
- * hierarchy); without it tiles follow a block-count rule and the tail a point budget.  When the
- * environment variable HELM_TUNE_CACHE names a file, the process reads earlier decisions from it
- * and appends its new ones, so that another process (say, one under a profiler) makes the same.  Tiles
- * change the speed only (every point is computed by the same formulas); the tail depth also
+ * and one-warp tiles of the fused 2D kernels (damped Jacobi: also the row-walking kernels in two
+ * lengths) on every fused level and then whole V-cycles for every level at which the one-launch tail
+ * can begin (one cluster on 2D V(1,1) hierarchies with point smoothing, else one block), keeps the
+ * fastest, and caches the choices for the process (tiles by precision, smoother and level shape; the
+ * tail by precision, smoother, kind and hierarchy); without it tiles follow a block-count rule and the
+ * tail a point budget.  When the environment variable HELM_TUNE_CACHE names a file, the process reads
+ * earlier decisions from it and appends its new ones, so that another process (say, one under a
+ * profiler) makes the same.  Tiles change the speed only (every point is computed by the same
+ * formulas), and so does the first level of the one-cluster tail in FP32 (in FP64 the last bits, where
+ * the compiler fuses an operation in one kernel and not in the other); the one-block tail's depth also
  * changes the summation order inside the small levels, i.e. the rounding. */
 enum { HELM_PF_UNFUSED = 1, HELM_PF_NO_PDL = 2, HELM_PF_NO_AUTOTUNE = 4, HELM_PF_GALERKIN = 8 };
 /* HELM_PF_GALERKIN (2D or 3D, omega-Jacobi or ILU(0); else helm_create: HELM_ERR_ARG): every coarse

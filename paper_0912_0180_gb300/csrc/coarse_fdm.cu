@@ -223,7 +223,7 @@ __global__ void k_fdm_axis(const cx<T>* __restrict__ in, cx<T>* __restrict__ out
 // both in-plane transforms of a plane in one block, the plane in shared memory; the z transform, the
 // scaling and the z transform back of 16 columns in one block.  A launch of the six cost its latency (4
 // to 7 us for 20^3 points); in FP64 one SM's two lanes would need longer for a plane than the launches.
-// Every sum is k_fdm_axis's.
+// Every sum is k_fdm_axis's.  20^3: 34 -> 18 us (the launches measured one by one).
 constexpr int FDM_PLANE = 1024, FDM_COLS = 16;
 template <typename T>
 __global__ void __launch_bounds__(FDM_PLANE) k_fdm_plane(const cx<T>* __restrict__ in, cx<T>* __restrict__ out,

@@ -15,6 +15,9 @@
 // most 600 unknowns in FP32 (166 KB of a block's shared memory; reading it there takes 1300 cycles,
 // a level's descent and ascent 5000) and 150 in FP64 (n^2 / 8 cycles of a block's FP64 pipe).
 //
+// Measured (whole V-cycles, us): 96^2 FP32 red-black 24.5 -> 14.0, 640^2 FP32 Jacobi 42 -> 31, FP64 118 ->
+// 108, MP2's Galerkin levels in FP64 109 -> 96.
+//
 // What bounds the kernel is the chain of phases: two cluster barriers and five block barriers a level,
 // and between them one or two points a thread, whose instructions count.
 //
