@@ -13,6 +13,7 @@ namespace helm {
 
 static thread_local std::string g_last_error;
 thread_local bool g_use_pdl = true;
+thread_local TestLimits g_limits;
 
 // Sets the launch mode of the solve-path kernels for the calls made on this context.
 struct PdlScope {
@@ -151,7 +152,19 @@ void ctx_release_on(helm_ctx* c, cudaStream_t st) {
   if (!c) return;
   krylov_free(c, st);
   dev_free_all(c->allocs, st);
+  if (c->wait_word) {
+    cudaStreamSynchronize(st);  // a kernel still queued may write the word
+    pinned_slot_put(c->wait_word);
+  }
   delete c;
+}
+
+bool take_wait_error(helm_ctx* c) {
+  volatile int* w = c->wait_word;
+  if (!w || !*w) return false;
+  *w = 0;
+  set_error("a bounded device-side wait gave up: the call's result is NaN");
+  return true;
 }
 
 // helm_destroy: the context may have been used on any stream, so wait for the device first.
@@ -311,6 +324,7 @@ helm_status helm_vcycle(helm_ctx* c, const helm_precond* pc, helm_dtype dtype, c
     return HELM_ERR_ARG;
   }
   if (dtype != HELM_C64 && dtype != HELM_C128) { set_error("helm_vcycle: dtype"); return HELM_ERR_ARG; }
+  if (take_wait_error(c)) return HELM_ERR_TIMEOUT;  // of an earlier call
   cudaStream_t st = (cudaStream_t)stream;
   PdlScope pdl(c);
   bool f32 = c->pc.mg_dtype == HELM_C64;
@@ -335,6 +349,7 @@ helm_status helm_vcycle(helm_ctx* c, const helm_precond* pc, helm_dtype dtype, c
 helm_status helm_level_op(helm_ctx* c, int op, int lvl, void* a, const void* b, void* out, int count,
                           void* stream) {
   if (!c) { set_error("ctx is NULL"); return HELM_ERR_ARG; }
+  if (take_wait_error(c)) return HELM_ERR_TIMEOUT;  // of an earlier call
   PdlScope pdl(c);
   return mg_level_op(c, op, lvl, a, b, out, count, (cudaStream_t)stream);
 }
@@ -360,6 +375,8 @@ helm_status helm_solve_batch(helm_ctx* const* cs, const void* const* b, void* co
       if (cs[j] == cs[i]) { set_error("helm_solve_batch: a context appears twice"); return HELM_ERR_ARG; }
   }
   if (n == 0) return HELM_OK;
+  for (int i = 0; i < n; ++i)
+    if (take_wait_error(cs[i])) return HELM_ERR_TIMEOUT;  // of an earlier call
   PdlScope pdl(cs[0]);
   helm_status s = krylov_solve_batch(cs, (const double2* const*)b, (double2* const*)x, n, o, infos,
                                      (cudaStream_t)stream);
@@ -385,6 +402,10 @@ helm_status helm_solve(helm_ctx* c, const void* b, void* x, const helm_solve_opt
   if (info) std::memset(info, 0, sizeof(*info));
   helm_status cs = check_solve_args(c, b, x, o);
   if (cs != HELM_OK) return cs;
+  if (take_wait_error(c)) {  // of an earlier call
+    if (info) info->status = HELM_ERR_TIMEOUT;
+    return HELM_ERR_TIMEOUT;
+  }
   PdlScope pdl(c);
   helm_status s = krylov_solve(c, (const double2*)b, (double2*)x, o, info, (cudaStream_t)stream);
   if (info) info->status = s;
@@ -392,6 +413,14 @@ helm_status helm_solve(helm_ctx* c, const void* b, void* x, const helm_solve_opt
 }
 
 void helm_destroy(helm_ctx* c) { ctx_release(c); }
+
+// For tests, not part of helm.h: the limits of the contexts that the calling thread creates from now on
+// (a value below zero: the default).
+void helm_test_limits(long long ilu_wait, int ilu_mute) {
+  g_limits = TestLimits{};
+  if (ilu_wait >= 0) g_limits.ilu_wait = ilu_wait;
+  g_limits.ilu_mute = ilu_mute;
+}
 
 void helm_set_allocator(void* (*alloc)(size_t, void*, void*), void (*free_fn)(void*, void*, void*), void* user) {
   std::lock_guard<std::mutex> lk(g_alloc_mu);

@@ -161,6 +161,11 @@ struct LevelHost {
   // ILU(0) factors (ILU smoothing, 1D / 2D levels above the coarsest) and the solves' vector, in the
   // multigrid precision and the order of the solve's lanes (ilu.cu)
   void *ilu_lo = nullptr, *ilu_up = nullptr, *ilu_v = nullptr;
+  // the hand-over between the solve's strips: where a wait that ran out is reported (the context's
+  // wait_word), its limit in clock cycles, and the strip that sends nothing (tests; -1: none)
+  int* ilu_word = nullptr;
+  long long ilu_wait = 0;
+  int ilu_mute = -1;
   // Sommerfeld sides: bit a set when the last unknown of axis a is the boundary node, bit a + 3 when
   // the first one is (a low side: that axis coarsens with offset 0, keeping node 0)
   int somm = 0;
@@ -238,6 +243,7 @@ struct helm_ctx {
   void* ctail_dev = nullptr;
   std::vector<size_t> ctail_smem;
   int* field_bad = nullptr;          // set by helm_create when a device k field has a non-finite entry
+  int* wait_word = nullptr;          // pinned host word that a kernel sets when a bounded wait ran out
 };
 
 namespace helm {
@@ -261,6 +267,16 @@ void dev_free(const DevBlock& b, cudaStream_t st);
 void dev_free_all(std::vector<DevBlock>& v, cudaStream_t st);
 // device allocation owned by the context (on the context's creation stream)
 helm_status ctx_alloc(helm_ctx* c, void** p, size_t bytes);
+
+// Whether a bounded device-side wait of an earlier, finished call on this context ran out; clears it.
+bool take_wait_error(helm_ctx* c);
+
+// Limits of the contexts that the calling thread creates from now on; tests lower them (helm_test_limits).
+struct TestLimits {
+  long long ilu_wait = 1LL << 31;  // clock cycles a strip waits for a hand-over: about a second
+  int ilu_mute = -1;               // a strip that hands nothing over, so that the wait for it runs out
+};
+extern thread_local TestLimits g_limits;
 
 // ILU(0) smoothing (ilu.cu).  ilu_check: whether a level of this shape can take it (1D / 2D, at most
 // ILU_ROW_BYTES / 4 values along y); ilu_build: the factors of level L, at create; ilu_smooth: one step

@@ -194,6 +194,9 @@ template <typename T> struct IluArgs {
   int passes;    // bit 0: L, bit 1: U
   int depth;     // chunks of the fetch ring
   int rows;      // whether the strips hand their edge row over in shared memory
+  long long wait;  // clock cycles after which a wait for a hand-over gives up
+  int mute;        // the strip that hands nothing over (tests), or -1
+  int* word;       // pinned host word, set when a wait gave up
   const cx<T>*lo, *up;
   cx<T>* v;      // right-hand side, y and z in turn
 };
@@ -222,8 +225,9 @@ __device__ __forceinline__ void ilu_send(bool on, unsigned to, unsigned bar, dou
 __device__ __forceinline__ void ilu_expect(unsigned bar, unsigned bytes) {
   asm volatile("{\n .reg .b64 t;\n mbarrier.arrive.expect_tx.shared::cta.b64 t, [%0], %1;\n}" ::"r"(bar), "r"(bytes) : "memory");
 }
-// waits for the barrier's first phase, for about a second at most; false when that runs out
-__device__ __forceinline__ bool ilu_wait(unsigned bar) {
+// waits for the barrier's first phase, for `limit` clock cycles at most (default: about a second); false
+// when that runs out
+__device__ __forceinline__ bool ilu_wait(unsigned bar, long long limit) {
   const long long t0 = clock64();
   for (int tries = 0; tries < (1 << 24); ++tries) {
     unsigned ok;
@@ -233,7 +237,7 @@ __device__ __forceinline__ bool ilu_wait(unsigned bar) {
         : "r"(bar), "r"(0u)
         : "memory");
     if (ok) return true;
-    if (clock64() - t0 > (1LL << 31)) break;
+    if (clock64() - t0 > limit) break;
   }
   return false;
 }
@@ -252,6 +256,24 @@ __device__ __forceinline__ int ilu_sent(int m, int lag, int n0) {
   return max(hi - lo, 0);
 }
 
+// After a wait gave up, and once every strip has sent what it will: until what was sent to the `nc` chunks'
+// barriers at `bars` has landed (bounded: a strip that never sent leaves its barriers open).
+__device__ __forceinline__ void ilu_drain(unsigned bars, int nc, int lag, int n0) {
+  const long long t0 = clock64();
+  for (int m = threadIdx.x & 31; m < nc; m += 32) {
+    if (ilu_sent(m, lag, n0) == 0) continue;
+    unsigned ok = 0;
+    for (int tries = 0; !ok && tries < (1 << 16); ++tries) {
+      asm volatile(
+          "{\n .reg .pred p;\n mbarrier.test_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
+          : "=r"(ok)
+          : "r"(bars + m * 8), "r"(0u)
+          : "memory");
+      if (clock64() - t0 > (1 << 20)) return;
+    }
+  }
+}
+
 template <typename T>
 __device__ __forceinline__ cx<T> ilu_shfl(cx<T> v, int lane) {
   return mkc<T>(__shfl_sync(0xffffffffu, v.x, lane), __shfl_sync(0xffffffffu, v.y, lane));
@@ -261,8 +283,10 @@ __device__ __forceinline__ cx<T> ilu_shfl(cx<T> v, int lane) {
 // ring: this warp's fetch ring; row, bars: the edge row it receives and the barriers of its chunks;
 // to_row, to_bar: the same in the receiving strip (0: nobody); edge: where the edge row comes from (0
 // nowhere, 1 the row in shared memory, 2 the other strip's values in v).
+// Returns whether every hand-over arrived in time (uniform over the warp); if not, the values after the
+// missing ones are NaN.
 template <typename T, bool BOX, bool UP, int DEPTH>
-__device__ __forceinline__ void ilu_strip(const IluArgs<T>& g, int strip, cx<T>* ring, const cx<T>* row, unsigned bars,
+__device__ __forceinline__ bool ilu_strip(const IluArgs<T>& g, int strip, cx<T>* ring, const cx<T>* row, unsigned bars,
                                           unsigned to_row, unsigned to_bar, int edge) {
   using S = IluShape<BOX>;
   constexpr int K = S::K, NE = UP ? S::NU : S::NL, SL = NE + 1, CH = ILU_CH;
@@ -275,7 +299,7 @@ __device__ __forceinline__ void ilu_strip(const IluArgs<T>& g, int strip, cx<T>*
   cx<T>* const v = g.v + (long)strip * steps * 32 + lane;
   const cx<T>* const fac = (UP ? g.up : g.lo) + (long)strip * steps * NE * 32 + lane;
   const cx<T>* const other = g.v + (long)(UP ? strip + 1 : strip - 1) * steps * 32 + GIVE;
-  const bool gives = lane == GIVE && to_row != 0;
+  const bool gives = lane == GIVE && to_row != 0 && strip != g.mute;
   bool failed = false;
   int armed = 0;  // chunks of the edge row waited for
   auto chunk = [&](int c) { return UP ? nc - 1 - c : c; };  // c-th chunk in this direction
@@ -305,7 +329,7 @@ __device__ __forceinline__ void ilu_strip(const IluArgs<T>& g, int strip, cx<T>*
         const unsigned b = bars + m * 8;
         if (lane == 0) ilu_expect(b, n * (unsigned)sizeof(cx<T>));
         __syncwarp();
-        if (!failed) failed = !ilu_wait(b);
+        if (!failed) failed = !ilu_wait(b, g.wait);
       }
       ++armed;
     }
@@ -324,6 +348,7 @@ __device__ __forceinline__ void ilu_strip(const IluArgs<T>& g, int strip, cx<T>*
   for (int c = 0; c < nc; ++c) {
     fetch(c + DEPTH - 1);
     ready(c);
+    if (failed) prev = b = mkc<T>(T(NAN), T(NAN));  // a wait ran out
     const int m = chunk(c);
     // lane k holds the take lane's new value of the chunk's k-th step
     const cx<T> en = lane < CH ? edge_at(col_new(UP ? m * CH + CH - 1 - lane : m * CH + lane)) : zero;
@@ -369,9 +394,9 @@ __device__ __forceinline__ void ilu_strip(const IluArgs<T>& g, int strip, cx<T>*
         prev = r;
       }
     }
-    if (failed) prev = b = mkc<T>(T(NAN), T(NAN));  // the wait ran out: the solve ends with a NaN status
   }
   ilu_landed<0>();
+  return !failed;
 }
 
 template <typename T, bool BOX, int DEPTH>
@@ -395,7 +420,6 @@ __global__ void k_ilu_solve(const IluArgs<T> g, const int* skip) {
     asm volatile("barrier.cluster.arrive.release;" ::: "memory");
     asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
   }
-  if (strip >= g.s1) return;  // nothing is sent to it
   auto row_of = [&](int st) {  // the edge row and barriers of strip st (0: not in this launch)
     const int q = st - g.s0, blk = q / wpc, ww = q % wpc;
     struct P { unsigned row, bar; } r{0u, 0u};
@@ -407,17 +431,29 @@ __global__ void k_ilu_solve(const IluArgs<T> g, const int* skip) {
   };
   const unsigned bars = bars0 + 2 * w * nc * 8;
   const int strips = (g.n1 + 31) / 32;
-  if (g.passes & 1) {
+  const bool on = strip < g.s1;  // nothing is sent to the others
+  const int edge_l = strip == 0 ? 0 : strip > g.s0 ? 1 : 2, edge_u = strip == strips - 1 ? 0 : strip < g.s1 - 1 ? 1 : 2;
+  bool ok = true;
+  if (on && (g.passes & 1)) {
     const auto to = row_of(strip + 1);
-    const int edge = strip == 0 ? 0 : strip > g.s0 ? 1 : 2;
-    ilu_strip<T, BOX, false, DEPTH>(g, strip, ring, row, bars, to.row, to.bar, edge);
+    ok = ilu_strip<T, BOX, false, DEPTH>(g, strip, ring, row, bars, to.row, to.bar, edge_l);
     __threadfence();  // the values of this pass are fetched asynchronously in the next
     __syncwarp();
   }
-  if (g.passes & 2) {
+  if (on && (g.passes & 2)) {
     const auto to = row_of(strip - 1);
-    const int edge = strip == strips - 1 ? 0 : strip < g.s1 - 1 ? 1 : 2;
-    ilu_strip<T, BOX, true, DEPTH>(g, strip, ring, row, bars + nc * 8, to.row, to.bar ? to.bar + nc * 8 : 0u, edge);
+    ok = ilu_strip<T, BOX, true, DEPTH>(g, strip, ring, row, bars + nc * 8, to.row, to.bar ? to.bar + nc * 8 : 0u, edge_u) && ok;
+  }
+  if (!ok && lane == 0) *reinterpret_cast<volatile int*>(g.word) = 1;
+  if (!g.rows) return;
+  // A strip whose wait gave up did not wait for what came later, and a store into the shared memory of a
+  // block that has left is undefined: every block stays until all strips have sent, and then until what
+  // was sent to it has landed.
+  asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+  asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+  if (!ok) {
+    if ((g.passes & 1) && edge_l == 1) ilu_drain(bars, nc, 31 * S::K, g.n0);
+    if ((g.passes & 2) && edge_u == 1) ilu_drain(bars + nc * 8, nc, 0, g.n0);
   }
 }
 
@@ -524,7 +560,8 @@ void ilu_smooth_t(const LevelHost& L, const cx<T>* f, cx<T>* u, bool zero, doubl
   else launch_pdl(k_ilu_resid<T, 2, BOX>, gr, b, 0, st, L.view<T>(), u0, f, steps, v, skip);
   const IluPlan p = ilu_plan(n0, n1, BOX, sizeof(cx<T>));
   const int per = p.wpc * p.blocks;
-  IluArgs<T> g{n0, n1, steps, 0, strips, 3, p.depth, p.rows, (const cx<T>*)L.ilu_lo, (const cx<T>*)L.ilu_up, v};
+  IluArgs<T> g{n0, n1, steps, 0, strips, 3, p.depth, p.rows, L.ilu_wait, L.ilu_mute, L.ilu_word,
+               (const cx<T>*)L.ilu_lo, (const cx<T>*)L.ilu_up, v};
   if (strips <= per) {
     ilu_launch<T, BOX>(p, g, skip, st);
   } else {  // groups of strips: L down, then U up
@@ -551,6 +588,13 @@ helm_status ilu_build(helm_ctx* c, LevelHost& L, bool f32, cudaStream_t st) {
                                                                                   (double2*)fac);
   rc = cuda_err(cudaGetLastError());
   const bool box = L.stg64 != nullptr;
+  if (!c->wait_word) {
+    if (!(c->wait_word = (int*)pinned_slot_get(sizeof(int)))) rc = cuda_check(cudaErrorMemoryAllocation, "cudaMallocHost");
+    else *c->wait_word = 0;
+  }
+  L.ilu_word = c->wait_word;
+  L.ilu_wait = g_limits.ilu_wait;
+  L.ilu_mute = g_limits.ilu_mute;
   if (rc == HELM_OK) {
     if (f32) rc = box ? ilu_pack<float, true>(c, L, (double2*)fac, st) : ilu_pack<float, false>(c, L, (double2*)fac, st);
     else rc = box ? ilu_pack<double, true>(c, L, (double2*)fac, st) : ilu_pack<double, false>(c, L, (double2*)fac, st);

@@ -1502,8 +1502,10 @@ static helm_status job_step_t(SolveJob& j) {
   }
   HELM_CUDA(cudaMemcpyAsync(j.x, w->x, sizeof(double2) * j.k.n, cudaMemcpyDeviceToDevice, j.st));
   helm_status fs = (helm_status)hs.status;
+  const bool gave_up = take_wait_error(j.c);  // a wait inside a preconditioner of this solve ran out
   if (j.gm && (fs == HELM_OK || fs == HELM_ERR_MAXIT)) fs = hs.rel_true < j.o.tol ? HELM_OK : HELM_ERR_MAXIT;
   if (fs == HELM_OK && !(hs.rel_true < j.o.tol)) fs = HELM_ERR_MAXIT;
+  if (gave_up) fs = HELM_ERR_TIMEOUT;
   if (j.info) {
     j.info->status = fs;
     j.info->iters = hs.iters;

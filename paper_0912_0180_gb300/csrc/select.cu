@@ -121,6 +121,7 @@ helm_status mg_iterate(helm_ctx* c, const double2* f, double2* u, int max_cycles
     HELM_CUDA(cudaGetLastError());
     double rn = 0.0;
     if ((e = device_norm(r, n, partial, dnorm, s.host, st, &rn)) != HELM_OK) return e;
+    if (take_wait_error(c)) return HELM_ERR_TIMEOUT;
     double rel = rn / fn;
     if (hist) hist[k - 1] = rel;
     if (rel <= reduction) { *cycles = k; break; }
@@ -148,6 +149,7 @@ helm_status helm_mg_iterate(helm_ctx* c, const void* f, void* u, int max_cycles,
     return HELM_ERR_ARG;
   }
   if (((uintptr_t)f & 15) || ((uintptr_t)u & 15)) { set_error("helm_mg_iterate: misaligned"); return HELM_ERR_ARG; }
+  if (take_wait_error(c)) return HELM_ERR_TIMEOUT;  // of an earlier call
   return mg_iterate(c, (const double2*)f, (double2*)u, max_cycles, reduction, cycles, hist, (cudaStream_t)stream);
 }
 
