@@ -1,0 +1,56 @@
+"""The FP32 2D cycle's error against 64 bits: the dense operator of the one-cluster tail neither adds more
+rounding than its operands carry, nor takes the cycle further from the exact one than its levels would."""
+import numpy as np
+import pytest
+import torch
+
+import helm_inputs as hi
+from oracle import Oracle
+
+pytestmark = pytest.mark.gpu
+
+U = 2.0 ** -24  # half a unit in the last place of a float
+
+
+@pytest.mark.parametrize("sm", [hi.SM_JACOBI, hi.SM_RBGS])
+@pytest.mark.parametrize("shape", [(26, 26), (22, 31), (14, 14)])
+def test_dense_operator_sum(shape, sm):
+    """The whole cycle is the operator (at most 600 unknowns).  A rounding is 0.42 u in the mean square: the matrix,
+    f and a chain of four products (1 + 2 + 3 + 4 quarters of the sum of squares) make sqrt(4.5) 0.42 u = 0.9 u
+    of the result; one chain over the 18 terms a lane has makes 2.1 u."""
+    from paper_0912_0180_gb300.helm import Helm
+    p = hi.make_problem(2, shape, 0, k0=0.4 * (max(shape) - 1), rhs="zero")
+    pc = hi.Precond(kind=hi.PC_CSG_UNIFORM, theta_beta=0.3, smoother=sm, omega=0.5)
+    h = Helm(p, pc, mg_dtype="c64")
+    # the operator the library holds, in FP64, column by column (a unit vector's cycle is exact)
+    eye = torch.eye(p.n, dtype=torch.complex128, device="cuda")
+    D = np.stack([h.vcycle(eye[q].contiguous(), dtype=torch.complex128).cpu().numpy() for q in range(p.n)], 1)
+    err = []
+    for s in range(8):
+        f = hi.random_vector(p.n, 70 + s)
+        z = h.vcycle(torch.from_numpy(f).cuda(), dtype=torch.complex128).cpu().numpy()
+        err.append(np.linalg.norm(z - D @ f) / np.linalg.norm(D @ f))
+    h.close()
+    assert np.mean(err) <= 1.5 * U, np.mean(err) / U
+
+
+@pytest.mark.parametrize("n_int,sm,kind", [((64, 64), hi.SM_RBGS, "const"), ((64, 64), hi.SM_JACOBI, "const"),
+                                           ((68, 63), hi.SM_JACOBI, "bump"), ((63, 88), hi.SM_RBGS, "bump")])
+def test_cycle_with_the_operator_is_as_exact_as_level_by_level(n_int, sm, kind):
+    """Mean error of 24 inputs with the tail and with one kernel per component on every level; 10 % for the spread of
+    the means (single errors spread by about 10 %, their means by 2 %)."""
+    from paper_0912_0180_gb300.helm import Helm
+    p = hi.make_problem(2, n_int, 16, extent=[1.0, (n_int[1] - 1) / (n_int[0] - 1)], theta_gamma=0.5,
+                        k0=20.0 if kind == "const" else 0.45 * (n_int[0] - 1), phi_kind=kind, rhs="zero")
+    pc = hi.Precond(kind=hi.PC_CSG_UNIFORM, theta_beta=0.3, smoother=sm, omega=0.5)
+    o = Oracle(p, pc)
+    err = []
+    hs = [Helm(p, pc, mg_dtype="c64", fused=f) for f in (True, False)]
+    for s in range(24):
+        r = hi.random_vector(p.n, 80 + s)
+        ref = o.vcycle(r)
+        err.append([np.linalg.norm(h.vcycle(torch.from_numpy(r).cuda()).cpu().numpy() - ref) / np.linalg.norm(ref) for h in hs])
+    for h in hs:
+        h.close()
+    fused, levels = np.mean(err, axis=0)
+    assert fused <= 1.1 * levels, (fused, levels)
