@@ -54,3 +54,49 @@ def test_cycle_with_the_operator_is_as_exact_as_level_by_level(n_int, sm, kind):
         h.close()
     fused, levels = np.mean(err, axis=0)
     assert fused <= 1.1 * levels, (fused, levels)
+
+
+def _perturbed(b, count, seed):
+    rng = np.random.default_rng(seed)
+    for _ in range(count):
+        v = rng.standard_normal(len(b)) + 1j * rng.standard_normal(len(b))
+        yield b + 1e-9 * np.linalg.norm(b) / np.linalg.norm(v) * v
+
+
+def test_fp32_cycle_at_the_edge_of_convergence():
+    """Bi-CGSTAB with the FP32 cycle on a Sommerfeld problem (64 x 39, 1e-7) at the edge of convergence: each right-hand
+    side is one draw, 21 % of which missed their tolerance in 3000 matvecs with one kernel per level.  Of 24 at least 12
+    converge (19 expected, 2 the deviation), each to its true residual, and all do with the FP64 cycle."""
+    from paper_0912_0180_gb300.helm import Helm
+    p = hi.make_problem(2, (65, 33), ((0, -1), (7, 0)), theta_gamma=0.4, k0=14.0, phi_kind="const", rhs="gauss", seed=29)
+    pc = hi.Precond(kind=hi.PC_CSL, shift=1 - 0.5j, smoother=hi.SM_JACOBI, omega=0.5)
+    for mg, need in (("c64", 12), ("c128", 24)):
+        h = Helm(p, pc, mg_dtype=mg)
+        done = 0
+        for b in _perturbed(p.b, 24, 3):
+            _, info = h.solve(torch.from_numpy(b).cuda(), tol=1e-7, maxmv=3000)
+            done += info.status == 0
+            assert info.status != 0 or info.rel_res_true < 1e-7
+        h.close()
+        assert done >= need, (mg, done)
+
+
+def test_fp32_cycle_solution_error_is_the_fp64_cycles():
+    """Error of solutions at tolerance 1e-6 (40 x 29 with layers, Bi-CGSTAB): it is cond(H) tol, whichever precision the
+    cycle has.  Median of 24 right-hand sides; the factor 2 is the spread of one solve's last residual below tol."""
+    from paper_0912_0180_gb300.helm import Helm
+    p = hi.make_problem(2, (40, 29), ((5, 0), (3, 8)), theta_gamma=0.4, k0=12.0, phi_kind="bump", rhs="point",
+                        bump_centre=(0.4, 0.6))
+    pc = hi.Precond(kind=hi.PC_CSG_UNIFORM, theta_beta=0.3, smoother=hi.SM_RBGS)
+    x_ref, _ = Oracle(p, pc).solve(p.b, hi.SolveOpts(method=hi.BICGSTAB, tol=1e-12, maxmv=3000))
+    med = {}
+    for mg in ("c64", "c128"):
+        h = Helm(p, pc, mg_dtype=mg)
+        err = []
+        for b in _perturbed(p.b, 24, 4):
+            x, info = h.solve(torch.from_numpy(b).cuda(), tol=1e-6, maxmv=1500)
+            assert info.status == 0
+            err.append(np.linalg.norm(x.cpu().numpy() - x_ref) / np.linalg.norm(x_ref))
+        h.close()
+        med[mg] = np.median(err)
+    assert med["c64"] <= 2 * med["c128"], med
