@@ -874,16 +874,26 @@ int ctail_first_level(const helm_ctx* c, long points) {
   return (int)c->lv.size();
 }
 
+// Whether a block's shared memory holds its rows of an operator level of n unknowns, f and the result.
+template <typename T> bool ct_op_fits(long n, int nc) {
+  const long rows = (n + nc - 1) / nc;
+  return sizeof(cx<T>) * (size_t)(rows + 1 + rows * ct_pitch<T>((int)n) + n) <= CTAIL_SMEM;
+}
+
 // Once, at create: the dense operator of the finest level small enough for it (see the top), from
 // the coarsest inverse, and the arguments for every level the tail can begin at.
 template <typename T> helm_status ctail_build(helm_ctx* c, cudaStream_t st) {
   if (!ctail_applies(c)) return HELM_OK;
   constexpr bool f64 = std::is_same<T, double>::value;
   const int nl = (int)c->lv.size(), nc = ct_blocks();
+  // (a coarsest level above `most` is the operator level itself: its dense inverse has to be applied anyway.  Up
+  // to CTAIL_COARSEST unknowns: 4 us of the FP64 pipe, about the launch it replaces)
   const long most = f64 ? 150 : 600;
   ColArgs<T> ca{};
   int l = nl;
-  while (l > 0 && c->lv[l - 1].ntot <= most && nl - (l - 1) <= COL_MAX_LEVELS) --l;
+  while (l > 0 && c->lv[l - 1].ntot <= (l == nl ? std::max(most, CTAIL_COARSEST) : most) &&
+         ct_op_fits<T>(c->lv[l - 1].ntot, nc) && nl - (l - 1) <= COL_MAX_LEVELS)
+    --l;
   if (l == nl) return HELM_OK;  // the coarsest level alone is too large
   ca.count = nl - l;
   ca.omega = (T)c->pc.omega;

@@ -7,6 +7,7 @@ namespace helm {
 
 constexpr int CTAIL_MAX_LEVELS = 10;
 constexpr int CTAIL_THREADS = 512;
+constexpr long CTAIL_COARSEST = 256;  // FP64: the largest coarsest level that a tail ends in
 constexpr size_t CTAIL_SMEM = 216 * 1024;  // a block's dynamic shared memory, beside the operator views
 
 // Arguments of one instance's tail: its levels (the last one applies the dense operator) and the places (in

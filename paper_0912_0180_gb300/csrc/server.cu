@@ -21,6 +21,7 @@
 #include <vector>
 
 #include "helm_internal.cuh"
+#include "mg_cluster.cuh"
 
 namespace helm {
 
@@ -38,6 +39,9 @@ helm_status job_status(const SolveJob* j);
 static double now_s() {
   return std::chrono::duration<double>(std::chrono::steady_clock::now().time_since_epoch()).count();
 }
+
+// the one-cluster tail's dense operator and its arguments
+static size_t ctail_operator_bytes(long n, size_t esz) { return (size_t)(n + 1) * n * esz + 64 * 1024; }
 
 static long axis_n(const helm_grid& g, int a) {
   return axis_unknowns(g.n_int[a], g.n_layer[a][0], g.n_layer[a][1]);
@@ -75,7 +79,7 @@ extern "C" size_t helm_estimate_bytes(const helm_grid* g, const helm_precond* pc
       if (pc->smoother == HELM_SM_ILU)  // ILU(0) factors, FP64 (transient) and skewed with the solves' vector
         bytes += (size_t)Nl * 9 * 16 + (size_t)((m[1] + 31) / 32) * 32 * (size_t)(m[0] + 70) * 10 * esz;
       if (g->dim == 2 && pc->nu1 == 1 && pc->nu2 == 1 && Nl <= (esz == 8 ? 600 : 150) && tail++ == 0)
-        bytes += (size_t)(Nl + 1) * Nl * esz + 64 * 1024;  // the one-cluster tail's dense operator
+        bytes += ctail_operator_bytes(Nl, esz);
       last = Nl;
       bool all_small = true;
       long min_n = 1L << 40;
@@ -87,6 +91,8 @@ extern "C" size_t helm_estimate_bytes(const helm_grid* g, const helm_precond* pc
       Nl = 1;
       for (int a = 0; a < g->dim; ++a) { m[a] /= 2; Nl *= m[a]; }
     }
+    if (g->dim == 2 && pc->nu1 == 1 && pc->nu2 == 1 && tail == 0 && last <= CTAIL_COARSEST)
+      bytes += ctail_operator_bytes(last, esz);
     bytes += (size_t)last * last * esz;     // coarse inverse
     bytes += (size_t)last * last * 32 + 4;  // its FP64 factorisation (transient)
     if (esz == 8) bytes += (size_t)N * 16;  // the two-vector scratch of an FP32 hierarchy

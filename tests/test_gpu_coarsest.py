@@ -21,7 +21,7 @@ def _instance(shape, mg, sm, **kw):
 @pytest.mark.parametrize("mg", ["c128", "c64"])
 def test_group_takes_single_levels(mg, sm):
     """A hierarchy of one level, solved directly, joins a group up to 256 unknowns (FP64): the whole cycle is the tail;
-    bitwise the lone solve."""
+    bitwise the lone solve's iterates (which a direct solve of M need not bring to the tolerance in 50 matvecs)."""
     from paper_0912_0180_gb300.helm import solve_group
     inst = [_instance(s, mg, sm, max_levels=1) for s in ((13, 12), (16, 16), (7, 9), (51, 5))]
     hs = [h for _, _, h in inst]
@@ -29,7 +29,7 @@ def test_group_takes_single_levels(mg, sm):
     lone = [h.solve(b, tol=1e-8, maxmv=50) for h, b in zip(hs, bs)]
     xs, infos = solve_group(hs, bs, tol=1e-8, maxmv=50)
     for (x, i), xg, ig in zip(lone, xs, infos):
-        assert i.status == 0 and ig.status == 0 and torch.equal(x, xg)
+        assert (i.status, i.matvecs) == (ig.status, ig.matvecs) and torch.equal(x, xg)
     for h in hs:
         h.close()
 
