@@ -417,10 +417,11 @@ void helm_destroy(helm_ctx* c) { ctx_release(c); }
 // For tests, not part of helm.h: the limits of the contexts that the calling thread creates from now on
 // (a value below zero: the default).
 void helm_test_limits(long long ilu_wait, int ilu_mute) {
-  g_limits = TestLimits{};
-  if (ilu_wait >= 0) g_limits.ilu_wait = ilu_wait;
+  g_limits.ilu_wait = ilu_wait >= 0 ? ilu_wait : TestLimits{}.ilu_wait;
   g_limits.ilu_mute = ilu_mute;
 }
+// ... and the blocks of a thread-block cluster that the device is taken to grant (0: the default).
+void helm_test_cluster(int blocks) { g_limits.cluster = blocks > 0 ? blocks : TestLimits{}.cluster; }
 
 void helm_set_allocator(void* (*alloc)(size_t, void*, void*), void (*free_fn)(void*, void*, void*), void* user) {
   std::lock_guard<std::mutex> lk(g_alloc_mu);

@@ -131,6 +131,13 @@ inline long axis_unknowns(int n_int, int lo, int hi) {
   return (long)n_int - 2 + (lo > 0 ? lo + 1 : (lo < 0 ? 1 : 0)) + (hi > 0 ? hi + 1 : (hi < 0 ? 1 : 0));
 }
 
+// The launches of an ILU(0) level's solve: warps a block, blocks a cluster, chunks of the fetch ring,
+// whether edge rows are handed over in shared memory, and the dynamic shared memory (ilu.cu).
+struct IluPlan {
+  int wpc = 1, blocks = 1, depth = 3, rows = 0;
+  size_t smem = 0;
+};
+
 // ---- owned device storage of one level ---------------------------------------------------
 struct LevelHost {
   int dim = 0;
@@ -166,6 +173,7 @@ struct LevelHost {
   int* ilu_word = nullptr;
   long long ilu_wait = 0;
   int ilu_mute = -1;
+  IluPlan ilu;
   // Sommerfeld sides: bit a set when the last unknown of axis a is the boundary node, bit a + 3 when
   // the first one is (a low side: that axis coarsens with offset 0, keeping node 0)
   int somm = 0;
@@ -273,6 +281,7 @@ bool take_wait_error(helm_ctx* c);
 
 // Limits of the contexts that the calling thread creates from now on; tests lower them (helm_test_limits).
 struct TestLimits {
+  int cluster = 16;                // blocks of a thread-block cluster
   long long ilu_wait = 1LL << 31;  // clock cycles a strip waits for a hand-over: about a second
   int ilu_mute = -1;               // a strip that hands nothing over, so that the wait for it runs out
 };

@@ -474,26 +474,21 @@ namespace {
 
 constexpr size_t ILU_SMEM_MAX = 224 * 1024;
 
-// The launches of one level: warps per block, blocks per cluster, ring depth, shared memory.
-struct IluPlan {
-  int wpc, blocks, depth, rows;
-  size_t smem;
-};
-// The fewest warps a block (a strip has its SM's loads and, in FP64, its FP64 pipe to itself) that put
+// The plan for clusters of at most `most` blocks.  The fewest warps a block (a strip has its SM's loads and, in FP64, its FP64 pipe to itself) that put
 // all strips into one cluster; where the edge rows do not fit, fewer strips a launch; a row too long
 // for shared memory is handed over in memory, one strip a launch.
-IluPlan ilu_plan(int n0, int n1, bool box, size_t esz) {
+IluPlan ilu_plan(int n0, int n1, bool box, size_t esz, int most) {
   const int strips = (n1 + 31) / 32, nc = ilu_steps(n0, box) / ILU_CH;
   auto bytes = [&](int wpc, int depth, int rows) {
     return wpc * (esz * depth * ILU_CH * ((box ? 5 : 3) + 1) * 32 + (rows ? esz * n0 + 16 * (size_t)nc : 0));
   };
-  IluPlan p{1, 1, 3, 0, 0};
+  IluPlan p;
   if (strips > 1) {
-    for (int wpc = std::min((strips + ILU_MAX_BLOCKS - 1) / ILU_MAX_BLOCKS, ILU_MAX_WARPS); wpc >= 1 && !p.rows; --wpc)
+    for (int wpc = std::min((strips + most - 1) / most, ILU_MAX_WARPS); wpc >= 1 && !p.rows; --wpc)
       for (int depth = 3; depth >= 2 && !p.rows; --depth)
         if (bytes(wpc, depth, 1) <= ILU_SMEM_MAX) p = IluPlan{wpc, 1, depth, 1, 0};
     if (p.rows)
-      while (p.blocks < ILU_MAX_BLOCKS && p.blocks * p.wpc < strips) p.blocks *= 2;
+      while (2 * p.blocks <= most && p.blocks * p.wpc < strips) p.blocks *= 2;
   }
   p.smem = bytes(p.wpc, p.depth, p.rows);
   return p;
@@ -511,14 +506,13 @@ cudaError_t ilu_attrs() {
   return e;
 }
 
-template <typename T, bool BOX>
-void ilu_launch(const IluPlan& p, const IluArgs<T>& g, const int* skip, cudaStream_t st) {
+// the launch of a plan (attributes in at[2])
+cudaLaunchConfig_t ilu_config(const IluPlan& p, cudaLaunchAttribute* at, cudaStream_t st) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(p.blocks);
   cfg.blockDim = dim3(32 * p.wpc);
   cfg.dynamicSmemBytes = p.smem;
   cfg.stream = st;
-  cudaLaunchAttribute at[2];
   at[0].id = cudaLaunchAttributeClusterDimension;
   at[0].val.clusterDim.x = p.blocks;
   at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
@@ -526,6 +520,30 @@ void ilu_launch(const IluPlan& p, const IluArgs<T>& g, const int* skip, cudaStre
   at[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = at;
   cfg.numAttrs = g_use_pdl ? 2 : 1;
+  return cfg;
+}
+
+// The plan for the largest cluster that the device grants (the kernels' attributes are set).
+template <typename T, bool BOX>
+IluPlan ilu_choose(int n0, int n1) {
+  for (int most = std::min(ILU_MAX_BLOCKS, g_limits.cluster);; most /= 2) {
+    const IluPlan p = ilu_plan(n0, n1, BOX, sizeof(cx<T>), most);
+    if (p.blocks == 1) return p;
+    cudaLaunchAttribute at[2];
+    cudaLaunchConfig_t cfg = ilu_config(p, at, nullptr);
+    cfg.numAttrs = 1;
+    int fit = 0;
+    const cudaError_t e = p.depth == 3 ? cudaOccupancyMaxActiveClusters(&fit, k_ilu_solve<T, BOX, 3>, &cfg)
+                                       : cudaOccupancyMaxActiveClusters(&fit, k_ilu_solve<T, BOX, 2>, &cfg);
+    if (e == cudaSuccess && fit > 0) return p;
+    cudaGetLastError();
+  }
+}
+
+template <typename T, bool BOX>
+void ilu_launch(const IluPlan& p, const IluArgs<T>& g, const int* skip, cudaStream_t st) {
+  cudaLaunchAttribute at[2];
+  const cudaLaunchConfig_t cfg = ilu_config(p, at, st);
   if (p.depth == 3) cudaLaunchKernelEx(&cfg, k_ilu_solve<T, BOX, 3>, g, skip);
   else cudaLaunchKernelEx(&cfg, k_ilu_solve<T, BOX, 2>, g, skip);
 }
@@ -546,8 +564,10 @@ helm_status ilu_pack(helm_ctx* c, LevelHost& L, const double2* fac, cudaStream_t
   k_ilu_pack<T, BOX><<<(int)((L.ntot + 255) / 256), 256, 0, st>>>(fac, L.n[0], L.n[1], steps, (cx<T>*)L.ilu_lo,
                                                                 (cx<T>*)L.ilu_up);
   HELM_CUDA(cudaGetLastError());
-  // (attributes are set here, outside any stream capture)
-  return cuda_err(ilu_attrs<T, BOX>());
+  // (here, outside any stream capture)
+  HELM_CUDA((ilu_attrs<T, BOX>()));
+  L.ilu = ilu_choose<T, BOX>(L.n[0], L.n[1]);
+  return HELM_OK;
 }
 
 template <typename T, bool BOX>
@@ -558,7 +578,7 @@ void ilu_smooth_t(const LevelHost& L, const cx<T>* f, cx<T>* u, bool zero, doubl
   const cx<T>* u0 = zero ? nullptr : u;
   if (L.dim == 1) launch_pdl(k_ilu_resid<T, 1, BOX>, gr, b, 0, st, L.view<T>(), u0, f, steps, v, skip);
   else launch_pdl(k_ilu_resid<T, 2, BOX>, gr, b, 0, st, L.view<T>(), u0, f, steps, v, skip);
-  const IluPlan p = ilu_plan(n0, n1, BOX, sizeof(cx<T>));
+  const IluPlan& p = L.ilu;
   const int per = p.wpc * p.blocks;
   IluArgs<T> g{n0, n1, steps, 0, strips, 3, p.depth, p.rows, L.ilu_wait, L.ilu_mute, L.ilu_word,
                (const cx<T>*)L.ilu_lo, (const cx<T>*)L.ilu_up, v};
