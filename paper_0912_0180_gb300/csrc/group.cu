@@ -158,6 +158,9 @@ const char* group_refusal(const helm_ctx* c, const helm_ctx* c0, int dev) {
   if (c->pc.flags & (HELM_PF_UNFUSED | HELM_PF_GALERKIN)) return "grouped solves need the fused rediscretised levels";
   if (c->fdm.on) return "grouped solves need a dense coarsest inverse";
   if (!c->lv.empty() && c->lv[0].any_offset0()) return "grouped solves do not take Sommerfeld low sides";
+  if (c->tail_first < (int)c->lv.size() &&
+      (c->tail_first >= (int)c->ctail_smem.size() || !c->ctail_smem[c->tail_first] || c->ctail_blocks != c0->ctail_blocks))
+    return "grouped solves need the thread-block cluster of the one-launch tail, one size for all";
   if ((int)c->lv.size() < 2 && c->tail_first > 0) return "grouped solves need at least two levels";
   if (c->pc.smoother == HELM_SM_ILU) return "grouped solves smooth with damped Jacobi or red-black Gauss-Seidel";
   if (c->pc.smoother != c0->pc.smoother) return "the instances of a group share one smoother kind";

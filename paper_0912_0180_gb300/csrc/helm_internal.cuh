@@ -247,6 +247,7 @@ struct helm_ctx {
   // one-cluster tail (mg_cluster.cu): operator level and its matrix; the arguments for each level it
   // can begin at, and the dynamic shared memory each needs (0: it cannot)
   int ctail_op = -1;
+  int ctail_blocks = 0;  // blocks of its cluster; 0: none granted
   void* ctail_dense = nullptr;
   void* ctail_dev = nullptr;
   std::vector<size_t> ctail_smem;

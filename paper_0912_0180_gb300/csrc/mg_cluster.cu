@@ -616,7 +616,7 @@ cudaError_t ct_prepare_all() {
 
 // Blocks per cluster on the current device, with the kernels' attributes set (outside any capture:
 // the hierarchy's setup asks first): 16 where a cluster of 16 such blocks fits, else the portable 8.
-int ct_blocks() {
+int ct_granted() {
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
   static std::mutex mu;
@@ -649,6 +649,12 @@ int ct_blocks() {
     cudaGetLastError();
   }
   return 0;
+}
+
+// the same under the thread's test limit
+int ct_blocks() {
+  const int nc = ct_granted();
+  return nc <= g_limits.cluster ? nc : g_limits.cluster >= 8 ? 8 : 0;
 }
 
 template <typename... KArgs, typename... Args>
@@ -864,7 +870,7 @@ __global__ void __launch_bounds__(COL_THREADS) k_ctail_columns(const __grid_cons
 bool ctail_applies(const helm_ctx* c) {
   return c->grid.dim == 2 && c->pc.nu1 == 1 && c->pc.nu2 == 1 && !(c->pc.flags & HELM_PF_UNFUSED) &&
          (c->pc.smoother == HELM_SM_JACOBI || c->pc.smoother == HELM_SM_RBGS) && !c->lv.empty() &&
-         !c->lv[0].any_offset0() && !c->fdm.on && ct_blocks() > 0;
+         !c->lv[0].any_offset0() && !c->fdm.on && c->ctail_blocks > 0;
 }
 
 int ctail_first_level(const helm_ctx* c, long points) {
@@ -883,9 +889,10 @@ template <typename T> bool ct_op_fits(long n, int nc) {
 // Once, at create: the dense operator of the finest level small enough for it (see the top), from
 // the coarsest inverse, and the arguments for every level the tail can begin at.
 template <typename T> helm_status ctail_build(helm_ctx* c, cudaStream_t st) {
+  c->ctail_blocks = ct_blocks();
   if (!ctail_applies(c)) return HELM_OK;
   constexpr bool f64 = std::is_same<T, double>::value;
-  const int nl = (int)c->lv.size(), nc = ct_blocks();
+  const int nl = (int)c->lv.size(), nc = c->ctail_blocks;
   // (a coarsest level above `most` is the operator level itself: its dense inverse has to be applied anyway.  Up
   // to CTAIL_COARSEST unknowns: 4 us of the FP64 pipe, about the launch it replaces)
   const long most = f64 ? 150 : 600;
@@ -937,7 +944,7 @@ helm_status ctail_vcycle(const helm_ctx* c, int first, const cx<TI>* f, void* ou
     return HELM_ERR_ARG;
   }
   const bool rb = c->pc.smoother == HELM_SM_RBGS;
-  const int nc = ct_blocks();
+  const int nc = c->ctail_blocks;
   if (out_f64) {
     if (rb) launch_cluster(k_ctail<T, true, double, TI>, nc, nc, smem, st, a, f, (double2*)out, skip);
     else launch_cluster(k_ctail<T, false, double, TI>, nc, nc, smem, st, a, f, (double2*)out, skip);
@@ -950,9 +957,9 @@ helm_status ctail_vcycle(const helm_ctx* c, int first, const cx<TI>* f, void* ou
 }
 
 template <typename T>
-void ctail_group(const GCTail<T>* args, const GroupList* LT, int li, int instances, bool rb, bool out_f64, size_t smem,
-                 cudaStream_t st) {
-  const int nc = ct_blocks(), grid = instances * nc;
+void ctail_group(const GCTail<T>* args, const GroupList* LT, int li, int instances, int nc, bool rb, bool out_f64,
+                 size_t smem, cudaStream_t st) {
+  const int grid = instances * nc;
   if (out_f64) {
     if (rb) launch_cluster(kg_ctail<T, true, double>, grid, nc, smem, st, args, LT, li);
     else launch_cluster(kg_ctail<T, false, double>, grid, nc, smem, st, args, LT, li);
@@ -969,7 +976,7 @@ template size_t ctail_args<double>(const helm_ctx*, int, const CTailArgs<double>
 template helm_status ctail_vcycle<float, double>(const helm_ctx*, int, const double2*, void*, bool, const int*, cudaStream_t);
 template helm_status ctail_vcycle<float, float>(const helm_ctx*, int, const float2*, void*, bool, const int*, cudaStream_t);
 template helm_status ctail_vcycle<double, double>(const helm_ctx*, int, const double2*, void*, bool, const int*, cudaStream_t);
-template void ctail_group<float>(const GCTail<float>*, const GroupList*, int, int, bool, bool, size_t, cudaStream_t);
-template void ctail_group<double>(const GCTail<double>*, const GroupList*, int, int, bool, bool, size_t, cudaStream_t);
+template void ctail_group<float>(const GCTail<float>*, const GroupList*, int, int, int, bool, bool, size_t, cudaStream_t);
+template void ctail_group<double>(const GCTail<double>*, const GroupList*, int, int, int, bool, bool, size_t, cudaStream_t);
 
 }  // namespace helm

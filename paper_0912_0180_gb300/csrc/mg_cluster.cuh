@@ -45,7 +45,7 @@ template <typename T, typename TI>
 helm_status ctail_vcycle(const helm_ctx* c, int first, const cx<TI>* f, void* out, bool out_f64, const int* skip,
                          cudaStream_t st);
 template <typename T>
-void ctail_group(const GCTail<T>* args, const GroupList* LT, int li, int instances, bool rb, bool out_f64, size_t smem,
-                 cudaStream_t st);
+void ctail_group(const GCTail<T>* args, const GroupList* LT, int li, int instances, int nc, bool rb, bool out_f64,
+                 size_t smem, cudaStream_t st);
 
 }  // namespace helm

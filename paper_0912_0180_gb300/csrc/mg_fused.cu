@@ -983,6 +983,7 @@ __global__ void kg_coarse(const GCoarse<T>* __restrict__ A, const GroupList* __r
 
 struct GroupVcycle {
   bool rb = false;
+  int nc = 0;  // blocks a cluster of the tails
   struct Launch {
     void* args = nullptr;  // device array of descriptors
     int li = -1;           // its work list
@@ -1018,6 +1019,7 @@ helm_status group_vcycle_build(helm_ctx* const* cs, int ni, const void* const* i
   *plan = nullptr;
   auto* P = new GroupVcycle();
   P->rb = cs[0]->pc.smoother == HELM_SM_RBGS;
+  P->nc = cs[0]->ctail_blocks;
   std::vector<int> tf(ni), stop(ni);
   int lmax = 0;
   for (int i = 0; i < ni; ++i) {
@@ -1075,6 +1077,11 @@ helm_status group_vcycle_build(helm_ctx* const* cs, int ni, const void* const* i
     if (tf[i] < nl) {
       GCTail<T> g;
       const size_t sm = ctail_args<T>(c, tf[i], &g.a);
+      if (!sm) {  // (group_refusal turns these away)
+        set_error("a grouped V-cycle's tail needs a thread-block cluster");
+        group_vcycle_free(P, st);
+        return HELM_ERR_ARG;
+      }
       g.skip = skip[i];
       if (tf[i] == 0) {
         g.f = (const cx<T>*)in[i];
@@ -1192,7 +1199,7 @@ static void group_vcycle_enqueue_t(const GroupVcycle* P, cudaStream_t st) {
     for (const auto& L : P->down[l]) group_down_launch<T, RB>(L, LT, st);
   for (const GroupVcycle::Launch* L : {&P->tail0, &P->tailk})
     if (L->li >= 0)
-      ctail_group<T>((const GCTail<T>*)L->args, LT, L->li, L->grid, RB, L == &P->tail0, L->smem, st);
+      ctail_group<T>((const GCTail<T>*)L->args, LT, L->li, L->grid, P->nc, RB, L == &P->tail0, L->smem, st);
   if (P->coarse.li >= 0)
     launch_pdl(kg_coarse<T>, dim3(P->coarse.grid), dim3(256), 0, st, (const GCoarse<T>*)P->coarse.args, LT,
                P->coarse.li);
