@@ -220,7 +220,8 @@ typedef struct helm_ctx helm_ctx;
  * and 2D grids whose finest level has at most 7,264 (complex64) or 3,632 (complex128) rows along
  * y, else HELM_ERR_ARG.  A smoothing step's two triangular solves are one launch of one thread-block
  * cluster, strips of 32 rows pipelined over its blocks; their n0 + 2 n1 (9-point levels) or n0 + n1
- * (5-point) steps are sequential, so the V-cycle is slower than with the point smoothers.  A strip waits
+ * (5-point) steps are sequential, so the V-cycle is slower than with the point smoothers.  A level holds 10
+ * (9-point) or 6 values an unknown, its rows counted in strips of 32 (fewer than 32: as they are).  A strip waits
  * about a second at most for the strip before it; should that run out, the step's result is NaN, a call
  * that synchronises (helm_solve, helm_solve_batch, helm_mg_iterate) returns HELM_ERR_TIMEOUT, and after
  * one that does not (helm_vcycle, helm_level_op) the next call on the context returns it. */

@@ -119,13 +119,15 @@ template <bool BOX> struct IluShape {
   static constexpr int NL = BOX ? 4 : 2;  // L's entries a point
   static constexpr int NU = BOX ? 5 : 3;  // U's, and the pivot's reciprocal first
 };
-__host__ __device__ inline int ilu_steps(int n0, bool box) {  // a strip's steps, whole chunks
-  return (n0 + 31 * (box ? 2 : 1) + ILU_CH - 1) / ILU_CH * ILU_CH;
+// stored rows of a strip: a level of fewer than 32 rows (a 1D level has one) stores only those
+__host__ __device__ inline int ilu_width(int n1) { return n1 < 32 ? n1 : 32; }
+__host__ __device__ inline int ilu_steps(int n0, int n1, bool box) {  // a strip's steps, whole chunks
+  return (n0 + (ilu_width(n1) - 1) * (box ? 2 : 1) + ILU_CH - 1) / ILU_CH * ILU_CH;
 }
-// place of point (i, j) in a skewed vector (entry e of `per` entries a point)
-__host__ __device__ inline long ilu_at(int i, int j, int steps, int k, int per, int e) {
+// place of point (i, j) in a skewed vector (entry e of `per` entries a point) of width w
+__host__ __device__ inline long ilu_at(int i, int j, int steps, int k, int per, int e, int w) {
   const int l = j & 31;
-  return (((long)(j >> 5) * steps + i + k * l) * per + e) * 32 + l;
+  return (((long)(j >> 5) * steps + i + k * l) * per + e) * w + l;
 }
 
 // Packs the natural factors for the solve: lo = L's entries, up = 1 / u_pp and U's entries times it.
@@ -137,13 +139,14 @@ __global__ void k_ilu_pack(const double2* __restrict__ f, int n0, int n1, int st
   if (p >= (long)n0 * n1) return;
   const int i = (int)(p % n0), j = (int)(p / n0);
   const double2* a = f + 9 * p;
+  const int w = ilu_width(n1);
   const int sl[4] = {BOX ? 0 : 1, BOX ? 1 : 3, 2, 3}, su[4] = {5, BOX ? 6 : 7, 7, 8};
 #pragma unroll
-  for (int e = 0; e < S::NL; ++e) lo[ilu_at(i, j, steps, S::K, S::NL, e)] = cconv<T, double>(a[sl[e]]);
-  up[ilu_at(i, j, steps, S::K, S::NU, 0)] = cconv<T, double>(a[4]);
+  for (int e = 0; e < S::NL; ++e) lo[ilu_at(i, j, steps, S::K, S::NL, e, w)] = cconv<T, double>(a[sl[e]]);
+  up[ilu_at(i, j, steps, S::K, S::NU, 0, w)] = cconv<T, double>(a[4]);
 #pragma unroll
   for (int e = 1; e < S::NU; ++e)
-    up[ilu_at(i, j, steps, S::K, S::NU, e)] = cconv<T, double>(cmul<double>(a[4], a[su[e - 1]]));
+    up[ilu_at(i, j, steps, S::K, S::NU, e, w)] = cconv<T, double>(cmul<double>(a[4], a[su[e - 1]]));
 }
 
 // v = f - M u (or f, from the zero guess) in the skewed order of the solve.
@@ -170,7 +173,7 @@ __global__ void k_ilu_resid(OpView<T> op, const cx<T>* __restrict__ u, const cx<
       r = csub<T>(r, op_row<T, T, DIM>(op, u, i, j, 0, p));
     }
   }
-  v[ilu_at(i, j, steps, IluShape<BOX>::K, 1, 0)] = r;
+  v[ilu_at(i, j, steps, IluShape<BOX>::K, 1, 0, ilu_width(op.n[1]))] = r;
 }
 
 // u += z (u = z from the zero guess), z skewed; wide: u also as complex128.
@@ -182,7 +185,7 @@ __global__ void k_ilu_add(int n0, int n1, int steps, const cx<T>* __restrict__ z
   const int i = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y * blockDim.y + threadIdx.y;
   if (i >= n0 || j >= n1) return;
   const long p = i + (long)n0 * j;
-  const cx<T> d = z[ilu_at(i, j, steps, IluShape<BOX>::K, 1, 0)];
+  const cx<T> d = z[ilu_at(i, j, steps, IluShape<BOX>::K, 1, 0, ilu_width(n1))];
   const cx<T> r = zero ? d : cadd<T>(u[p], d);
   u[p] = r;
   if (wide) wide[p] = cconv<double, T>(r);
@@ -283,9 +286,10 @@ __device__ __forceinline__ cx<T> ilu_shfl(cx<T> v, int lane) {
 // ring: this warp's fetch ring; row, bars: the edge row it receives and the barriers of its chunks;
 // to_row, to_bar: the same in the receiving strip (0: nobody); edge: where the edge row comes from (0
 // nowhere, 1 the row in shared memory, 2 the other strip's values in v).
+// FEW: the level's only strip, of fewer than 32 rows.
 // Returns whether every hand-over arrived in time (uniform over the warp); if not, the values after the
 // missing ones are NaN.
-template <typename T, bool BOX, bool UP, int DEPTH>
+template <typename T, bool BOX, bool UP, int DEPTH, bool FEW>
 __device__ __forceinline__ bool ilu_strip(const IluArgs<T>& g, int strip, cx<T>* ring, const cx<T>* row, unsigned bars,
                                           unsigned to_row, unsigned to_bar, int edge) {
   using S = IluShape<BOX>;
@@ -296,22 +300,23 @@ __device__ __forceinline__ bool ilu_strip(const IluArgs<T>& g, int strip, cx<T>*
   const int n0 = g.n0, steps = g.steps, nc = steps / CH;
   const bool has_row = strip * 32 + lane < g.n1;
   const cx<T> zero = mkc<T>(T(0), T(0));
-  cx<T>* const v = g.v + (long)strip * steps * 32 + lane;
-  const cx<T>* const fac = (UP ? g.up : g.lo) + (long)strip * steps * NE * 32 + lane;
+  const int W = FEW ? g.n1 : 32;
+  cx<T>* const v = g.v + (long)strip * steps * W + lane;
+  const cx<T>* const fac = (UP ? g.up : g.lo) + (long)strip * steps * NE * W + lane;
   const cx<T>* const other = g.v + (long)(UP ? strip + 1 : strip - 1) * steps * 32 + GIVE;
   const bool gives = lane == GIVE && to_row != 0 && strip != g.mute;
   bool failed = false;
   int armed = 0;  // chunks of the edge row waited for
   auto chunk = [&](int c) { return UP ? nc - 1 - c : c; };  // c-th chunk in this direction
   auto fetch = [&](int c) {
-    if (c < nc) {
+    if (c < nc && (!FEW || has_row)) {
       cx<T>* const to = ring + (c % DEPTH) * CH * SL * 32 + lane;
       const long t0 = (long)chunk(c) * CH;
 #pragma unroll
       for (int k = 0; k < CH; ++k) {
 #pragma unroll
-        for (int e = 0; e < NE; ++e) ilu_fetch(to + (k * SL + e) * 32, fac + ((t0 + k) * NE + e) * 32);
-        ilu_fetch(to + (k * SL + NE) * 32, v + (t0 + k) * 32);
+        for (int e = 0; e < NE; ++e) ilu_fetch(to + (k * SL + e) * 32, fac + ((t0 + k) * NE + e) * W);
+        ilu_fetch(to + (k * SL + NE) * 32, v + (t0 + k) * W);
       }
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
@@ -387,7 +392,7 @@ __device__ __forceinline__ bool ilu_strip(const IluArgs<T>& g, int strip, cx<T>*
         }
         const bool in = has_row && i >= 0 && i < n0;
         if (!in) r = zero;  // a point outside the grid is zero for the neighbours
-        else v[(long)t * 32] = r;
+        else v[(long)t * W] = r;
         ilu_send(gives && in, to_row + (unsigned)(i * (int)sizeof(cx<T>)), to_bar + m * 8, r);
         a = b;
         b = nw;
@@ -399,7 +404,7 @@ __device__ __forceinline__ bool ilu_strip(const IluArgs<T>& g, int strip, cx<T>*
   return !failed;
 }
 
-template <typename T, bool BOX, int DEPTH>
+template <typename T, bool BOX, int DEPTH, bool FEW>
 __global__ void k_ilu_solve(const IluArgs<T> g, const int* skip) {
   pdl_entry();
   if (skip && *skip) return;
@@ -436,13 +441,13 @@ __global__ void k_ilu_solve(const IluArgs<T> g, const int* skip) {
   bool ok = true;
   if (on && (g.passes & 1)) {
     const auto to = row_of(strip + 1);
-    ok = ilu_strip<T, BOX, false, DEPTH>(g, strip, ring, row, bars, to.row, to.bar, edge_l);
+    ok = ilu_strip<T, BOX, false, DEPTH, FEW>(g, strip, ring, row, bars, to.row, to.bar, edge_l);
     __threadfence();  // the values of this pass are fetched asynchronously in the next
     __syncwarp();
   }
   if (on && (g.passes & 2)) {
     const auto to = row_of(strip - 1);
-    ok = ilu_strip<T, BOX, true, DEPTH>(g, strip, ring, row, bars + nc * 8, to.row, to.bar ? to.bar + nc * 8 : 0u, edge_u) && ok;
+    ok = ilu_strip<T, BOX, true, DEPTH, FEW>(g, strip, ring, row, bars + nc * 8, to.row, to.bar ? to.bar + nc * 8 : 0u, edge_u) && ok;
   }
   if (!ok && lane == 0) *reinterpret_cast<volatile int*>(g.word) = 1;
   if (!g.rows) return;
@@ -478,7 +483,7 @@ constexpr size_t ILU_SMEM_MAX = 224 * 1024;
 // all strips into one cluster; where the edge rows do not fit, fewer strips a launch; a row too long
 // for shared memory is handed over in memory, one strip a launch.
 IluPlan ilu_plan(int n0, int n1, bool box, size_t esz, int most) {
-  const int strips = (n1 + 31) / 32, nc = ilu_steps(n0, box) / ILU_CH;
+  const int strips = (n1 + 31) / 32, nc = ilu_steps(n0, n1, box) / ILU_CH;
   auto bytes = [&](int wpc, int depth, int rows) {
     return wpc * (esz * depth * ILU_CH * ((box ? 5 : 3) + 1) * 32 + (rows ? esz * n0 + 16 * (size_t)nc : 0));
   };
@@ -501,8 +506,9 @@ cudaError_t ilu_attrs() {
     if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ILU_SMEM_MAX);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
   };
-  one(k_ilu_solve<T, BOX, 2>);
-  one(k_ilu_solve<T, BOX, 3>);
+  one(k_ilu_solve<T, BOX, 2, false>);
+  one(k_ilu_solve<T, BOX, 3, false>);
+  one(k_ilu_solve<T, BOX, 3, true>);
   return e;
 }
 
@@ -533,8 +539,8 @@ IluPlan ilu_choose(int n0, int n1) {
     cudaLaunchConfig_t cfg = ilu_config(p, at, nullptr);
     cfg.numAttrs = 1;
     int fit = 0;
-    const cudaError_t e = p.depth == 3 ? cudaOccupancyMaxActiveClusters(&fit, k_ilu_solve<T, BOX, 3>, &cfg)
-                                       : cudaOccupancyMaxActiveClusters(&fit, k_ilu_solve<T, BOX, 2>, &cfg);
+    const cudaError_t e = p.depth == 3 ? cudaOccupancyMaxActiveClusters(&fit, k_ilu_solve<T, BOX, 3, false>, &cfg)
+                                       : cudaOccupancyMaxActiveClusters(&fit, k_ilu_solve<T, BOX, 2, false>, &cfg);
     if (e == cudaSuccess && fit > 0) return p;
     cudaGetLastError();
   }
@@ -544,15 +550,16 @@ template <typename T, bool BOX>
 void ilu_launch(const IluPlan& p, const IluArgs<T>& g, const int* skip, cudaStream_t st) {
   cudaLaunchAttribute at[2];
   const cudaLaunchConfig_t cfg = ilu_config(p, at, st);
-  if (p.depth == 3) cudaLaunchKernelEx(&cfg, k_ilu_solve<T, BOX, 3>, g, skip);
-  else cudaLaunchKernelEx(&cfg, k_ilu_solve<T, BOX, 2>, g, skip);
+  if (g.n1 < 32) cudaLaunchKernelEx(&cfg, k_ilu_solve<T, BOX, 3, true>, g, skip);  // (one strip: depth 3)
+  else if (p.depth == 3) cudaLaunchKernelEx(&cfg, k_ilu_solve<T, BOX, 3, false>, g, skip);
+  else cudaLaunchKernelEx(&cfg, k_ilu_solve<T, BOX, 2, false>, g, skip);
 }
 
 template <typename T, bool BOX>
 helm_status ilu_pack(helm_ctx* c, LevelHost& L, const double2* fac, cudaStream_t st) {
   using S = IluShape<BOX>;
-  const int steps = ilu_steps(L.n[0], BOX), strips = (L.n[1] + 31) / 32;
-  const size_t pts = (size_t)strips * steps * 32;
+  const int steps = ilu_steps(L.n[0], L.n[1], BOX), strips = (L.n[1] + 31) / 32;
+  const size_t pts = (size_t)strips * steps * ilu_width(L.n[1]);
   helm_status rc;
   if ((rc = ctx_alloc(c, &L.ilu_lo, sizeof(cx<T>) * S::NL * pts)) != HELM_OK) return rc;
   if ((rc = ctx_alloc(c, &L.ilu_up, sizeof(cx<T>) * S::NU * pts)) != HELM_OK) return rc;
@@ -572,7 +579,7 @@ helm_status ilu_pack(helm_ctx* c, LevelHost& L, const double2* fac, cudaStream_t
 
 template <typename T, bool BOX>
 void ilu_smooth_t(const LevelHost& L, const cx<T>* f, cx<T>* u, bool zero, double2* wide, const int* skip, cudaStream_t st) {
-  const int n0 = L.n[0], n1 = L.n[1], steps = ilu_steps(n0, BOX), strips = (n1 + 31) / 32;
+  const int n0 = L.n[0], n1 = L.n[1], steps = ilu_steps(n0, n1, BOX), strips = (n1 + 31) / 32;
   cx<T>* const v = (cx<T>*)L.ilu_v;
   const dim3 b(32, 8), gr((n0 + 31) / 32, (n1 + 7) / 8);
   const cx<T>* u0 = zero ? nullptr : u;

@@ -76,8 +76,10 @@ extern "C" size_t helm_estimate_bytes(const helm_grid* g, const helm_precond* pc
       bytes += (size_t)Nl * (8 + 4 + 2 * esz + (levels == 1 ? 1 : 3) * esz);
       if (levels > 1 && (pc->flags & HELM_PF_GALERKIN))  // the stencil, FP64 and the V-cycle precision
         bytes += (size_t)Nl * (g->dim == 3 ? 27 : 9) * (16 + (esz == 8 ? 8 : 0)) + (size_t)Nl * 8;
-      if (pc->smoother == HELM_SM_ILU)  // ILU(0) factors, FP64 (transient) and skewed with the solves' vector
-        bytes += (size_t)Nl * 9 * 16 + (size_t)((m[1] + 31) / 32) * 32 * (size_t)(m[0] + 70) * 10 * esz;
+      if (pc->smoother == HELM_SM_ILU) {  // ILU(0) factors, FP64 (transient) and skewed with the solves' vector
+        const long rows = m[1] < 32 ? m[1] : (m[1] + 31) / 32 * 32, skew = m[1] < 32 ? m[1] - 1 : 31;
+        bytes += (size_t)Nl * 9 * 16 + (size_t)rows * (size_t)(m[0] + 2 * skew + 8) * 10 * esz;
+      }
       if (g->dim == 2 && pc->nu1 == 1 && pc->nu2 == 1 && Nl <= (esz == 8 ? 600 : 150) && tail++ == 0)
         bytes += ctail_operator_bytes(Nl, esz);
       last = Nl;
