@@ -142,8 +142,9 @@ typedef struct {
  * limits such levels to HELM_COARSE_MAX_UNKNOWNS unknowns (4 GiB in FP64 during create). */
 #define HELM_COARSE_MAX_UNKNOWNS 16384
 
-/* helm_precond.flags: HELM_PF_UNFUSED runs every V-cycle component as its own kernel (the
- * same arithmetic as the default fused kernels; for testing the fusion); HELM_PF_NO_PDL
+/* helm_precond.flags: HELM_PF_UNFUSED runs every V-cycle component as its own kernel (for testing the
+ * fusion: the same formulas; in FP32 the rounding can differ, in 2D since the fused rows sum each axis apart
+ * and the tail applies the smallest levels as one matrix); HELM_PF_NO_PDL
  * launches the solve-path kernels without programmatic dependent launch (same kernels);
  * HELM_PF_NO_AUTOTUNE skips the autotuner of helm_create, which times the large, small, square, wide
  * and one-warp tiles of the fused 2D kernels (damped Jacobi: also the row-walking kernels in two

@@ -852,8 +852,8 @@ __global__ void __launch_bounds__(128) k_restrict3z(Dims d, const cx<T>* __restr
 // value needs the black points around it only, and the residual itself never goes to memory.  A lane
 // owns the fine pair (2t, 2t + 1) -- coarse column t -- of the fine rows 2J .. 2J + 2 and walks the
 // planes; V(k, p) is the black value of its pair in row 2J - 1 + k, plane p.  Per point the arithmetic
-// is that of the RESID sweep and of k_restrict, so the result is bitwise theirs (the products' fused
-// forms spelled out as the compiler chose them there).  30 coarse columns a
+// is that of the RESID sweep and of k_restrict, so the result is bitwise theirs where k_rbgs3z2 sweeps (the
+// products' fused forms spelled out as the compiler chose them there; in k_rbgs3z it fuses another).  30 coarse columns a
 // warp (the outer lanes are the halo).  With u_c it also runs the red half of the coarse level's sweep
 // from the zero guess, whose f it has just made.  160^3 level: 10.4 + 14.9 us in two kernels and 4.1 for
 // the coarse red half, 15.9 us together (bound by the latency of a thread's chain of planes).
@@ -1511,7 +1511,7 @@ static void vcycle_unfused(helm_ctx* c, int l, const cx<T>* f, cx<T>* out, const
     bool done = false;
     if constexpr (std::is_same<T, float>::value) {
       float2* uc = C.xs && l + 1 < nl - 1 ? (float2*)C.u : nullptr;
-      done = pc.nu1 == 1 && pc.smoother == HELM_SM_RBGS && resrest3z(L, C, b[cur], fc, uc, skip, st);
+      done = pc.nu1 == 1 && pc.smoother == HELM_SM_RBGS && !(pc.flags & HELM_PF_UNFUSED) && resrest3z(L, C, b[cur], fc, uc, skip, st);
       red_next = done && uc;
     }
     // residual into the spare buffer; after a single sweep from zero without the diagonal
@@ -1592,7 +1592,7 @@ helm_status mg_vcycle_from_c128(helm_ctx* c, const double2* r, void* buf, void* 
     return HELM_OK;
   }
   const LevelHost& L0 = c->lv[0];
-  if (L0.xs && c->pc.nu1 > 0) {  // (x-split levels smooth with red-black Gauss-Seidel)
+  if (L0.xs && c->pc.nu1 > 0 && !(c->pc.flags & HELM_PF_UNFUSED)) {  // (x-split levels smooth with red-black Gauss-Seidel)
     const long rows = L0.ntot / L0.n[0];
     const int gy = (int)std::min<long>(rows, 65535), h = (L0.n[0] + 1) / 2;
     const int thr = std::min(128, (h + 31) / 32 * 32);
