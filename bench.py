@@ -482,7 +482,8 @@ def main():
 
 
 # Algorithmic cost of the fused first half of a V(1,1) level (smoothing sweep from the zero guess,
-# residual, full weighting), per fine unknown: reads f and omega/D, writes u, writes a quarter of a
+# residual, full weighting) as the level operation runs it, per fine unknown: reads f and omega/D, writes
+# u (which the FP32 cycle's own kernel leaves to the up kernel: 18 instead of 26 B), writes a quarter of a
 # coarse value; flops: u = f (omega/D) (complex multiply, 6), residual (1 - omega) f - a (sum of
 # four neighbours) (3 complex adds, 1 complex multiply, 1 scale, 1 subtract: 16), full weighting
 # (8 complex adds and a scale per coarse unknown: 18 / 4).
@@ -574,7 +575,7 @@ def kernel_rooflines(torch, L, ctxs, p, dev, flush) -> dict:
                 "note": "DADD, DMUL and DFMA each take one FP64-pipe slot; ncu: the FP64 pipe is 76-80% busy over "
                         "active cycles, DRAM reads = the algorithmic reads (f and omega/D; writes stay in L2); "
                         "executed FP64 lane slots 22-33 per fine point against 20.5 algorithmic (halo, partial warps)"}
-    fp32 = {"kernel": "k_down2d<float> (same kernel in the FP32 V-cycle)", "bound": "hbm",
+    fp32 = {"kernel": "k_down2d<float> storing its iterate (the FP32 V-cycle's own instance stores none)", "bound": "hbm",
             "achieved": d32["GB/s"], "peak": hbm, "unit": "GB/s", "frac": d32["GB/s"] / hbm,
             "traffic": DOWN_TRAFFIC_BYTES["c64"],
             "peak_source": hbm_src, "bytes_per_launch": d32["bytes"], "launch_us": d32["us"]}

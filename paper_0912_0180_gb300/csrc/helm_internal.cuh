@@ -400,6 +400,8 @@ helm_status tail_vcycle(helm_ctx* c, int first, const cx<T>* f, void* out, bool 
                         cudaStream_t st);
 template <typename T, typename TI>
 void fused_down2d(const helm_ctx* c, int l, const cx<TI>* f, cx<T>* u_out, cx<T>* fc, const int* skip, cudaStream_t st);
+template <typename T>
+void fused_down2d_stored(const helm_ctx* c, int l, const cx<T>* f, cx<T>* u_out, cx<T>* fc, cudaStream_t st);
 template <typename T, typename TI>
 void fused_up2d(const helm_ctx* c, int l, const cx<T>* u_in, const cx<T>* ec, const cx<TI>* f, void* out,
                 bool out_f64, const int* skip, cudaStream_t st);

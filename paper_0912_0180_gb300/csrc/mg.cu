@@ -1675,9 +1675,7 @@ static helm_status level_op_t(helm_ctx* c, int op, int lvl, void* a, const void*
     case HELM_OP_DOWN:
       if (lvl >= nl - 1 || L.dim != 2 || c->pc.nu1 != 1 || L.stg64 || L.any_offset0() || !A || !B || !O)
         return HELM_ERR_ARG;
-      fused_down2d<T, T>(c, lvl, B, A, O, nullptr, st);
-      // (FP32 damped Jacobi: the fused kernel leaves the iterate to the up kernel)
-      if (std::is_same<T, float>::value && c->pc.smoother != HELM_SM_RBGS) o.jacobi(nullptr, B, A, (T)c->pc.omega, nullptr, st);
+      fused_down2d_stored<T>(c, lvl, B, A, O, st);
       break;
     default: return HELM_ERR_ARG;
   }

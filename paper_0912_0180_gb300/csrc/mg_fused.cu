@@ -77,7 +77,8 @@ template <typename T, bool RBGS> constexpr bool keeps_u() { return RBGS || sizeo
 // vector, narrowed as it is read (no conversion pass).  NINE: a Galerkin level's 9-point rows (damped
 // Jacobi; they were three kernels down and two up: at 256^2 in FP64 16 -> 12 and 14 -> 11 us, the MP2 cycle
 // 100.7 -> 93.7 us).
-template <typename T, bool RBGS, int CX, int CY, int NT, typename TI, bool NINE = false>
+// KEEP: the iterate is stored (the level operation HELM_OP_DOWN stores it in every case).
+template <typename T, bool RBGS, int CX, int CY, int NT, typename TI, bool NINE = false, bool KEEP = keeps_u<T, RBGS>()>
 __device__ __forceinline__ void down2d_body(int bx_, int by_, const OpView<T>& op, int nc0, int nc1, const cx<TI>* __restrict__ f, cx<T>* __restrict__ u_out,
          cx<T>* __restrict__ fc, T omega) {
   constexpr int HF = RBGS ? 2 : 1;
@@ -137,7 +138,7 @@ __device__ __forceinline__ void down2d_body(int bx_, int by_, const OpView<T>& o
   }
   // write the smoothed iterate of the points this tile owns (the last tile also owns the
   // fine point past the last coarse node when n is odd)
-  if constexpr (keeps_u<T, RBGS>()) {
+  if constexpr (KEEP) {
     const int oi1 = (I0 + CX >= nc0) ? n0 : 2 * (I0 + CX);
     const int oj1 = (J0 + CY >= nc1) ? n1 : 2 * (J0 + CY);
     const int wx = oi1 - 2 * I0, wy = oj1 - 2 * J0;
@@ -198,14 +199,14 @@ __device__ __forceinline__ void down2d_body(int bx_, int by_, const OpView<T>& o
     fc[I + nc0 * J] = cscale<T>(T(0.0625), acc);
   }
 }
-template <typename T, bool RBGS, int CX, int CY, int NT, typename TI, bool NINE = false>
+template <typename T, bool RBGS, int CX, int CY, int NT, typename TI, bool NINE = false, bool KEEP = keeps_u<T, RBGS>()>
 __global__ void __launch_bounds__(NT)
 k_down2d(OpView<T> op, int nc0, int nc1, const cx<TI>* __restrict__ f, cx<T>* __restrict__ u_out,
          cx<T>* __restrict__ fc, T omega, const int* skip, int early) {
   if (early) pdl_trigger();
   pdl_entry();
   if (skip && *skip) return;
-  down2d_body<T, RBGS, CX, CY, NT, TI, NINE>(blockIdx.x, blockIdx.y, op, nc0, nc1, f, u_out, fc, omega);
+  down2d_body<T, RBGS, CX, CY, NT, TI, NINE, KEEP>(blockIdx.x, blockIdx.y, op, nc0, nc1, f, u_out, fc, omega);
 }
 
 // ---- up: prolongation + correction + post-smoothing (2D, nu2 = 1), out of place --------------
@@ -359,14 +360,14 @@ k_up2d(OpView<T> op, int nc0, int nc1, const cx<T>* __restrict__ u_in, const cx<
 }
 
 // ---- the row-walking kernels (damped Jacobi) ---------------------------------------------------
-template <typename T, typename TI, int CR>
+template <typename T, typename TI, int CR, bool KEEP>
 __global__ void __launch_bounds__(MARCH_THREADS)
 k_march_down(OpView<T> op, int nc0, int nc1, const cx<TI>* __restrict__ f, cx<T>* __restrict__ u_out,
              cx<T>* __restrict__ fc, T omega, int vec, const int* skip, int early) {
   if (early) pdl_trigger();
   pdl_entry();
   if (skip && *skip) return;
-  march_down<T, TI, CR, keeps_u<T, false>()>(blockIdx.x, blockIdx.y, op, nc0, nc1, f, u_out, fc, omega, vec != 0);
+  march_down<T, TI, CR, KEEP>(blockIdx.x, blockIdx.y, op, nc0, nc1, f, u_out, fc, omega, vec != 0);
 }
 template <typename T, typename TO, typename TI, int CR>
 __global__ void __launch_bounds__(MARCH_THREADS)
@@ -722,11 +723,11 @@ static bool big_tiles(const helm_ctx* c, long blocks) {
   return blocks >= 2L * sms;
 }
 
-template <typename T, bool RB, int CX, int CY, int NT, typename TI, bool NINE = false>
+template <typename T, bool RB, int CX, int CY, int NT, typename TI, bool NINE = false, bool KEEP = keeps_u<T, RB>()>
 static void down_launch(const LevelHost& F, const LevelHost& C, const cx<TI>* f, cx<T>* u_out, cx<T>* fc, T om,
                         const int* skip, cudaStream_t st, int early) {
   dim3 g((C.n[0] + CX - 1) / CX, (C.n[1] + CY - 1) / CY);
-  launch_pdl(k_down2d<T, RB, CX, CY, NT, TI, NINE>, dim3(g), dim3(NT), 0, st, F.view<T>(), C.n[0], C.n[1], f, u_out, fc, om, skip,
+  launch_pdl(k_down2d<T, RB, CX, CY, NT, TI, NINE, KEEP>, dim3(g), dim3(NT), 0, st, F.view<T>(), C.n[0], C.n[1], f, u_out, fc, om, skip,
              early);
 }
 
@@ -737,11 +738,11 @@ static int march_vec(const LevelHost& F, const void* f, const void* b) {
   if (sizeof(T) != 4) return 0;
   return F.n[0] % 2 == 0 && ((((uintptr_t)f | (uintptr_t)b | (uintptr_t)F.dinv32) & 15) == 0);
 }
-template <typename T, int CR, typename TI>
+template <typename T, int CR, typename TI, bool KEEP>
 static void march_down_launch(const LevelHost& F, const LevelHost& C, const cx<TI>* f, cx<T>* u_out, cx<T>* fc, T om,
                               const int* skip, cudaStream_t st, int early) {
   dim3 g(march_strips((F.n[0] + 1) / 2), (C.n[1] + CR - 1) / CR);
-  launch_pdl(k_march_down<T, TI, CR>, g, dim3(MARCH_THREADS), 0, st, F.view<T>(), C.n[0], C.n[1], f, u_out, fc, om,
+  launch_pdl(k_march_down<T, TI, CR, KEEP>, g, dim3(MARCH_THREADS), 0, st, F.view<T>(), C.n[0], C.n[1], f, u_out, fc, om,
              march_vec<T>(F, f, u_out), skip, early);
 }
 template <typename T, typename TO, int CR, typename TI>
@@ -752,18 +753,18 @@ static void march_up_launch(const LevelHost& F, const LevelHost& C, const cx<T>*
              (cx<TO>*)out, om, march_vec<T>(F, f, out), skip);
 }
 
-template <typename T, bool RB, typename TI = T>
+template <typename T, bool RB, typename TI = T, bool KEEP = keeps_u<T, RB>()>
 static void down_tile(int tile, const LevelHost& F, const LevelHost& C, const cx<TI>* f, cx<T>* u_out, cx<T>* fc, T om,
                       const int* skip, cudaStream_t st, int early = 0) {
   if constexpr (!RB) {
-    if (tile == TILE_LONG) return march_down_launch<T, MARCH_LONG, TI>(F, C, f, u_out, fc, om, skip, st, early);
-    if (tile == TILE_SHORT) return march_down_launch<T, MARCH_SHORT, TI>(F, C, f, u_out, fc, om, skip, st, early);
+    if (tile == TILE_LONG) return march_down_launch<T, MARCH_LONG, TI, KEEP>(F, C, f, u_out, fc, om, skip, st, early);
+    if (tile == TILE_SHORT) return march_down_launch<T, MARCH_SHORT, TI, KEEP>(F, C, f, u_out, fc, om, skip, st, early);
   }
-  if (tile == TILE_BIG) down_launch<T, RB, DN_CX, DN_CY, FUSED_THREADS, TI>(F, C, f, u_out, fc, om, skip, st, early);
-  else if (tile == TILE_TINY) down_launch<T, RB, DN_TCX, DN_TCY, FUSED_TINY_THREADS, TI>(F, C, f, u_out, fc, om, skip, st, early);
-  else if (tile == TILE_SQUARE) down_launch<T, RB, DN_QCX, DN_QCY, FUSED_SMALL_THREADS, TI>(F, C, f, u_out, fc, om, skip, st, early);
-  else if (tile == TILE_WIDE) down_launch<T, RB, DN_WCX, DN_WCY, FUSED_THREADS, TI>(F, C, f, u_out, fc, om, skip, st, early);
-  else down_launch<T, RB, DN_SCX, DN_SCY, FUSED_SMALL_THREADS, TI>(F, C, f, u_out, fc, om, skip, st, early);
+  if (tile == TILE_BIG) down_launch<T, RB, DN_CX, DN_CY, FUSED_THREADS, TI, false, KEEP>(F, C, f, u_out, fc, om, skip, st, early);
+  else if (tile == TILE_TINY) down_launch<T, RB, DN_TCX, DN_TCY, FUSED_TINY_THREADS, TI, false, KEEP>(F, C, f, u_out, fc, om, skip, st, early);
+  else if (tile == TILE_SQUARE) down_launch<T, RB, DN_QCX, DN_QCY, FUSED_SMALL_THREADS, TI, false, KEEP>(F, C, f, u_out, fc, om, skip, st, early);
+  else if (tile == TILE_WIDE) down_launch<T, RB, DN_WCX, DN_WCY, FUSED_THREADS, TI, false, KEEP>(F, C, f, u_out, fc, om, skip, st, early);
+  else down_launch<T, RB, DN_SCX, DN_SCY, FUSED_SMALL_THREADS, TI, false, KEEP>(F, C, f, u_out, fc, om, skip, st, early);
 }
 
 // The tile a level's fused kernels use (the autotuner's choice, else the block-count rule) and the
@@ -825,6 +826,16 @@ void fused_down2d(const helm_ctx* c, int l, const cx<TI>* f, cx<T>* u_out, cx<T>
   }
   if (c->pc.smoother == HELM_SM_RBGS) down_tile<T, true, TI>(tile, F, C, f, u_out, fc, om, skip, st, early);
   else down_tile<T, false, TI>(tile, F, C, f, u_out, fc, om, skip, st, early);
+}
+
+// the level operation: the tile's kernel with the iterate stored
+template <typename T>
+void fused_down2d_stored(const helm_ctx* c, int l, const cx<T>* f, cx<T>* u_out, cx<T>* fc, cudaStream_t st) {
+  int bx, by;
+  const int tile = down_tile_of(c, l, &bx, &by);
+  const T om = (T)c->pc.omega;
+  if (c->pc.smoother == HELM_SM_RBGS) down_tile<T, true, T, true>(tile, c->lv[l], c->lv[l + 1], f, u_out, fc, om, nullptr, st);
+  else down_tile<T, false, T, true>(tile, c->lv[l], c->lv[l + 1], f, u_out, fc, om, nullptr, st);
 }
 
 template <typename T, bool RB, typename TO, int FX, int FY, int NT, typename TI, bool NINE = false>
@@ -1433,6 +1444,8 @@ template int tail_first_level<float>(const helm_ctx*);
 template int tail_first_level<double>(const helm_ctx*);
 template helm_status tail_vcycle<float>(helm_ctx*, int, const float2*, void*, bool, const int*, cudaStream_t);
 template helm_status tail_vcycle<double>(helm_ctx*, int, const double2*, void*, bool, const int*, cudaStream_t);
+template void fused_down2d_stored<float>(const helm_ctx*, int, const float2*, float2*, float2*, cudaStream_t);
+template void fused_down2d_stored<double>(const helm_ctx*, int, const double2*, double2*, double2*, cudaStream_t);
 template void fused_down2d<float, float>(const helm_ctx*, int, const float2*, float2*, float2*, const int*, cudaStream_t);
 template void fused_down2d<float, double>(const helm_ctx*, int, const double2*, float2*, float2*, const int*, cudaStream_t);
 template void fused_down2d<double, double>(const helm_ctx*, int, const double2*, double2*, double2*, const int*, cudaStream_t);
