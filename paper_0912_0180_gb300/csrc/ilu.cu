@@ -195,7 +195,6 @@ template <typename T> struct IluArgs {
   int n0, n1, steps;
   int s0, s1;    // strips of this launch, one after another over its blocks' warps
   int passes;    // bit 0: L, bit 1: U
-  int depth;     // chunks of the fetch ring
   int rows;      // whether the strips hand their edge row over in shared memory
   long long wait;  // clock cycles after which a wait for a hand-over gives up
   int mute;        // the strip that hands nothing over (tests), or -1
@@ -587,7 +586,7 @@ void ilu_smooth_t(const LevelHost& L, const cx<T>* f, cx<T>* u, bool zero, doubl
   else launch_pdl(k_ilu_resid<T, 2, BOX>, gr, b, 0, st, L.view<T>(), u0, f, steps, v, skip);
   const IluPlan& p = L.ilu;
   const int per = p.wpc * p.blocks;
-  IluArgs<T> g{n0, n1, steps, 0, strips, 3, p.depth, p.rows, L.ilu_wait, L.ilu_mute, L.ilu_word,
+  IluArgs<T> g{n0, n1, steps, 0, strips, 3, p.rows, L.ilu_wait, L.ilu_mute, L.ilu_word,
                (const cx<T>*)L.ilu_lo, (const cx<T>*)L.ilu_up, v};
   if (strips <= per) {
     ilu_launch<T, BOX>(p, g, skip, st);

@@ -703,7 +703,7 @@ __device__ __forceinline__ int interp1(int i, int nc, int o, int* ci) {
   return k;
 }
 
-// u += P ec (or u = P ec when overwrite), bilinear / trilinear interpolation.  All terms of a fine
+// u += P ec (or u = P ec when overwrite), linear / bilinear interpolation (1D, 2D).  All terms of a fine
 // point carry the same weight (1/2 per even axis), so they are summed first and scaled once.
 template <typename T, int DIM>
 __global__ void k_prolong(Dims d, const cx<T>* __restrict__ ec, cx<T>* __restrict__ u, int overwrite,
@@ -712,23 +712,19 @@ __global__ void k_prolong(Dims d, const cx<T>* __restrict__ ec, cx<T>* __restric
   if (skip && *skip) return;
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   int j = blockIdx.y * blockDim.y + threadIdx.y;
-  int l = blockIdx.z;
   if (i >= d.f[0] || j >= d.f[1]) return;
-  int ci[2], cj[2] = {0, 0}, cl[2] = {0, 0};
+  int ci[2], cj[2] = {0, 0};
   int ni = interp1(i, d.c[0], d.o[0], ci);
   int nj = DIM > 1 ? interp1(j, d.c[1], d.o[1], cj) : 1;
-  int nl = DIM > 2 ? interp1(l, d.c[2], d.o[2], cl) : 1;
   auto on_coarse = [](int x, int o) { return x - o >= 0 && !((x - o) & 1); };
   T w = on_coarse(i, d.o[0]) ? T(1) : T(0.5);
   if (DIM > 1 && !on_coarse(j, d.o[1])) w *= T(0.5);
-  if (DIM > 2 && !on_coarse(l, d.o[2])) w *= T(0.5);
   cx<T> acc = mkc<T>(T(0), T(0));
-  for (int c3 = 0; c3 < nl; ++c3)
-    for (int c2 = 0; c2 < nj; ++c2) {
-      const cx<T>* row = ec + (long)d.c[0] * (cj[c2] + (long)d.c[1] * cl[c3]);
-      for (int c1 = 0; c1 < ni; ++c1) acc = cadd<T>(acc, row[xpos(ci[c1], d.ch)]);
-    }
-  long p = xpos(i, d.fh) + (long)d.f[0] * (j + (long)d.f[1] * l);
+  for (int c2 = 0; c2 < nj; ++c2) {
+    const cx<T>* row = ec + (long)d.c[0] * cj[c2];
+    for (int c1 = 0; c1 < ni; ++c1) acc = cadd<T>(acc, row[ci[c1]]);
+  }
+  long p = i + (long)d.f[0] * j;
   if (overwrite) u[p] = cscale<T>(w, acc);
   else {
     cx<T> uo = u[p];
@@ -738,8 +734,8 @@ __global__ void k_prolong(Dims d, const cx<T>* __restrict__ ec, cx<T>* __restric
 
 // Trilinear prolongation in natural order, a thread per pair of columns (2t, 2t + 1): no lane runs the other
 // parity's sums, and in FP64 the two points share the sums over their common coarse column (1.75 complex
-// additions a point; k_prolong's lanes paid for 4.5; 129 x 145 x 113 points: 67 -> 49 us).  FP32 adds in k_prolong's
-// order, bit for bit its result; so does BLACK, which corrects only the black points, before a red-black
+// additions a point; a lane a point paid for 4.5; 129 x 145 x 113 points: 67 -> 49 us).  FP32 adds planes, rows and
+// columns in ascending order, as a lane a point does; so does BLACK, which corrects only the black points, before a red-black
 // sweep (whose red half overwrites the red ones): one column a row, the same for all its lanes.
 template <typename T, bool BLACK>
 __global__ void __launch_bounds__(128) k_prolong3p(Dims d, const cx<T>* __restrict__ ec, cx<T>* __restrict__ u,
@@ -969,7 +965,7 @@ __global__ void __launch_bounds__(128) k_resrest3z(OpView<float> op, Dims d, con
 // Trilinear prolongation onto an x-split fine level: thread (t, j) owns the fine pair (2t, 2t + 1)
 // of row j and walks fine planes [l0, l1).  The pair reads coarse columns a = t - o and a + 1, the
 // row coarse rows jA (and jB); the coarse values of the two coarse planes a fine plane can need
-// stay in registers.  Every fine point sums its coarse values in k_prolong's order (lower plane,
+// stay in registers.  Every fine point sums its coarse values in that order too (lower plane,
 // row, column first) and scales once.
 // BLACK: only the black points, before a red-black sweep (whose red half overwrites the red points from
 // the black ones): half the bytes and sums (160^3 level 26 -> 16 us).
@@ -1011,7 +1007,7 @@ __global__ void __launch_bounds__(128) k_prolong3z(Dims d, const cx<T>* __restri
   };
   const T wy = yon ? T(1) : T(0.5);
   const T wxe = o0 ? T(0.5) : T(1), wxo = o0 ? T(1) : T(0.5);
-  // the coarse values of one fine point in k_prolong's order: planes, rows, columns ascending
+  // the coarse values of one fine point: planes, rows, columns ascending
   auto point = [&](const Cp& A, const Cp& B, bool two, bool odd) -> cx<T> {
     cx<T> acc = zero;
     // the even column uses {a, a + 1} when o = 1, {a} when o = 0; the odd one {a + 1} / {a, a + 1}
