@@ -12,8 +12,8 @@
 // right-hand side, is applied as what it is, one dense matrix (built at create from the levels'
 // operators in FP64 arithmetic, one block per column), split by rows over the blocks.  That replaces a
 // chain of some twenty dependent phases of a few hundred points by one.  The level is the finest one with
-// at most 600 unknowns in FP32 (166 KB of a block's shared memory; reading it there takes 1300 cycles, the
-// compensated sums 1900, a level's descent and ascent 5000) and 150 in FP64 (n^2 / 8 cycles of a block's
+// at most 600 unknowns in FP32 (166 KB of a block's shared memory; reading it there takes 1300 cycles,
+// a level's descent and ascent 5000) and 150 in FP64 (n^2 / 8 cycles of a block's
 // FP64 pipe).
 //
 // Measured (whole V-cycles, us): 96^2 FP32 red-black 24.5 -> 14.0, 640^2 FP32 Jacobi 42 -> 31, FP64 118 ->
@@ -135,11 +135,6 @@ __device__ __forceinline__ unsigned long long f2_add(unsigned long long a, unsig
   asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
   return r;
 }
-__device__ __forceinline__ unsigned long long f2_mul(unsigned long long a, unsigned long long b) {
-  unsigned long long r;
-  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
 __device__ __forceinline__ unsigned long long f2_fma(unsigned long long a, unsigned long long b, unsigned long long c) {
   unsigned long long r;
   asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
@@ -168,6 +163,7 @@ struct Sum2 {
     return r;
   }
 };
+constexpr int SUM_TERMS = 4;  // complex products of a partial sum
 // hi + lo; an overflowed sum stays infinite (its lo is not a number)
 __device__ __forceinline__ float sum2_value(float hi, float lo) { return isinf(hi) ? hi : hi + lo; }
 
@@ -379,18 +375,25 @@ __device__ __forceinline__ void ctail_body(const CTailArgs<T>* __restrict__ ga, 
       const cx<T>* row2 = two ? row + NW * a.pitch : row;
       const cx<T>* row3 = three ? row + 2 * NW * a.pitch : row;
       if constexpr (sizeof(T) == 4) {
-        // FP32: every product is added to a sum of two floats.  A plain sum's roundings were 4 times those of the
-        // matrix and f (1.2e-7 of the result against 0.33e-7) and put cycles of 96^2 unknowns up to 24 % further
-        // from the exact ones than a cycle of levels; partial sums of 4 terms left 6 %.  Against the plain sum
-        // 0.6 us a cycle (the 96^2 solve 3640 -> 3720 us).
+        // FP32: partial sums of SUM_TERMS products, added up in sums of two floats.  One chain over the 18 products
+        // that a lane has made 4 times the rounding of the matrix and f (1.2e-7 of the result against 0.33e-7).  Over
+        // 50 cycles of 63^2 to 420^2 unknowns the error against 64 bits falls by 5 % and in none rises by more than
+        // 2 %, for 0.3 to 0.5 us (96^2 red-black 11.8 -> 12.3 us); one product at a time: 8 % for 1.6 us.
         Sum2 s[3];
-#pragma unroll 2
-        for (int c = lane; c < nop; c += 32) {
-          const float2 f = fl[c], r0 = row[c], r1 = row2[c], r2 = row3[c];
-          const unsigned long long ff = f2_pack(f.x, f.y), fi = f2_pack(-f.y, f.x);
-          s[0].add(f2_fma(f2_pack(r0.x, r0.x), ff, f2_mul(f2_pack(r0.y, r0.y), fi)));
-          if (two) s[1].add(f2_fma(f2_pack(r1.x, r1.x), ff, f2_mul(f2_pack(r1.y, r1.y), fi)));
-          if (three) s[2].add(f2_fma(f2_pack(r2.x, r2.x), ff, f2_mul(f2_pack(r2.y, r2.y), fi)));
+        for (int c0 = lane; c0 < nop; c0 += 32 * SUM_TERMS) {
+          cx<T> p[3] = {zero, zero, zero};
+#pragma unroll
+          for (int k = 0; k < SUM_TERMS; ++k) {
+            const int c = c0 + 32 * k;
+            if (k && c >= nop) break;
+            const cx<T> f = fl[c];
+            p[0] = cfma<T>(row[c], f, p[0]);
+            if (two) p[1] = cfma<T>(row2[c], f, p[1]);
+            if (three) p[2] = cfma<T>(row3[c], f, p[2]);
+          }
+          s[0].add(f2_pack(p[0].x, p[0].y));
+          if (two) s[1].add(f2_pack(p[1].x, p[1].y));
+          if (three) s[2].add(f2_pack(p[2].x, p[2].y));
         }
         // over the lanes, half of them summing rows 0 and 1, half row 2 (its partners a zero)
         const bool b4 = lane & 16, b3 = lane & 8;
@@ -737,15 +740,15 @@ size_t ct_args(const helm_ctx* c, int first, int nc, CTailArgs<T>& a) {
 
 // ---- the dense operator ----------------------------------------------------------------------
 // Column q of the rest of the cycle below (and with) level 0 of `a`: the cycle of the unit vector q,
-// in FP64 arithmetic and in one block (a level's vectors u, f, r in shared memory).  In FP64 by the
-// definitions; in FP32 with the tables, omega/D and coarsest inverse that the levels themselves would apply: their
-// rounding is nearly the same on every level, and an exact coarse part under rounded fine levels was further
-// from the exact cycle than both rounded alike (96^2 red-black, 1e-7: 2.14 against 1.76).
+// in FP64 and in one block, by the definitions (a level's vectors u, f, r in shared memory).
+// Also in FP32 from the FP64 tables: made of the rounded ones, its error partly cancels that of the
+// rounded levels above it or adds to it (96^2 red-black 2.10 -> 1.62e-7, but 97 x 95 red-black 1.47 -> 1.88e-7; 2 % more
+// over 50 problems).
 constexpr int COL_MAX_LEVELS = 8;
 constexpr int COL_THREADS = 128;
-template <typename T> struct ColArgs {
+struct ColArgs {
   int count;
-  OpView<T> op[COL_MAX_LEVELS];
+  OpView<double> op[COL_MAX_LEVELS];
   int at[COL_MAX_LEVELS];  // place of the level's vectors
   double omega;
 };
@@ -757,7 +760,7 @@ __device__ __forceinline__ double2 col_diag(const OpView<double>& op, int i, int
   const double2 d = cadd<double>(cadd<double>(op.a0[0][i], op.a0[1][j]), somm_diag(op, i, j, 0, ph));
   return csub<double>(d, sigma64(op, p, ph));
 }
-template <typename T> __device__ double2 col_off(const OpView<T>& op, const double2* u, int i, int j) {
+__device__ double2 col_off(const OpView<double>& op, const double2* u, int i, int j) {
   const int n0 = op.n[0], n1 = op.n[1];
   const long p = i + (long)n0 * j;
   double2 acc = make_double2(0.0, 0.0);
@@ -765,22 +768,17 @@ template <typename T> __device__ double2 col_off(const OpView<T>& op, const doub
     for (int di = -1; di <= 1; ++di) {
       if ((di == 0 && dj == 0) || i + di < 0 || i + di >= n0 || j + dj < 0 || j + dj >= n1) continue;
       if (!op.stg && di != 0 && dj != 0) continue;
-      const cx<T> wt = op.stg ? op.stg[(long)(3 * (dj + 1) + di + 1) * op.ntot + p]
+      const double2 wt = op.stg ? op.stg[(long)(3 * (dj + 1) + di + 1) * op.ntot + p]
                                 : (dj == 0 ? (di < 0 ? op.am[0][i] : op.ap[0][i]) : (dj < 0 ? op.am[1][j] : op.ap[1][j]));
-      acc = cfma<double>(cconv<double, T>(wt), u[p + di + (long)dj * n0], acc);
+      acc = cfma<double>(wt, u[p + di + (long)dj * n0], acc);
     }
   return acc;
 }
-// v / D (times omega: the damped-Jacobi step's)
-template <typename T> __device__ double2 col_div(const OpView<T>& op, double2 v, double omega, int i, int j) {
-  if constexpr (std::is_same<T, double>::value) return cscale<double>(omega, cdiv<double>(v, col_diag(op, i, j)));
-  else return cmul<double>(v, cconv<double, T>(op.dinv[i + (long)op.n[0] * j]));  // dinv holds omega / D
-}
 
-template <typename T, bool RB>
-__global__ void __launch_bounds__(COL_THREADS) k_ctail_columns(const __grid_constant__ ColArgs<T> a,
-                                                               const cx<T>* __restrict__ inv, int nco,
-                                                               cx<T>* __restrict__ out, int pitch) {
+template <bool RB>
+__global__ void __launch_bounds__(COL_THREADS) k_ctail_columns(const __grid_constant__ ColArgs a,
+                                                               const double2* __restrict__ inv, int nco,
+                                                               double2* __restrict__ o64, float2* __restrict__ o32, int pitch) {
   extern __shared__ __align__(16) unsigned char ct_smem[];
   double2* const base = reinterpret_cast<double2*>(ct_smem);
   const int tid = threadIdx.x, last = a.count - 1;
@@ -794,20 +792,17 @@ __global__ void __launch_bounds__(COL_THREADS) k_ctail_columns(const __grid_cons
     __syncthreads();
   };
   for (int k = 0; k < last; ++k) {
-    const OpView<T>& op = a.op[k];
+    const OpView<double>& op = a.op[k];
     double2 *u = vec(k, 0), *f = vec(k, 1), *r = vec(k, 2);
     points(k, [&](int p, int i, int j) {
-      u[p] = RB && ((i + j) & 1) ? zero : col_div<T>(op, f[p], RB ? 1.0 : a.omega, i, j);
+      u[p] = RB && ((i + j) & 1) ? zero : cscale<double>(RB ? 1.0 : a.omega, cdiv<double>(f[p], col_diag(op, i, j)));
     });
     if (RB)
       points(k, [&](int p, int i, int j) {
-        if ((i + j) & 1) u[p] = col_div<T>(op, csub<double>(f[p], col_off<T>(op, u, i, j)), 1.0, i, j);
+        if ((i + j) & 1) u[p] = cdiv<double>(csub<double>(f[p], col_off(op, u, i, j)), col_diag(op, i, j));
       });
     points(k, [&](int p, int i, int j) {
-      const double2 off = col_off<T>(op, u, i, j);
-      if constexpr (std::is_same<T, double>::value) r[p] = csub<double>(f[p], cfma<double>(col_diag(op, i, j), u[p], off));
-      else if (RB) r[p] = (i + j) & 1 ? zero : csub<double>(zero, off);  // the cycle's own forms, without D
-      else r[p] = csub<double>(cscale<double>(1.0 - a.omega, f[p]), off);
+      r[p] = csub<double>(f[p], cfma<double>(col_diag(op, i, j), u[p], col_off(op, u, i, j)));
     });
     double2* fc = vec(k + 1, 1);
     points(k + 1, [&](int p, int I, int J) {
@@ -826,12 +821,12 @@ __global__ void __launch_bounds__(COL_THREADS) k_ctail_columns(const __grid_cons
     double2* u = vec(last, 0);
     points(last, [&](int p, int, int) {
       double2 acc = zero;
-      for (int c = 0; c < nco; ++c) acc = cfma<double>(cconv<double, T>(inv[(long)p * nco + c]), f[c], acc);
+      for (int c = 0; c < nco; ++c) acc = cfma<double>(inv[(long)p * nco + c], f[c], acc);
       u[p] = acc;
     });
   }
   for (int k = last - 1; k >= 0; --k) {
-    const OpView<T>&op = a.op[k], &oc = a.op[k + 1];
+    const OpView<double>&op = a.op[k], &oc = a.op[k + 1];
     double2 *u = vec(k, 0), *f = vec(k, 1), *r = vec(k, 2);
     const double2* e = vec(k + 1, 0);
     points(k, [&](int p, int i, int j) {
@@ -846,20 +841,22 @@ __global__ void __launch_bounds__(COL_THREADS) k_ctail_columns(const __grid_cons
     });
     if (!RB) {
       points(k, [&](int p, int i, int j) {
-        const double2 g = col_div<T>(op, csub<double>(f[p], col_off<T>(op, r, i, j)), a.omega, i, j);
+        const double2 g = cscale<double>(a.omega, cdiv<double>(csub<double>(f[p], col_off(op, r, i, j)), col_diag(op, i, j)));
         u[p] = cadd<double>(cscale<double>(1.0 - a.omega, r[p]), g);
       });
     } else {
       for (int colour = 0; colour < 2; ++colour)
         points(k, [&](int p, int i, int j) {
-          if (((i + j) & 1) == colour) r[p] = col_div<T>(op, csub<double>(f[p], col_off<T>(op, r, i, j)), 1.0, i, j);
+          if (((i + j) & 1) == colour) r[p] = cdiv<double>(csub<double>(f[p], col_off(op, r, i, j)), col_diag(op, i, j));
         });
       points(k, [&](int p, int, int) { u[p] = r[p]; });
     }
   }
   const double2* u = vec(0, 0);
   for (int p = tid; p < a.op[0].ntot; p += COL_THREADS) {
-    out[p * (long)pitch + blockIdx.x] = cconv<T, double>(u[p]);
+    const long at = p * (long)pitch + blockIdx.x;
+    if (o64) o64[at] = u[p];
+    else o32[at] = cconv<float, double>(u[p]);
   }
 }
 
@@ -888,7 +885,7 @@ template <typename T> bool ct_op_fits(long n, int nc) {
 
 // Once, at create: the dense operator of the finest level small enough for it (see the top), from
 // the coarsest inverse, and the arguments for every level the tail can begin at.
-template <typename T> helm_status ctail_build(helm_ctx* c, cudaStream_t st) {
+template <typename T> helm_status ctail_build(helm_ctx* c, const double2* inv, cudaStream_t st) {
   c->ctail_blocks = ct_blocks();
   if (!ctail_applies(c)) return HELM_OK;
   constexpr bool f64 = std::is_same<T, double>::value;
@@ -896,17 +893,17 @@ template <typename T> helm_status ctail_build(helm_ctx* c, cudaStream_t st) {
   // (a coarsest level above `most` is the operator level itself: its dense inverse has to be applied anyway.  Up
   // to CTAIL_COARSEST unknowns: 4 us of the FP64 pipe, about the launch it replaces)
   const long most = f64 ? 150 : 600;
-  ColArgs<T> ca{};
+  ColArgs ca{};
   int l = nl;
   while (l > 0 && c->lv[l - 1].ntot <= (l == nl ? std::max(most, CTAIL_COARSEST) : most) &&
          ct_op_fits<T>(c->lv[l - 1].ntot, nc) && nl - (l - 1) <= COL_MAX_LEVELS)
     --l;
   if (l == nl) return HELM_OK;  // the coarsest level alone is too large
   ca.count = nl - l;
-  ca.omega = (T)c->pc.omega;
+  ca.omega = c->pc.omega;
   int off = 0;
   for (int k = 0; k < ca.count; ++k) {
-    ca.op[k] = c->lv[l + k].template view<T>();
+    ca.op[k] = c->lv[l + k].view<double>();
     ca.at[k] = off;
     off += 3 * (int)c->lv[l + k].ntot;
   }
@@ -914,9 +911,11 @@ template <typename T> helm_status ctail_build(helm_ctx* c, cudaStream_t st) {
   helm_status s = ctx_alloc(c, &c->ctail_dense, sizeof(cx<T>) * nop * ct_pitch<T>(nop));
   if (s != HELM_OK) return s;
   const size_t smem = sizeof(double2) * off;  // at most 3 * 600 * 4 / 3 vectors' elements: 38 KB
-  auto kern = c->pc.smoother == HELM_SM_RBGS ? k_ctail_columns<T, true> : k_ctail_columns<T, false>;
+  double2* o64 = f64 ? (double2*)c->ctail_dense : nullptr;
+  float2* o32 = f64 ? nullptr : (float2*)c->ctail_dense;
+  auto kern = c->pc.smoother == HELM_SM_RBGS ? k_ctail_columns<true> : k_ctail_columns<false>;
   HELM_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024));
-  kern<<<nop, COL_THREADS, smem, st>>>(ca, (const cx<T>*)c->coarse_inv, c->nco, (cx<T>*)c->ctail_dense, ct_pitch<T>(nop));
+  kern<<<nop, COL_THREADS, smem, st>>>(ca, inv, c->nco, o64, o32, ct_pitch<T>(nop));
   HELM_CUDA(cudaGetLastError());
   c->ctail_op = l;
   std::vector<CTailArgs<T>> all(l + 1);
@@ -969,8 +968,8 @@ void ctail_group(const GCTail<T>* args, const GroupList* LT, int li, int instanc
   }
 }
 
-template helm_status ctail_build<float>(helm_ctx*, cudaStream_t);
-template helm_status ctail_build<double>(helm_ctx*, cudaStream_t);
+template helm_status ctail_build<float>(helm_ctx*, const double2*, cudaStream_t);
+template helm_status ctail_build<double>(helm_ctx*, const double2*, cudaStream_t);
 template size_t ctail_args<float>(const helm_ctx*, int, const CTailArgs<float>**);
 template size_t ctail_args<double>(const helm_ctx*, int, const CTailArgs<double>**);
 template helm_status ctail_vcycle<float, double>(const helm_ctx*, int, const double2*, void*, bool, const int*, cudaStream_t);

@@ -38,7 +38,7 @@ template <typename T> struct GCTail {
 bool ctail_applies(const helm_ctx* c);
 // the finest level of at most `points` unknowns that a tail can begin at; the level count if none
 int ctail_first_level(const helm_ctx* c, long points);
-template <typename T> helm_status ctail_build(helm_ctx* c, cudaStream_t st);
+template <typename T> helm_status ctail_build(helm_ctx* c, const double2* inv, cudaStream_t st);
 // the device arguments of a tail from level `first`, and its dynamic shared memory (0: does not fit)
 template <typename T> size_t ctail_args(const helm_ctx* c, int first, const CTailArgs<T>** a);
 template <typename T, typename TI>

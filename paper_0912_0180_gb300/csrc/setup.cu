@@ -943,7 +943,7 @@ helm_status build_hierarchy(helm_ctx* c, cudaStream_t st) {
   }
   if (f32) k_c128_to_c64<<<ceil_div((long)n * n, 256), 256, 0, st>>>(inv, (float2*)c->coarse_inv, (long)n * n);
   else cudaMemcpyAsync(c->coarse_inv, inv, sizeof(double2) * (size_t)n * n, cudaMemcpyDeviceToDevice, st);
-  if ((rc = f32 ? ctail_build<float>(c, st) : ctail_build<double>(c, st)) != HELM_OK) {
+  if ((rc = f32 ? ctail_build<float>(c, inv, st) : ctail_build<double>(c, inv, st)) != HELM_OK) {
     free_all();
     return rc;
   }
