@@ -314,9 +314,8 @@ helm_status helm_solve_batch(helm_ctx* const* ctxs, const void* const* b, void* 
  * V-cycle kernels (L = the largest number of fused levels) and one condition kernel, whatever n.
  * Requirements (else HELM_ERR_ARG, checked on the host): n >= 1 distinct contexts on the current
  * device, 2D grids, a CSL or CSG preconditioner with V(1,1) cycles on rediscretised fused levels
- * (no HELM_PF_UNFUSED or HELM_PF_GALERKIN) and a dense coarsest inverse, one smoother kind (not
- * HELM_SM_ILU) and one
- * mg_dtype for all.  Grids, k fields, preconditioner parameters and sizes may all differ.
+ * (no HELM_PF_UNFUSED or HELM_PF_GALERKIN) and a dense coarsest inverse, the thread-block cluster of
+ * the one-launch tail where they have one, one smoother kind (not HELM_SM_ILU) and one mg_dtype for all.  Grids, k fields, preconditioner parameters and sizes may all differ.
  * Each instance keeps its own block decomposition and reduction order, so its iterates, statistics
  * and solution are bitwise those helm_solve gives it alone; infos[i].kernels is the group's total
  * launch count.  Synchronises `stream` at the end. */

@@ -242,7 +242,7 @@ struct helm_ctx {
   void* scratch = nullptr;           // FP32 hierarchies: 2N complex64, the unfused V-cycle's level-0
                                      // output before widening, then helm_vcycle's converted input
   cudaStream_t alloc_stream = nullptr;  // stream of the stream-ordered allocations of helm_create
-  int tail_first = 1 << 30;          // first level run by the single-block tail kernel
+  int tail_first = 1 << 30;          // first level run by the one-launch tail (one cluster, or one block)
   FdmCoarse fdm;                     // separable coarsest solve (constant phi there), or off
   // one-cluster tail (mg_cluster.cu): operator level and its matrix; the arguments for each level it
   // can begin at, and the dynamic shared memory each needs (0: it cannot)

@@ -27,8 +27,12 @@
 // read them ([strip][step][entry][lane]) and fetched 16 to 24 steps ahead (cp.async), since nothing
 // else runs on the SM to hide a load.  One block walking the wavefronts with a barrier each cost 1.1
 // us a wavefront in FP32; a V(0,1) cycle of MP3's operators on 640^2 unknowns went from 8.40 to 0.99
-// ms, 0.96 with the factors of eight steps read into registers at once (about 0.1 us a step, 54 instructions of
+// ms, 0.95 with the factors of eight steps read into registers at once (about 0.1 us a step, 54 instructions of
 // which half wait on the one before).
+//
+// The waits for a hand-over are bounded (about a second).  One that runs out makes the rest NaN and sets a
+// pinned host word; a cluster barrier at the end keeps every block until all have sent (no measurable cost: 951 us
+// against 956 without it).  The cluster is as large as the device grants, 16 blocks on GB300.
 #include <algorithm>
 #include <type_traits>
 #include <vector>

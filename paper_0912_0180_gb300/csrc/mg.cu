@@ -40,6 +40,9 @@ template <int DIM> static void rb_cfg(const int n[3], dim3& g, dim3& b) {
 // plane by other threads of the last column of blocks: lanes along y, packed.  FP64 only: its pipe (2 lanes
 // a clock) bills a warp's 32 lanes whatever they do -- a row of 129 points cost five chunks (129 x 145 x
 // 113 points: sweep 160 -> 129 us, residual 113 -> 90 us).  A point's formula depends on its indices alone.
+// Packed against not, (128 + m) x 96 x 80 points, matvec and V-cycle in us: m = 1 33 / 41 and 222 / 247, 8 35 / 41 and
+// 241 / 262, 16 37 / 41 and 258 / 272, 24 39 / 41 and 266 / 272, 31 41 / 41 and 274 / 273; likewise at 64 + m.  The
+// line at half a chunk is on the safe side: packing gains to about 28.
 constexpr int TAIL_COLS = 16;
 template <typename T, int DIM>
 __device__ __forceinline__ bool point_of(const int (&n)[3], int& i, int& j, int& l) {

@@ -13,11 +13,12 @@
 // operators in FP64 arithmetic, one block per column), split by rows over the blocks.  That replaces a
 // chain of some twenty dependent phases of a few hundred points by one.  The level is the finest one with
 // at most 600 unknowns in FP32 (166 KB of a block's shared memory; reading it there takes 1300 cycles,
-// a level's descent and ascent 5000) and 150 in FP64 (n^2 / 8 cycles of a block's
-// FP64 pipe).
+// a level's descent and ascent 5000) and 150 in FP64 (n^2 / 8 cycles of a block's FP64 pipe), or a larger
+// coarsest level itself.
 //
-// Measured (whole V-cycles, us): 96^2 FP32 red-black 24.5 -> 14.0, 640^2 FP32 Jacobi 42 -> 31, FP64 118 ->
-// 108, MP2's Galerkin levels in FP64 109 -> 96.
+// Measured (whole V-cycles, us, a launch per level / with this kernel, paired when it was made): 96^2 FP32
+// red-black 33.5 / 17.1, 640^2 FP32 Jacobi 50.0 / 33.8, FP64 125 / 116, MP2's Galerkin levels in FP64 119 / 101.
+// Now, from graphs of cycles: 12.3 and 31.9 in FP32; paired runs: 116 and 94 in FP64.
 //
 // What bounds the kernel is the chain of phases: two cluster barriers and five block barriers a level,
 // and between them one or two points a thread, whose instructions count.

@@ -68,7 +68,7 @@ __device__ __forceinline__ bool colour_item(int k, int W, int gi0, int gj0, int 
 // Whether the smoothed iterate of the zero guess goes through memory between the two halves of a level.
 // In FP32 damped Jacobi the up kernel forms it again, u = (omega / D) f, from the f and omega / D that it
 // reads anyway: 16 bytes a point less, one product more (2304^2 cycle with the narrowing below 158 ->
-// 141 us, 640^2 33.8 -> 29.4 us).
+// 141 us, 640^2 about 2 us of 34).
 // In FP64 the product is dearer than the bytes (2 FP64 lanes a clock), and red-black sweeps would need
 // their neighbours.
 template <typename T, bool RBGS> constexpr bool keeps_u() { return RBGS || sizeof(T) == 8; }
@@ -1342,7 +1342,7 @@ static helm_status autotune_t(helm_ctx* c, cudaStream_t st) {
   if (fused2d) {
     std::lock_guard<std::mutex> lk(g_tune_mu);
     for (int l = 0; l < nl - 1; ++l) {
-      if (c->lv[l].stg64) continue;  // Galerkin levels do not run the fused kernels
+      if (c->lv[l].stg64) continue;  // 9-point levels take the tiles of the block-count rule, untimed
       auto it = g_tune.find(std::make_tuple((int)sizeof(T), (int)RB, c->lv[l].n[0], c->lv[l].n[1]));
       auto valid = [](int t) { return t >= 0 && t < (RB ? TILE_LONG : NUM_TILES); };
       if (it != g_tune.end() && valid(it->second.first) && valid(it->second.second)) {
